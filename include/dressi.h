@@ -141,11 +141,12 @@ typedef struct {
                             the same scene (positions unchanged), views and params -- vertex
                             transform, face table, normals and, for layer_ids == NULL, the
                             tile lists -- and the backward takes it instead of rebuilding it
-                            (with layer_ids == NULL it still re-rasterizes: layers and
-                            barycentrics are recomputed, each pixel's K-list starting from the
+                            (with layer_ids == NULL layers are recomputed where several are
+                            blended, inside the edge mask, each pixel's K-list starting from the
                             K-th (key, face) that a forward without layer ids kept in the
                             workspace, which culls the candidates that cannot reach the K
-                            layers).  0 = rebuild.  The caller guarantees the precondition; a
+                            layers; outside the mask the front layer it kept serves, and
+                            barycentrics are recomputed everywhere).  0 = rebuild.  The caller guarantees the precondition; a
                             workspace written by another call since gives wrong gradients. */
 } dressi_params;
 

@@ -322,13 +322,24 @@ static void run_setup(Globals &g, const Plan &P, char *ws, bool need_bins, cudaS
     if (need_bins) launch_bin(g, (int)P.views.size(), P.max_nf_view, s);
 }
 
-// a forward that stores no layer ids keeps every pixel's K-th (key, id) in the workspace
-// for a re-rasterizing adjoint; the flag says whether the last forward did
-static void keep_kth(Globals &g, const Plan &P, char *ws, cudaStream_t s)
+// Whether a pass without stored layer ids needs the layers behind the front one only inside the
+// edge mask (outside it a pixel shows its front hard layer alone).  Not where the mask is
+// everywhere; not for the inverse UV, which samples a soft front layer outside the mask too; and
+// keys have to stay below 2 for the words that the forward leaves (r < 2 screens).
+static bool fronts_only(const dressi_params *p)
+{
+    const bool inv_uv = p->texgrad_mode == 2 && p->shade_mode != 0;
+    return p->edge_mode != 1 && !inv_uv && p->r < 2.f;
+}
+
+// a forward that stores no layer ids leaves every pixel's word (K-th entry, or front layer with
+// E and S^H) in the workspace for a re-rasterizing adjoint; the flag says which, if any
+static void keep_kth(Globals &g, const Plan &P, const dressi_params *p, char *ws, cudaStream_t s)
 {
     const bool keep = g.ids == nullptr;
+    g.fronts = keep && fronts_only(p);
     g.kth = keep ? reinterpret_cast<unsigned long long *>(ws + P.lay.kth) : nullptr;
-    cudaMemsetAsync(ws + P.lay.kth_flag, keep ? 1 : 0, sizeof(int), s);
+    cudaMemsetAsync(ws + P.lay.kth_flag, keep ? (g.fronts ? 2 : 1) : 0, sizeof(int), s);
 }
 
 // the per-tile kernel, persistent (longest face list first when the lists exist) or
@@ -466,7 +477,7 @@ int dressi_forward(const dressi_scene *scene, const dressi_view *views, int32_t 
     Globals g = make_globals(scene, params, P, w, n_pix, dev_status);
     g.out = out_rgba;
     g.ids = layer_ids;
-    keep_kth(g, P, w, s);
+    keep_kth(g, P, params, w, s);
     run_setup(g, P, w, true, s);
     run_tiles(g, P, w, true, 0, s);
     return cudaGetLastError() == cudaSuccess ? DRESSI_OK : DRESSI_ERR_LAUNCH;
@@ -493,7 +504,7 @@ int dressi_forward_l2(const dressi_scene *scene, const dressi_view *views, int32
     g.l2_target = target;
     g.l2_grad = grad_rgba;
     g.l2_loss = loss_accum;
-    keep_kth(g, P, w, s);
+    keep_kth(g, P, params, w, s);
     run_setup(g, P, w, true, s);
     run_tiles(g, P, w, true, 0, s);
     return cudaGetLastError() == cudaSuccess ? DRESSI_OK : DRESSI_ERR_LAUNCH;
@@ -580,7 +591,8 @@ int dressi_backward_ex(const dressi_scene *scene, const dressi_view *views, int3
     if (!tex_records) g.texgrad_mode = 0;
     if (gather) cudaMemsetAsync(w + P.lay.tg_keys, 0xff, sizeof(unsigned) * (size_t)P.lay.tg_slots, s);
     if (inv_uv) cudaMemsetAsync(w + P.lay.inv_uv, 0xff, sizeof(int) * (size_t)P.n_texels, s);
-    // re-rasterizing after a forward on this workspace: its K-th keys, if it kept them
+    g.fronts = !layer_ids && fronts_only(params);
+    // re-rasterizing after a forward on this workspace: its pixels' words, if it kept them
     if (params->reuse_setup && !layer_ids) g.kth = reinterpret_cast<unsigned long long *>(w + P.lay.kth);
     if (!params->reuse_setup) run_setup(g, P, w, layer_ids == nullptr, s);
     run_tiles(g, P, w, layer_ids == nullptr, 1, s);

@@ -74,13 +74,18 @@ struct __align__(16) VRec {
 // swapped bits of the flags are always 0, 0, 1 for a live face): the evaluations pick no
 // endpoints at run time.  FLAG_ODD records whether that order is an odd permutation of the
 // face's own corner order (the normal map's tangent-frame handedness needs the latter).
-// the geometric part (the first 20 words): all that SignedDist, the hard test and Shift
+// The geometric part (the first 20 words): all that SignedDist, the hard test and Shift
 // read, and what the raster stages in shared memory
+struct __align__(16) Corner {
+    float xh, xl, yh, yl;   // pixel position as float pairs
+};
+
 struct __align__(16) FaceGeo {
-    float xh[3], xl[3], yh[3], yl[3];
-    float invL[3];   // 1 / length of edge i (canonical), correctly rounded
+    Corner c[3];     // one 16-byte load each, so that a soft pair's exact path reads two of them
+    float invL[3];   // 1 / length of edge i, correctly rounded, negative where the canonical
+                     // edge's cross product is negative inside the face
     float z[3];
-    float invA;      // 1 / |twice the signed area|
+    float invA;      // 1 / (twice the signed area)
     int flags;       // bit 0: orient > 0; bits 1-3: edge i swapped; bits 4-6: edge i owns;
                      // FLAG_LIVE: not culled; FLAG_RANGE: a vertex index is out of range;
                      // FLAG_ODD: corners permuted oddly
@@ -131,14 +136,16 @@ struct Globals {
     int *queue;           // tile queue head (zeroed before each pass)
     const int *tile_order;  // tiles by descending face-list length, or nullptr
     int *lpt_hist;        // [LPT_BINS] scratch of the ordering sort
-    // the forward without stored layer ids keeps each pixel's K-th (key, id) here (per view
-    // pixel, at slot_base + pixel; *kth_flag nonzero once it did); the re-rasterizing adjoint
-    // that takes the forward's setup starts every K-list with it, so that pairs whose key
-    // bound lies above it are culled from the start
+    // the forward without stored layer ids leaves a word per view pixel here (at slot_base +
+    // pixel; *kth_flag says which kind): the K-th (key, id), or, where only fronts are wanted,
+    // E and S^H with the K-th (key, id) of an edge-masked pixel and the front one of another.
+    // The re-rasterizing adjoint that takes the forward's setup starts its K-lists with the
+    // K-th entries, so that pairs whose key bound lies above are culled from the start, and
+    // rasterizes nothing where the mask is empty
     unsigned long long *kth;
     int *kth_flag;
+    int fronts;           // layers beyond the front one are only needed inside the edge mask
     int zero_bins;        // the vertex transform clears tile_count and tile_cursor
-    int pad2;
     // forward
     float *out;
     int *ids;             // [K][n_pix] or nullptr
@@ -206,19 +213,19 @@ __device__ __forceinline__ bool face_load(const Globals &g, const MeshK &m, cons
     for (int i = 0; i < 3; ++i) {
         const float4 *rec = reinterpret_cast<const float4 *>(vr + R.vi[i]);
         const float4 p = rec[0], q = rec[1];
-        R.xh[i] = p.x; R.xl[i] = p.y; R.yh[i] = p.z; R.yl[i] = p.w;
+        R.c[i].xh = p.x; R.c[i].xl = p.y; R.c[i].yh = p.z; R.c[i].yl = p.w;
         R.z[i] = q.x; R.iw[i] = q.y;
         live = live && (__float_as_int(q.z) != 0);
     }
     // corners in lexicographic order (a three-element sorting network), counting the swaps
     bool odd = false;
     auto order = [&](int a, int b) {
-        if (lex_less(R.xh[b], R.xl[b], R.yh[b], R.yl[b], R.xh[a], R.xl[a], R.yh[a], R.yl[a])) {
+        if (lex_less(R.c[b].xh, R.c[b].xl, R.c[b].yh, R.c[b].yl, R.c[a].xh, R.c[a].xl, R.c[a].yh, R.c[a].yl)) {
             float t;
-            t = R.xh[a]; R.xh[a] = R.xh[b]; R.xh[b] = t;
-            t = R.xl[a]; R.xl[a] = R.xl[b]; R.xl[b] = t;
-            t = R.yh[a]; R.yh[a] = R.yh[b]; R.yh[b] = t;
-            t = R.yl[a]; R.yl[a] = R.yl[b]; R.yl[b] = t;
+            t = R.c[a].xh; R.c[a].xh = R.c[b].xh; R.c[b].xh = t;
+            t = R.c[a].xl; R.c[a].xl = R.c[b].xl; R.c[b].xl = t;
+            t = R.c[a].yh; R.c[a].yh = R.c[b].yh; R.c[b].yh = t;
+            t = R.c[a].yl; R.c[a].yl = R.c[b].yl; R.c[b].yl = t;
             t = R.z[a]; R.z[a] = R.z[b]; R.z[b] = t;
             t = R.iw[a]; R.iw[a] = R.iw[b]; R.iw[b] = t;
             const int v = R.vi[a]; R.vi[a] = R.vi[b]; R.vi[b] = v;
@@ -229,10 +236,10 @@ __device__ __forceinline__ bool face_load(const Globals &g, const MeshK &m, cons
     order(1, 2);
     order(0, 1);
     // twice the signed area from accurate corner differences
-    const float ux = fadd(fsub(R.xh[1], R.xh[0]), fsub(R.xl[1], R.xl[0]));
-    const float uy = fadd(fsub(R.yh[1], R.yh[0]), fsub(R.yl[1], R.yl[0]));
-    const float wx = fadd(fsub(R.xh[2], R.xh[0]), fsub(R.xl[2], R.xl[0]));
-    const float wy = fadd(fsub(R.yh[2], R.yh[0]), fsub(R.yl[2], R.yl[0]));
+    const float ux = fadd(fsub(R.c[1].xh, R.c[0].xh), fsub(R.c[1].xl, R.c[0].xl));
+    const float uy = fadd(fsub(R.c[1].yh, R.c[0].yh), fsub(R.c[1].yl, R.c[0].yl));
+    const float wx = fadd(fsub(R.c[2].xh, R.c[0].xh), fsub(R.c[2].xl, R.c[0].xl));
+    const float wy = fadd(fsub(R.c[2].yh, R.c[0].yh), fsub(R.c[2].yl, R.c[0].yl));
     const float A2 = ffma(ux, wy, -fmul(uy, wx));
     if (!(A2 != 0.f) || !isfinite(A2)) live = false;
     const bool orient = A2 > 0.f;
@@ -240,23 +247,24 @@ __device__ __forceinline__ bool face_load(const Globals &g, const MeshK &m, cons
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         const int ia = i, ib = (i + 1) % 3;
-        const bool sw = lex_less(R.xh[ib], R.xl[ib], R.yh[ib], R.yl[ib], R.xh[ia], R.xl[ia], R.yh[ia], R.yl[ia]);
+        const bool sw = lex_less(R.c[ib].xh, R.c[ib].xl, R.c[ib].yh, R.c[ib].yl, R.c[ia].xh, R.c[ia].xl, R.c[ia].yh, R.c[ia].yl);
         // canonical edge P -> Q
-        const float Pxh = sw ? R.xh[ib] : R.xh[ia], Pxl = sw ? R.xl[ib] : R.xl[ia];
-        const float Pyh = sw ? R.yh[ib] : R.yh[ia], Pyl = sw ? R.yl[ib] : R.yl[ia];
-        const float Qxh = sw ? R.xh[ia] : R.xh[ib], Qxl = sw ? R.xl[ia] : R.xl[ib];
-        const float Qyh = sw ? R.yh[ia] : R.yh[ib], Qyl = sw ? R.yl[ia] : R.yl[ib];
+        const float Pxh = sw ? R.c[ib].xh : R.c[ia].xh, Pxl = sw ? R.c[ib].xl : R.c[ia].xl;
+        const float Pyh = sw ? R.c[ib].yh : R.c[ia].yh, Pyl = sw ? R.c[ib].yl : R.c[ia].yl;
+        const float Qxh = sw ? R.c[ia].xh : R.c[ib].xh, Qxl = sw ? R.c[ia].xl : R.c[ib].xl;
+        const float Qyh = sw ? R.c[ia].yh : R.c[ib].yh, Qyl = sw ? R.c[ia].yl : R.c[ib].yl;
         const float ex = fadd(fsub(Qxh, Pxh), fsub(Qxl, Pxl));
         const float ey = fadd(fsub(Qyh, Pyh), fsub(Qyl, Pyl));
         const float L = __fsqrt_rn(ffma(ex, ex, fmul(ey, ey)));
-        R.invL[i] = __fdiv_rn(1.f, L);
+        const float iL = __fdiv_rn(1.f, L);
+        R.invL[i] = orient != sw ? iL : -iL;
         // oriented edge ia -> ib
         const float eox = sw ? -ex : ex, eoy = sw ? -ey : ey;
         const bool owns = orient ? (eoy < 0.f || (eoy == 0.f && eox > 0.f)) : (eoy > 0.f || (eoy == 0.f && eox < 0.f));
         flags |= (sw ? 1 : 0) << (1 + i);
         flags |= (owns ? 1 : 0) << (4 + i);
     }
-    R.invA = __fdiv_rn(1.f, fabsf(A2));
+    R.invA = __fdiv_rn(1.f, A2);
     if (live) flags |= FLAG_LIVE;
     if (odd) flags |= FLAG_ODD;
     R.flags = flags;
@@ -281,7 +289,7 @@ __device__ __forceinline__ bool face_get(const Globals &g, const ViewK &V, const
     }
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        R.xh[i] = w[i]; R.xl[i] = w[3 + i]; R.yh[i] = w[6 + i]; R.yl[i] = w[9 + i];
+        R.c[i].xh = w[4 * i]; R.c[i].xl = w[4 * i + 1]; R.c[i].yh = w[4 * i + 2]; R.c[i].yl = w[4 * i + 3];
         R.invL[i] = w[12 + i]; R.z[i] = w[15 + i];
         R.vi[i] = __float_as_int(w[21 + i]); R.iw[i] = w[24 + i];
     }
@@ -332,7 +340,8 @@ __device__ __forceinline__ void face_complete(const Globals &g, const ViewK &V, 
 struct Frag {
     float dist;      // signed pixel distance (positive inside the hard face)
     float key;       // Shift() key
-    float Fn[3];     // oriented edge numerators: lam_{(i+2)%3} = Fn[i] * invA
+    float c[3];      // cross products of the canonical edges: with edge 2 (0 -> 2, against the
+                     // others' sense) negated, lam_{(i+2)%3} = c[i] * invA
     float t;         // soft fragment on edge `feat`: closest point = P + t (Q - P), canonical P, Q
     int hard;
     int feat;        // 0..2: edge i interior; 3..5: corner (feat - 3)
@@ -341,47 +350,46 @@ struct Frag {
 // SignedDist, candidate rule, hard test (top-left fill rule) and Shift (Eq. Shift) of
 // face R at pixel centre (px, py).  Returns false when the face is not a candidate
 // (farther than r_px outside).  Pure function of (R, px, py, r_px, half_inv_S).
-// Every array index below is a compile-time constant (canonical endpoints are
-// chosen by selects), so nothing spills to local memory.  An edge distance is the
-// canonical cross product times the record's 1/L and a corner distance the square
+// Every array index below is a compile-time constant (endpoints are chosen by selects:
+// with the corners in lexicographic order the canonical edges are 0 -> 1, 1 -> 2 and 0 -> 2),
+// so nothing spills to local memory.  An edge distance is the canonical cross product times
+// the record's 1/L, whose sign makes it positive inside, and a corner distance the square
 // root at the shared corner, so the faces around a shared edge or corner compute
 // bit-identical distances to it.
 // With LAMBDA false the closest point's parameter o.t is left at 0: the peel needs the
 // key alone, shading and the adjoint re-evaluate the kept layers with LAMBDA.
+// hard_only accepts hard fragments alone.
 template <bool LAMBDA = true>
 __device__ __forceinline__ bool eval_face(const FaceGeo &R, float px, float py, float r_px, float half_inv_S,
-                                          Frag &o)
+                                          Frag &o, bool hard_only = false)
 {
     float dx[3], dy[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        dx[i] = fsub(fsub(px, R.xh[i]), R.xl[i]);
-        dy[i] = fsub(fsub(py, R.yh[i]), R.yl[i]);
+        dx[i] = fsub(fsub(px, R.c[i].xh), R.c[i].xl);
+        dy[i] = fsub(fsub(py, R.c[i].yh), R.c[i].yl);
     }
-    const bool orient = R.flags & 1;
-    // canonical endpoint offsets p - P and p - Q of every edge
-    float pX[3], pY[3], qX[3], qY[3], c[3], F[3];
-    bool early_out = false;
+    // cross(Q - P, p - P) == cross(p - P, p - Q) of each canonical edge
+    float F[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        const bool sw = i == 2;   // corners in lexicographic order
-        const int ia = i, ib = (i + 1) % 3;
-        pX[i] = sw ? dx[ib] : dx[ia]; pY[i] = sw ? dy[ib] : dy[ia];
-        qX[i] = sw ? dx[ia] : dx[ib]; qY[i] = sw ? dy[ia] : dy[ib];
-        // cross(Q - P, p - P) == cross(p - P, p - Q)
-        c[i] = ffma(pX[i], qY[i], -fmul(pY[i], qX[i]));
-        const float fn = (orient != sw) ? c[i] : -c[i];
-        o.Fn[i] = fn;
-        F[i] = fmul(fn, R.invL[i]);
-        early_out |= F[i] < -r_px;
+        const int P = i == 2 ? 0 : i, Q = i == 2 ? 2 : i + 1;
+        o.c[i] = ffma(dx[P], dy[Q], -fmul(dy[P], dx[Q]));
+        F[i] = fmul(o.c[i], R.invL[i]);
     }
-    if (early_out) return false;
-    bool inside = true;
+    const float Fmin = fminf(F[0], fminf(F[1], F[2]));
+    if (Fmin < -r_px) return false;
+    bool inside = F[0] > 0.f && F[1] > 0.f && F[2] > 0.f;
+    if (!inside && !(Fmin < 0.f)) {
+        // on an edge's line (or an edge of no length): the fill rule decides
+        inside = true;
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        const bool owns = (R.flags >> (4 + i)) & 1;
-        inside &= (o.Fn[i] > 0.f) || (o.Fn[i] == 0.f && owns);
+        for (int i = 0; i < 3; ++i) {
+            const bool owns = (R.flags >> (4 + i)) & 1;
+            inside &= (R.invL[i] > 0.f ? o.c[i] > 0.f : o.c[i] < 0.f) || (o.c[i] == 0.f && owns);
+        }
     }
+    if (hard_only && !inside) return false;
     float dist, bt = 0.f;
     int feat;
     // the edge whose line the pixel is farthest outside of (smallest F), and the gap to
@@ -398,47 +406,41 @@ __device__ __forceinline__ bool eval_face(const FaceGeo &R, float px, float py, 
         // (its interior, or one of its endpoints).  That edge alone is measured unless
         // the two smallest F are within EDGE_TIE_PX of each other (slivers, where rounding
         // could swap them): then every edge is, and the closest taken.
-        const float fmid = emin == 0 ? fminf(F[1], F[2]) : (emin == 1 ? fminf(F[0], F[2]) : fminf(F[0], F[1]));
-        const bool single = fsub(fmid, fmin1) > EDGE_TIE_PX;
+        const float fmid = fmaxf(fminf(F[0], F[1]), fminf(fmaxf(F[0], F[1]), F[2]));
         // squared distances compared without branches; one square root for a corner
         float best2 = 3.4e38f, bsel = -1.f, btn = 0.f, btd = 1.f;
         feat = 0;
-        if (single) {
-            const int i = emin;
-            const float Pxi = i == 0 ? pX[0] : (i == 1 ? pX[1] : pX[2]);
-            const float Pyi = i == 0 ? pY[0] : (i == 1 ? pY[1] : pY[2]);
-            const float Qxi = i == 0 ? qX[0] : (i == 1 ? qX[1] : qX[2]);
-            const float Qyi = i == 0 ? qY[0] : (i == 1 ? qY[1] : qY[2]);
-            const float ci = i == 0 ? c[0] : (i == 1 ? c[1] : c[2]);
-            const float iLi = i == 0 ? R.invL[0] : (i == 1 ? R.invL[1] : R.invL[2]);
-            const bool sw = i == 2;   // corners in lexicographic order
-            const int ia = i, ib = i == 2 ? 0 : i + 1;
-            const float ex = fsub(Pxi, Qxi), ey = fsub(Pyi, Qyi);   // V_Q - V_P
-            const float tP = ffma(Pxi, ex, fmul(Pyi, ey));
-            const float tQ = ffma(Qxi, ex, fmul(Qyi, ey));
+        if (fsub(fmid, fmin1) > EDGE_TIE_PX) {
+            const float Px = emin == 1 ? dx[1] : dx[0], Py = emin == 1 ? dy[1] : dy[0];
+            const float Qx = emin == 0 ? dx[1] : dx[2], Qy = emin == 0 ? dy[1] : dy[2];
+            const float ex = fsub(Px, Qx), ey = fsub(Py, Qy);   // V_Q - V_P
+            const float tP = ffma(Px, ex, fmul(Py, ey));
+            const float tQ = ffma(Qx, ex, fmul(Qy, ey));
             const bool atP = tP <= 0.f, atQ = !atP && tQ >= 0.f;
-            const float cx = atQ ? Qxi : Pxi, cy = atQ ? Qyi : Pyi;
+            const float cx = atQ ? Qx : Px, cy = atQ ? Qy : Py;
             best2 = ffma(cx, cx, fmul(cy, cy));
-            feat = atP ? 3 + (sw ? ib : ia) : atQ ? 3 + (sw ? ia : ib) : i;
-            bsel = (atP || atQ) ? -1.f : fmul(fabsf(ci), iLi);
-            btn = tP;
-            btd = ffma(ex, ex, fmul(ey, ey));
+            bsel = (atP || atQ) ? -1.f : -fmin1;   // |cross| / L
+            if (LAMBDA) {
+                feat = atP ? 3 + (emin == 1) : atQ ? (emin == 0 ? 4 : 5) : emin;
+                btn = tP;
+                btd = ffma(ex, ex, fmul(ey, ey));
+            }
         } else {
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
-                const bool sw = i == 2;   // corners in lexicographic order
-                const int ia = i, ib = (i + 1) % 3;
-                const float ex = fsub(pX[i], qX[i]), ey = fsub(pY[i], qY[i]);   // V_Q - V_P
-                const float tP = ffma(pX[i], ex, fmul(pY[i], ey));
-                const float tQ = ffma(qX[i], ex, fmul(qY[i], ey));
-                const float dP2 = ffma(pX[i], pX[i], fmul(pY[i], pY[i]));
-                const float dQ2 = ffma(qX[i], qX[i], fmul(qY[i], qY[i]));
-                const float se = fmul(fabsf(c[i]), R.invL[i]);
+                const int P = i == 2 ? 0 : i, Q = i == 2 ? 2 : i + 1;
+                const float ex = fsub(dx[P], dx[Q]), ey = fsub(dy[P], dy[Q]);   // V_Q - V_P
+                const float tP = ffma(dx[P], ex, fmul(dy[P], ey));
+                const float tQ = ffma(dx[Q], ex, fmul(dy[Q], ey));
+                const float dP2 = ffma(dx[P], dx[P], fmul(dy[P], dy[P]));
+                const float dQ2 = ffma(dx[Q], dx[Q], fmul(dy[Q], dy[Q]));
+                const float se = fabsf(F[i]);
                 const bool atP = tP <= 0.f, atQ = !atP && tQ >= 0.f;
                 const float s2 = atP ? dP2 : atQ ? dQ2 : fmul(se, se);
-                const int ft = atP ? 3 + (sw ? ib : ia) : atQ ? 3 + (sw ? ia : ib) : i;
                 if (s2 < best2) {
-                    best2 = s2; feat = ft; bsel = (atP || atQ) ? -1.f : se;
+                    best2 = s2;
+                    feat = atP ? 3 + P : atQ ? 3 + Q : i;
+                    bsel = (atP || atQ) ? -1.f : se;
                     btn = tP; btd = ffma(ex, ex, fmul(ey, ey));
                 }
             }
@@ -453,8 +455,8 @@ __device__ __forceinline__ bool eval_face(const FaceGeo &R, float px, float py, 
     o.feat = feat;
     o.t = bt;
     if (inside) {
-        // z(p) = sum lam_j z_j,  lam_{(i+2)%3} = Fn[i] / |A2|
-        float zs = ffma(o.Fn[1], R.z[0], ffma(o.Fn[2], R.z[1], fmul(o.Fn[0], R.z[2])));
+        // z(p) = sum lam_j z_j
+        float zs = ffma(o.c[1], R.z[0], ffma(-o.c[2], R.z[1], fmul(o.c[0], R.z[2])));
         o.key = fmul(0.5f, fmul(zs, R.invA));
     } else {
         o.key = ffma(-dist, half_inv_S, 0.5f);
@@ -468,9 +470,9 @@ __device__ __forceinline__ bool eval_face(const FaceGeo &R, float px, float py, 
 __device__ __forceinline__ void frag_lambda(const FaceGeo &R, const Frag &fr, float lam[3])
 {
     if (fr.hard) {
-        lam[0] = fmul(fr.Fn[1], R.invA);
-        lam[1] = fmul(fr.Fn[2], R.invA);
-        lam[2] = fmul(fr.Fn[0], R.invA);
+        lam[0] = fmul(fr.c[1], R.invA);
+        lam[1] = fmul(-fr.c[2], R.invA);
+        lam[2] = fmul(fr.c[0], R.invA);
         return;
     }
     if (fr.feat >= 3) {
@@ -492,8 +494,8 @@ __device__ __forceinline__ bool hard_test(const FaceGeo &R, float px, float py)
     float dx[3], dy[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        dx[i] = fsub(fsub(px, R.xh[i]), R.xl[i]);
-        dy[i] = fsub(fsub(py, R.yh[i]), R.yl[i]);
+        dx[i] = fsub(fsub(px, R.c[i].xh), R.c[i].xl);
+        dy[i] = fsub(fsub(py, R.c[i].yh), R.c[i].yl);
     }
     const bool orient = R.flags & 1;
     bool inside = true;

@@ -189,16 +189,16 @@ __global__ void k_normal_csr(Globals g)
 // touches.  The face table kernel counts, k_bin fills.  Order inside a list is
 // irrelevant: the peel keeps the K smallest (key, id) pairs.
 // ---------------------------------------------------------------------------
-// the tiles [tx0, tx1] x [ty0, ty1] that the grown box of screen corners (xh, yh)
+// the tiles [tx0, tx1] x [ty0, ty1] that the grown box of the face's screen corners
 // touches; false when it misses the view
-__device__ __forceinline__ bool bin_rect(const Globals &g, const ViewK &V, const float (&xh)[3], const float (&yh)[3],
-                                         int &tx0, int &tx1, int &ty0, int &ty1)
+__device__ __forceinline__ bool bin_rect(const Globals &g, const ViewK &V, const FaceGeo &R, int &tx0, int &tx1,
+                                         int &ty0, int &ty1)
 {
     const float Tinv = 1.f / (float)g.tile;
-    const float x0 = fminf(xh[0], fminf(xh[1], xh[2])) - V.bin_R;
-    const float x1 = fmaxf(xh[0], fmaxf(xh[1], xh[2])) + V.bin_R;
-    const float y0 = fminf(yh[0], fminf(yh[1], yh[2])) - V.bin_R;
-    const float y1 = fmaxf(yh[0], fmaxf(yh[1], yh[2])) + V.bin_R;
+    const float x0 = fminf(R.c[0].xh, fminf(R.c[1].xh, R.c[2].xh)) - V.bin_R;
+    const float x1 = fmaxf(R.c[0].xh, fmaxf(R.c[1].xh, R.c[2].xh)) + V.bin_R;
+    const float y0 = fminf(R.c[0].yh, fminf(R.c[1].yh, R.c[2].yh)) - V.bin_R;
+    const float y1 = fmaxf(R.c[0].yh, fmaxf(R.c[1].yh, R.c[2].yh)) + V.bin_R;
     if (x1 < 0.f || y1 < 0.f || x0 > (float)V.W || y0 > (float)V.H) return false;
     tx0 = max(0, (int)floorf(x0 * Tinv));
     tx1 = min(V.tiles_x - 1, (int)floorf(x1 * Tinv));
@@ -283,13 +283,12 @@ __global__ void __launch_bounds__(256) k_face(Globals g)
                 // out of range: nothing else of the record is meaningful
                 bad = true;
 #pragma unroll
-                for (int i = 0; i < 3; ++i) { R.vi[i] = 0; R.xh[i] = R.xl[i] = R.yh[i] = R.yl[i] = 0.f; }
+                for (int i = 0; i < 3; ++i) { R.vi[i] = 0; R.c[i].xh = R.c[i].xl = R.c[i].yh = R.c[i].yl = 0.f; }
             }
             live = (R.flags & FLAG_LIVE) != 0;
             float4 *d = ws + lane * 7;   // 112-byte lane stride: no bank conflict within 8 lanes
-            d[0] = make_float4(R.xh[0], R.xh[1], R.xh[2], R.xl[0]);
-            d[1] = make_float4(R.xl[1], R.xl[2], R.yh[0], R.yh[1]);
-            d[2] = make_float4(R.yh[2], R.yl[0], R.yl[1], R.yl[2]);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) d[i] = make_float4(R.c[i].xh, R.c[i].xl, R.c[i].yh, R.c[i].yl);
             d[3] = make_float4(R.invL[0], R.invL[1], R.invL[2], R.z[0]);
             d[4] = make_float4(R.z[1], R.z[2], R.invA, __int_as_float(R.flags));
             d[5] = make_float4(__int_as_float(R.id), __int_as_float(R.vi[0]), __int_as_float(R.vi[1]),
@@ -306,7 +305,7 @@ __global__ void __launch_bounds__(256) k_face(Globals g)
         __syncwarp();   // the staged records are read before the next iteration writes them
         if (COUNT) {
             int tx0 = 0, tx1 = -1, ty0 = 0, ty1 = -1;
-            const bool any = live && bin_rect(g, V, R.xh, R.yh, tx0, tx1, ty0, ty1);
+            const bool any = live && bin_rect(g, V, R, tx0, tx1, ty0, ty1);
             if (f < M.nF) g.brect[V.frec_off + f] = pack_brect(any, tx0, tx1, ty0, ty1);
             bin_walk<0>(g, V, f, any, tx0, tx1, ty0, ty1);
         }
@@ -327,7 +326,7 @@ __global__ void k_bin(Globals g)
         bool any = false;
         if (b == BRECT_WIDE) {
             FaceRec R;
-            any = face_get(g, V, M, f, R) && bin_rect(g, V, R.xh, R.yh, tx0, tx1, ty0, ty1);
+            any = face_get(g, V, M, f, R) && bin_rect(g, V, R, tx0, tx1, ty0, ty1);
         } else if (b != BRECT_NONE) {
             tx0 = b & 2047;
             ty0 = (b >> 11) & 2047;

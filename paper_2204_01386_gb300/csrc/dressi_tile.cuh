@@ -14,7 +14,8 @@
 //      warps; each pixel keeps its K smallest (key, id) pairs in shared memory (depth
 //      peeling of Alg. 2 as a per-pixel K-selection, the rows of K-lists rotated so that
 //      neighbouring pixels use different banks; the re-rasterizing adjoint starts from
-//      the forward's K-th pair when the forward kept it);
+//      the forward's words when the forward left them); without stored layer ids only the
+//      front hard fragment is kept first, and the K layers follow inside the edge mask;
 //   3. the hard stencil S^H of a ring of rho pixels around the tile is built from the
 //      same staged faces (hard test only), so the edge mask E of every tile pixel is
 //      known without a second pass over the image;
@@ -48,6 +49,13 @@ constexpr unsigned long long EMPTY = ~0ULL;
 constexpr int WQ = 160;                // a warp's queue of pretested pairs (31 waiting + 32 items x 4)
 constexpr int QN = NT / 32 * WQ;       // the CTA's warp queues
 constexpr int NBLK = 1024;             // pair blocks of 32 with a table entry (32,768 items)
+// the raster's passes (tile_body)
+constexpr int ST_FRONT = 0, ST_LAYERS = 1, ST_DONE = 2;
+// a pixel's word from a forward without layer ids: nothing, the K-th (key, id) of every pixel, or
+// E and S^H with the K-th (key, id) where E = 1, else the front one (keys are below 2: the two top
+// bits are free)
+constexpr int KTH_NONE = 0, KTH_LAST = 0x01010101, KTH_FRONTS = 0x02020202;
+constexpr unsigned long long KTH_SH = 1ull << 63, KTH_E = 1ull << 62, KTH_BITS = KTH_E - 1;
 
 // conservative tile-local data of a staged face: edge equations in pixels relative to
 // the tile origin (FP32, a few 1e-6 px of error) and the smallest corner depth.  12 words:
@@ -77,8 +85,8 @@ __device__ __forceinline__ void make_pre(const FaceGeo &R, bool live, float tx0,
     float vx[3], vy[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        vx[i] = (R.xh[i] - tx0) + R.xl[i];
-        vy[i] = (R.yh[i] - ty0) + R.yl[i];
+        vx[i] = (R.c[i].xh - tx0) + R.c[i].xl;
+        vy[i] = (R.c[i].yh - ty0) + R.c[i].yl;
     }
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
@@ -87,7 +95,7 @@ __device__ __forceinline__ void make_pre(const FaceGeo &R, bool live, float tx0,
         float nx = orient ? -ey : ey, ny = orient ? ex : -ex;
         // 1 / |edge| of the record (same edge, accurate corners): within a few ulp of
         // this edge's own length, far inside the pretest's slack
-        const float s = isfinite(R.invL[i]) ? R.invL[i] : 0.f;
+        const float s = isfinite(R.invL[i]) ? fabsf(R.invL[i]) : 0.f;
         nx *= s; ny *= s;
         P.nx[i] = nx; P.ny[i] = ny;
         P.c[i] = -(nx * vx[i] + ny * vy[i]);
@@ -361,8 +369,8 @@ __device__ __forceinline__ bool layer_adjoint(const Globals &g, const ViewK &V, 
     float dx[3], dy[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        dx[i] = (px - R.xh[i]) - R.xl[i];
-        dy[i] = (py - R.yh[i]) - R.yl[i];
+        dx[i] = (px - R.c[i].xh) - R.c[i].xl;
+        dy[i] = (py - R.c[i].yh) - R.c[i].yl;
     }
     float gX[3] = {0.f, 0.f, 0.f}, gY[3] = {0.f, 0.f, 0.f}, gW[3] = {0.f, 0.f, 0.f};
     const float o = (R.flags & 1) ? 1.f : -1.f;
@@ -562,7 +570,7 @@ __device__ __forceinline__ bool layer_adjoint(const Globals &g, const ViewK &V, 
         }
         if (L.fr.hard) {
             // lam_i = cross(V_B - V_A, p - V_A) / A2,  A = i+1, B = i+2
-            const float iA2 = o * R.invA;
+            const float iA2 = R.invA;
             float gA2 = 0.f;
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
@@ -659,6 +667,8 @@ struct Smem {
     int item_ctr;        // raster: the next (face, row segment) item of the chunk a warp takes
     int qn[2];           // the stored-ids adjoint: its layer ring's items queued / taken
     unsigned long long m0[HS_MAX], m1[HS_MAX];   // per halo row: columns with S^H = 0 / 1
+    unsigned eb[TT_MAX], hb[TT_MAX];   // per tile row: pixels with E = 1, with S^H = 1
+    unsigned rm[TT_MAX];               // per tile row: pixels that the raster pass serves
     unsigned char sh[HS_MAX * HS_MAX];
     // the raster (forward and re-rasterizing adjoint) only: the modes from stored layer
     // ids are launched with the shared memory up to F (the stored-ids adjoint adds its
@@ -667,7 +677,7 @@ struct Smem {
     FaceGeo F[CH];       // the staged chunk's faces (geometric part)
     int fid[CH];         // their face ids
     Pre P[CH];
-    int rect[CH];        // tile pairs: x0 | y0 << 8 | w << 16 | h << 24 (tile-local, x0/y0 >= 0)
+    int rect[CH];        // tile pixels: x0 | y0 << 8 | w << 16 | h << 24 (tile-local, x0/y0 >= 0)
     int hrect[CH];       // ring pairs: (x0 + 16) | (y0 + 16) << 8 | w << 16 | h << 24
     int start[CH];       // exclusive prefix of tile segments (4-pixel row pieces of the rects)
     int hstart[CH];      // exclusive prefix of ring pairs
@@ -773,16 +783,58 @@ __device__ __forceinline__ bool kept_hard(const Globals &g, const ViewK &V, cons
            eval_face<false>(R, px, py, V.r_px, V.half_inv_S, fr) && fr.hard;
 }
 
-// edge mask (Sec. 3.4.3) of tile pixel (lx, ly): the window of radius rho sees both
-// S^H = 0 and 1 (S.m0 / S.m1 hold the columns of each halo row with either value)
-__device__ __forceinline__ bool edge_mask(const Globals &g, const Smem &S, int lx, int ly, int rho)
+// per halo row, the columns holding S^H = 0 and S^H = 1 (hs <= 48 fits 64 bits)
+template <int TT>
+__device__ __forceinline__ void halo_rows(Smem &S, int hs)
 {
-    if (g.edge_mode != 0) return g.edge_mode == 1;
-    unsigned long long a0 = 0ull, a1 = 0ull;
-    for (int wy = 0; wy <= 2 * rho; ++wy) { a0 |= S.m0[ly + wy]; a1 |= S.m1[ly + wy]; }
-    const unsigned long long wm = (2ull << (2 * rho)) - 1ull;   // columns lx .. lx + 2 rho
-    return ((a0 >> lx) & wm) && ((a1 >> lx) & wm);
+    const int lane = threadIdx.x & 31;
+    for (int row = threadIdx.x >> 5; row < hs; row += NT / 32) {
+        unsigned long long b0 = 0ull, b1 = 0ull;
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const int col = half * 32 + lane;
+            const unsigned char v = col < hs ? S.sh[row * hs + col] : (unsigned char)2;
+            b0 |= (unsigned long long)__ballot_sync(0xffffffffu, v == 0) << (32 * half);
+            b1 |= (unsigned long long)__ballot_sync(0xffffffffu, v == 1) << (32 * half);
+        }
+        if (lane == 0) { S.m0[row] = b0; S.m1[row] = b1; }
+    }
 }
+
+// rows[ly] bit lx = pred, for the 32 consecutive tile pixels p of a warp (all lanes call it)
+template <int TT>
+__device__ __forceinline__ void row_masks(unsigned *rows, int p, bool pred)
+{
+    const unsigned b = __ballot_sync(0xffffffffu, pred);
+    if (TT == 32) {
+        if ((p & 31) == 0) rows[p / 32] = b;
+    } else if ((p & 15) == 0) {
+        rows[p / 16] = (b >> (p & 16)) & 0xffffu;
+    }
+}
+
+// S^H and the edge mask E (Sec. 3.4.3) of the tile's pixels as row bitmasks, from S.m0 / S.m1
+// (per halo row the columns with S^H = 0 and 1): E where the window of radius rho holds both.
+// One thread per row: the window's rows are or-ed, then shifted copies of the result, instead
+// of a window walk per pixel.  The caller's next barrier publishes the rows.
+template <int TT>
+__device__ __forceinline__ void edge_rows(const Globals &g, Smem &S, int rho, int wlim, int hlim)
+{
+    const int ly = threadIdx.x;
+    if (ly >= TT) return;
+    const unsigned in = ly < hlim ? 0xffffffffu >> (32 - wlim) : 0u;
+    unsigned e = g.edge_mode == 1 ? in : 0u;
+    if (g.edge_mode == 0) {
+        unsigned long long a0 = 0ull, a1 = 0ull;
+        for (int wy = 0; wy <= 2 * rho; ++wy) { a0 |= S.m0[ly + wy]; a1 |= S.m1[ly + wy]; }
+        unsigned long long d0 = 0ull, d1 = 0ull;
+        for (int wx = 0; wx <= 2 * rho; ++wx) { d0 |= a0 >> wx; d1 |= a1 >> wx; }
+        e = (unsigned)(d0 & d1) & in;
+    }
+    S.eb[ly] = e;
+    S.hb[ly] = (unsigned)(S.m1[ly + rho] >> rho) & in;
+}
+__device__ __forceinline__ bool row_bit(const unsigned *rows, int lx, int ly) { return (rows[ly] >> lx) & 1u; }
 
 // the adjoint of the edge-mask blend (Sec. 3.4.3) at one pixel: the colour
 // sum_k D_k C_k / sum_k D_k and the silhouette 1 - prod_k (1 - D_k), from the nl layers'
@@ -862,18 +914,16 @@ __device__ __forceinline__ bool pixel_weights(const Globals &g, const ViewK &V, 
 // ring.
 template <int K, int TT, bool EXTRA>
 __device__ __forceinline__ unsigned adjoint_pixel(const Globals &g, const Smem &S, const ViewK &V, const MeshK &M,
-                                                  int X0, int Y0, int lx, int ly, int rho, const int (&ids)[K],
+                                                  int X0, int Y0, int lx, int ly, const int (&ids)[K],
                                                   float *gl)
 {
     const int X = X0 + lx, Y = Y0 + ly;   // view-local pixel coordinates
     const float px = (float)X + 0.5f, py = (float)Y + 0.5f;
-    const int hs = TT + 2 * rho;
     const long long pix = V.pix_off + (long long)Y * V.W + X;
     int nl = 0;
 #pragma unroll
     for (int k = 0; k < K; ++k) nl += (ids[k] != 0x7fffffff) ? 1 : 0;
-    const bool SH = S.sh[(ly + rho) * hs + (lx + rho)] == 1;
-    const bool E = edge_mask(g, S, lx, ly, rho);
+    const bool SH = row_bit(S.hb, lx, ly), E = row_bit(S.eb, lx, ly);
 
     unsigned layers = 0;
     const bool inv = EXTRA && g.texgrad_mode == 2;
@@ -915,13 +965,12 @@ __device__ __forceinline__ unsigned adjoint_pixel(const Globals &g, const Smem &
 // shuffles and blends them in layer order.
 template <int K, int TT, bool EXTRA>
 __device__ __forceinline__ unsigned finish_forward(const Globals &g, const Smem &S, const ViewK &V, const MeshK &M,
-                                                   int X0, int Y0, int p, int rho, bool in, const int (&ids)[K],
+                                                   int X0, int Y0, int p, bool in, const int (&ids)[K],
                                                    unsigned hardbits, bool single_chunk, float &l2acc)
 {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int lx = p % TT, ly = p / TT;
-    const int hs = TT + 2 * rho;
     int nl = 0;
     bool SH = false, E = false;
     long long pix = 0;
@@ -929,8 +978,8 @@ __device__ __forceinline__ unsigned finish_forward(const Globals &g, const Smem 
         pix = V.pix_off + (long long)(Y0 + ly) * V.W + (X0 + lx);
 #pragma unroll
         for (int k = 0; k < K; ++k) nl += (ids[k] != 0x7fffffff) ? 1 : 0;
-        SH = S.sh[(ly + rho) * hs + (lx + rho)] == 1;
-        E = edge_mask(g, S, lx, ly, rho);
+        SH = row_bit(S.hb, lx, ly);
+        E = row_bit(S.eb, lx, ly);
         if (g.ids) {
 #pragma unroll
             for (int k = 0; k < K; ++k) {
@@ -1044,12 +1093,11 @@ __device__ __forceinline__ unsigned finish_forward(const Globals &g, const Smem 
 // back-propagates the layers with a gradient as a second list.
 template <int K, int TT>
 __device__ __forceinline__ unsigned adjoint_warp(const Globals &g, const Smem &S, const ViewK &V, const MeshK &M,
-                                                 int X0, int Y0, int p, int rho, bool in, const int (&ids)[K])
+                                                 int X0, int Y0, int p, bool in, const int (&ids)[K])
 {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int lx = p % TT, ly = p / TT;
-    const int hs = TT + 2 * rho;
     int nl = 0;
     bool E = false, SH = false, active = false;
     float4 gi4 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1060,8 +1108,8 @@ __device__ __forceinline__ unsigned adjoint_warp(const Globals &g, const Smem &S
             gi4 = __ldg(reinterpret_cast<const float4 *>(g.gin) + V.pix_off + (long long)(Y0 + ly) * V.W + (X0 + lx));
             active = gi4.x != 0.f || gi4.y != 0.f || gi4.z != 0.f || gi4.w != 0.f;
             if (active) {
-                SH = S.sh[(ly + rho) * hs + (lx + rho)] == 1;
-                E = edge_mask(g, S, lx, ly, rho);
+                SH = row_bit(S.hb, lx, ly);
+                E = row_bit(S.eb, lx, ly);
             }
         }
     }
@@ -1207,7 +1255,7 @@ __host__ __device__ constexpr size_t adj_smem_bytes()
 
 template <int K, int TT>
 __device__ __forceinline__ unsigned adjoint_queued(const Globals &g, Smem &S, const ViewK &V, const MeshK &M,
-                                                   int X0, int Y0, int rho, int wlim, int hlim)
+                                                   int X0, int Y0, int wlim, int hlim)
 {
     constexpr int PPT = TT * TT / NT;
     constexpr int QC = adj_ring<K>();
@@ -1216,7 +1264,6 @@ __device__ __forceinline__ unsigned adjoint_queued(const Globals &g, Smem &S, co
     float4 *dc = reinterpret_cast<float4 *>(qi + QC);    // [thread][layer]: (C_k, D_k)
     unsigned short *bq = reinterpret_cast<unsigned short *>(dc + NT * K);   // thread | layer << 8
     const int tid = threadIdx.x, lane = tid & 31;
-    const int hs = TT + 2 * rho;
     unsigned layers = 0;
     // S.qn[0]: adjoint items queued, S.qn[1]: taken (both zero at the tile's start);
     // S.totals[0]: blend items of the round
@@ -1260,10 +1307,9 @@ __device__ __forceinline__ unsigned adjoint_queued(const Globals &g, Smem &S, co
 #pragma unroll
             for (int k = 0; k < K; ++k) nl += idk[k] != -1 ? 1 : 0;
             if (nl > 0 && (gi4.x != 0.f || gi4.y != 0.f || gi4.z != 0.f || gi4.w != 0.f)) {
-                E = edge_mask(g, S, lx, ly, rho);
+                E = row_bit(S.eb, lx, ly);
                 // outside the mask the pixel is its front layer's colour where S^H = 1
-                front = !E && S.sh[(ly + rho) * hs + (lx + rho)] == 1 &&
-                        (gi4.x != 0.f || gi4.y != 0.f || gi4.z != 0.f);
+                front = !E && row_bit(S.hb, lx, ly) && (gi4.x != 0.f || gi4.y != 0.f || gi4.z != 0.f);
                 id0 = idk[0] & 0x7fffffff;
             }
         }
@@ -1353,16 +1399,19 @@ __device__ __forceinline__ unsigned adjoint_queued(const Globals &g, Smem &S, co
 // WQ entries in shared memory), and whenever it holds 32 of them the warp evaluates them
 // exactly with all lanes and merges the candidates into the pixels' K-lists (other warps
 // merge into the same lists concurrently: the atomicMin cascade is order independent).
+// The pass takes fragments within `reach` of the pixels in S.rm, or (fronts) the front hard
+// fragment alone, which slot 0 then holds.
 // A queue entry is x | y << 5 | face << 10 with the top 14 bits of the key lower bound
 // above (truncated: still a lower bound).
 template <int K, int TT>
 __device__ __forceinline__ void raster_items(Smem &S, unsigned long long *kbuf, unsigned *wq,
                                              const unsigned char *blk, const ViewK &V, int X0, int Y0, int nch,
-                                             int total, bool count, unsigned &n_pairs, unsigned &n_exact,
-                                             unsigned &n_cand)
+                                             int total, float reach, bool fronts, bool count, unsigned &n_pairs,
+                                             unsigned &n_exact, unsigned &n_cand)
 {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
+    const int sl = fronts ? 0 : K - 1;   // the list slot that a pair has to beat
     int head = 0, qn = 0;   // the warp's queue: qn entries from wq[head] on (warp-uniform)
     // exact evaluation of the n <= 32 entries at the queue's head, one per lane
     auto evaluate = [&](int n) {
@@ -1372,14 +1421,19 @@ __device__ __forceinline__ void raster_items(Smem &S, unsigned long long *kbuf, 
             const unsigned ent = wq[q];
             const int x = ent & 31, y = (ent >> 5) & 31, f = (ent >> 10) & 0xff;
             unsigned long long *slots = kbuf + kslot<TT>(x, y) * K;
-            const unsigned long long last = *reinterpret_cast<volatile unsigned long long *>(slots + K - 1);
+            const unsigned long long last = *reinterpret_cast<volatile unsigned long long *>(slots + sl);
             if (!(__uint_as_float(ent & 0xfffc0000u) > __uint_as_float((unsigned int)(last >> 32)))) {
                 Frag fr;
                 ++n_exact;
-                if (eval_face<false>(S.F[f], (float)(X0 + x) + 0.5f, (float)(Y0 + y) + 0.5f, V.r_px, V.half_inv_S,
-                                     fr)) {
+                if (eval_face<false>(S.F[f], (float)(X0 + x) + 0.5f, (float)(Y0 + y) + 0.5f, reach, V.half_inv_S, fr,
+                                     fronts)) {
                     ++n_cand;
-                    kbuf_insert<K>(slots, pack_frag(fr.key, S.fid[f]));
+                    const unsigned long long v = pack_frag(fr.key, S.fid[f]);
+                    // the slot's entry only ever gets smaller: a value not below it stays out
+                    if (v < last) {
+                        if (fronts) atomicMin(slots, v);
+                        else kbuf_insert<K>(slots, v);
+                    }
                 }
             }
         }
@@ -1407,6 +1461,7 @@ __device__ __forceinline__ void raster_items(Smem &S, unsigned long long *kbuf, 
             y = ((rc >> 8) & 0xff) + qy;
             const int np = min(4, (rc & 0xff) + w - x);
             if (count) n_pairs += np;
+            const unsigned todo = (S.rm[y] >> x) & ((1u << np) - 1u);
             const Pre &P = S.P[f];
             const float fx = (float)x + 0.5f, fy = (float)y + 0.5f;
             float e0 = fmaf(P.nx[0], fx, fmaf(P.ny[0], fy, P.c[0]));
@@ -1415,14 +1470,14 @@ __device__ __forceinline__ void raster_items(Smem &S, unsigned long long *kbuf, 
             const float klb_in = 0.5f * P.zmin * (1.f - 1e-6f);
             // the K-th slots change under other warps' merges; any value read is an upper
             // bound of the final one, so a pair culled against it stays culled
-            const volatile unsigned long long *last = kbuf + K - 1;
+            const volatile unsigned long long *last = kbuf + sl;
             const int row = y * TT, sw = kswz(y);
 #pragma unroll
             for (int d = 0; d < 4; ++d) {
                 // F(p) ~ the smallest edge value: outside, the distance is at least -F;
                 // inside, the depth is at least the smallest corner depth
                 const float fmin = fminf(e0, fminf(e1, e2));
-                if (d < np && fmin >= -V.r_px - APPROX_EPS) {
+                if (((todo >> d) & 1u) && fmin >= -reach - APPROX_EPS) {
                     const float klb = fmin > APPROX_EPS    ? klb_in
                                       : fmin < -APPROX_EPS ? fmaf(-fmin - APPROX_EPS, V.half_inv_S, 0.5f)
                                                            : 0.f;
@@ -1506,6 +1561,7 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
     if (light_grad) glacc[0] = glacc[1] = glacc[2] = 0.f;
     bool single_chunk = false;
     bool empty = false;   // a forward over a tile that no face reaches
+    bool handed = false;  // E, S^H and the front layers come from the forward's words
     unsigned n_pairs = 0, n_exact = 0, n_cand = 0, n_layers = 0;
     float l2acc = 0.f;   // the fused L2 loss: this thread's sum of squares
     if (!from_ids) {
@@ -1518,10 +1574,40 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
         // a forward over such a tile has no layer and S^H = 0 in the tile and its ring (no
         // face comes within the binning radius), so E = 0 or no layer to blend: background
         empty = n == 0;
+        // what the forward left in the workspace for a re-rasterizing adjoint
+        const int words = BWD && g.kth ? *g.kth_flag : 0;
+        handed = words == KTH_FRONTS;
+        bool layered = !g.fronts;   // the K layers of every pixel are wanted
+        int stage = g.fronts ? ST_FRONT : ST_LAYERS;
         if (!empty)   // 16-byte stores (TT^2 K is even; kbuf is 16-byte aligned)
             for (int i = tid; i < TT * TT * K / 2; i += NT)
                 reinterpret_cast<ulonglong2 *>(kbuf)[i] = make_ulonglong2(EMPTY, EMPTY);
-        if (BWD && g.kth && *g.kth_flag) {
+        if (tid < TT_MAX) S.rm[tid] = 0xffffffffu;
+        if (handed) {
+            bool any = false, some = false;
+            __syncthreads();   // after the clearing stores
+#pragma unroll
+            for (int j = 0; j < PPT; ++j) {
+                const int p = tid + j * NT, lx = p % TT, ly = p / TT;
+                bool E = false, SH = false;
+                if (lx < wlim && ly < hlim) {
+                    const unsigned long long w = g.kth[V.slot_base + (long long)(Y0 + ly) * V.W + (X0 + lx)];
+                    E = (w & KTH_E) != 0;
+                    SH = (w & KTH_SH) != 0;
+                    const unsigned long long v = w & KTH_BITS;
+                    // an edge-masked pixel's K-th entry seeds its list; else the front layer
+                    if (v != KTH_BITS) kbuf[kslot<TT>(lx, ly) * K + (E ? K - 1 : 0)] = v;
+                }
+                row_masks<TT>(S.eb, p, E);
+                row_masks<TT>(S.hb, p, SH);
+                row_masks<TT>(S.rm, p, E);
+                any |= E;
+                some |= E || SH;
+            }
+            // only front layers outside the edge mask, and nothing at all: done
+            if (!__syncthreads_or(some)) return;
+            stage = __syncthreads_or(any) ? ST_LAYERS : ST_DONE;
+        } else if (words == KTH_LAST) {
             // the forward's K-th (key, id) of every pixel as a first entry of its K-list: it
             // is the K-th smallest of the pixel's candidates, so it stays in the last slot and
             // every pair whose key bound exceeds it is culled; its own pair finds it there
@@ -1531,147 +1617,220 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
                 if (lx < wlim && ly < hlim)
                     kbuf[kslot<TT>(lx, ly) * K + K - 1] = g.kth[V.slot_base + (long long)(Y0 + ly) * V.W + (X0 + lx)];
             }
+            stage = ST_LAYERS;
+            layered = true;
         }
+        // The raster's passes over the face list:
+        //   ST_FRONT  hard fragments alone, the front one kept: all that a pixel outside the edge
+        //             mask shows.  Where the mask holds a pixel of the tile, ST_LAYERS follows for
+        //             the masked pixels, from empty lists.
+        //   ST_LAYERS the K nearest fragments of the pixels in S.rm.
+        // Soft candidates are the bulk of the pairs (a face of 2.6 px grown by r = 2 px covers 13
+        // times its area), and without stored ids nothing outside the mask reads them: on two
+        // 2048^2 views of a 1.31 M-face mesh 127 -> 45 M pairs and 53 -> 8 M exact evaluations, the
+        // forward 1667 -> 1130 us, the adjoint 1541 -> 764 us (four 768^2 views of 32,000 faces:
+        // 310 -> 244 and 350 -> 217 us).
+        bool ring = rho > 0 && !handed;
         single_chunk = n <= CH;
         // the id -> slot hash serves the forward's shading of a tile staged in one chunk
         const bool use_hash = !BWD && single_chunk;
-        for (int c0 = 0; c0 < n; c0 += CH) {
-            const int nch = min(CH, n - c0);
-            // the next chunk's face ids, loaded under this chunk's staging: their records
-            // are prefetched into L2 once this chunk is staged
-            const int nnext = min(CH, n - c0 - CH);
-            int fnext = -1;
-            if (tid < nnext) fnext = fallback ? c0 + CH + tid : g.lists[lb + c0 + CH + tid];
-            __syncthreads();   // previous chunk consumed
-            if (use_hash) {
-                for (int i = tid; i < HASH; i += NT) S.hash[i] = make_int2(-1, -1);
-                __syncthreads();
-            }
-            int cnt = 0, hcnt = 0;
-            if (tid < nch) {
-                const int f = fallback ? c0 + tid : g.lists[lb + c0 + tid];
-                FaceGeo &R = S.F[tid];
-                S.fid[tid] = f;
-                const bool live = face_stage(g, V, M, f, R);
-                Box B;
-                make_pre(R, live, (float)X0, (float)Y0, V.r_px, S.P[tid], B);
-                if (live) {
-                    // pixel centres lx + 1/2 inside [bx0, bx1] (grown by r), clipped to the tile and image
-                    const int x0 = max(0, (int)ceilf(B.bx0 - 0.5f - APPROX_EPS));
-                    const int x1 = min(wlim - 1, (int)floorf(B.bx1 - 0.5f + APPROX_EPS));
-                    const int y0 = max(0, (int)ceilf(B.by0 - 0.5f - APPROX_EPS));
-                    const int y1 = min(hlim - 1, (int)floorf(B.by1 - 0.5f + APPROX_EPS));
-                    const int w = x1 - x0 + 1, h = y1 - y0 + 1;
-                    if (w > 0 && h > 0) {
-                        cnt = ((w + 3) >> 2) * h;   // segments of up to 4 pixels per row
-                        S.rect[tid] = x0 | (y0 << 8) | (w << 16) | (h << 24);
-                        S.rdiv[tid] = rect_div((w + 3) >> 2);
-                    }
-                    if (rho > 0) {
-                        // hard bbox (without r) against the ring [-rho, TT + rho), clipped to the image
-                        const float r = V.r_px;
-                        const int hx0 = max(max(-rho, -X0), (int)ceilf(B.bx0 + r - 0.5f - APPROX_EPS));
-                        const int hx1 = min(min(TT + rho, V.W - X0) - 1, (int)floorf(B.bx1 - r - 0.5f + APPROX_EPS));
-                        const int hy0 = max(max(-rho, -Y0), (int)ceilf(B.by0 + r - 0.5f - APPROX_EPS));
-                        const int hy1 = min(min(TT + rho, V.H - Y0) - 1, (int)floorf(B.by1 - r - 0.5f + APPROX_EPS));
-                        // only faces reaching outside the tile interior have ring pixels; a box
-                        // that leaves the tile across one side only is cut to its part outside
-                        const bool ring = hx0 < 0 || hy0 < 0 || hx1 >= TT || hy1 >= TT;
-                        int rx0 = hx0, rx1 = hx1, ry0 = hy0, ry1 = hy1;
-                        if (hx0 >= 0 && hx1 < TT) {
-                            if (hy1 < TT) ry1 = min(hy1, -1);
-                            else if (hy0 >= 0) ry0 = max(hy0, TT);
-                        } else if (hy0 >= 0 && hy1 < TT) {
-                            if (hx1 < TT) rx1 = min(hx1, -1);
-                            else if (hx0 >= 0) rx0 = max(hx0, TT);
+        while (stage != ST_DONE && !empty) {
+            const float reach = stage == ST_FRONT ? 0.f : V.r_px;
+            for (int c0 = 0; c0 < n; c0 += CH) {
+                const int nch = min(CH, n - c0);
+                // the next chunk's face ids, loaded under this chunk's staging: their records
+                // are prefetched into L2 once this chunk is staged
+                const int nnext = min(CH, n - c0 - CH);
+                int fnext = -1;
+                if (tid < nnext) fnext = fallback ? c0 + CH + tid : g.lists[lb + c0 + CH + tid];
+                __syncthreads();   // previous chunk consumed
+                if (use_hash) {
+                    for (int i = tid; i < HASH; i += NT) S.hash[i] = make_int2(-1, -1);
+                    __syncthreads();
+                }
+                int cnt = 0, hcnt = 0;
+                if (tid < nch) {
+                    const int f = fallback ? c0 + tid : g.lists[lb + c0 + tid];
+                    FaceGeo &R = S.F[tid];
+                    S.fid[tid] = f;
+                    const bool live = face_stage(g, V, M, f, R);
+                    Box B;
+                    make_pre(R, live, (float)X0, (float)Y0, reach, S.P[tid], B);
+                    if (live) {
+                        // pixel centres lx + 1/2 inside [bx0, bx1] (grown by the reach), clipped to the tile and image
+                        const int x0 = max(0, (int)ceilf(B.bx0 - 0.5f - APPROX_EPS));
+                        const int x1 = min(wlim - 1, (int)floorf(B.bx1 - 0.5f + APPROX_EPS));
+                        const int y0 = max(0, (int)ceilf(B.by0 - 0.5f - APPROX_EPS));
+                        const int y1 = min(hlim - 1, (int)floorf(B.by1 - 0.5f + APPROX_EPS));
+                        const int w = x1 - x0 + 1, h = y1 - y0 + 1;
+                        if (w > 0 && h > 0) {
+                            cnt = ((w + 3) >> 2) * h;   // segments of up to 4 pixels per row
+                            S.rect[tid] = x0 | (y0 << 8) | (w << 16) | (h << 24);
+                            S.rdiv[tid] = rect_div((w + 3) >> 2);
                         }
-                        const int hw = rx1 - rx0 + 1, hh = ry1 - ry0 + 1;
-                        if (hw > 0 && hh > 0 && ring) {
-                            hcnt = hw * hh;
-                            S.hrect[tid] = (rx0 + 16) | ((ry0 + 16) << 8) | (hw << 16) | (hh << 24);
-                            S.hdiv[tid] = rect_div(hw);
+                        if (ring) {
+                            // hard bbox (without the reach) against the ring [-rho, TT + rho), clipped to the image
+                            const float r = reach;
+                            const int hx0 = max(max(-rho, -X0), (int)ceilf(B.bx0 + r - 0.5f - APPROX_EPS));
+                            const int hx1 = min(min(TT + rho, V.W - X0) - 1, (int)floorf(B.bx1 - r - 0.5f + APPROX_EPS));
+                            const int hy0 = max(max(-rho, -Y0), (int)ceilf(B.by0 + r - 0.5f - APPROX_EPS));
+                            const int hy1 = min(min(TT + rho, V.H - Y0) - 1, (int)floorf(B.by1 - r - 0.5f + APPROX_EPS));
+                            // only faces reaching outside the tile interior have ring pixels; a box
+                            // that leaves the tile across one side only is cut to its part outside
+                            const bool out = hx0 < 0 || hy0 < 0 || hx1 >= TT || hy1 >= TT;
+                            int rx0 = hx0, rx1 = hx1, ry0 = hy0, ry1 = hy1;
+                            if (hx0 >= 0 && hx1 < TT) {
+                                if (hy1 < TT) ry1 = min(hy1, -1);
+                                else if (hy0 >= 0) ry0 = max(hy0, TT);
+                            } else if (hy0 >= 0 && hy1 < TT) {
+                                if (hx1 < TT) rx1 = min(hx1, -1);
+                                else if (hx0 >= 0) rx0 = max(hx0, TT);
+                            }
+                            const int hw = rx1 - rx0 + 1, hh = ry1 - ry0 + 1;
+                            if (hw > 0 && hh > 0 && out) {
+                                hcnt = hw * hh;
+                                S.hrect[tid] = (rx0 + 16) | ((ry0 + 16) << 8) | (hw << 16) | (hh << 24);
+                                S.hdiv[tid] = rect_div(hw);
+                            }
                         }
-                    }
-                    // id -> slot for the shading phase
-                    if (use_hash) {
-                        unsigned hsh = ((unsigned)f * 2654435761u) & (HASH - 1);
-                        for (int probe = 0; probe < HASH; ++probe) {
-                            const int prev = atomicCAS(&S.hash[hsh].x, -1, f);
-                            if (prev == -1 || prev == f) { S.hash[hsh].y = tid; break; }
-                            hsh = (hsh + 1) & (HASH - 1);
+                        // id -> slot for the shading phase
+                        if (use_hash) {
+                            unsigned hsh = ((unsigned)f * 2654435761u) & (HASH - 1);
+                            for (int probe = 0; probe < HASH; ++probe) {
+                                const int prev = atomicCAS(&S.hash[hsh].x, -1, f);
+                                if (prev == -1 || prev == f) { S.hash[hsh].y = tid; break; }
+                                hsh = (hsh + 1) & (HASH - 1);
+                            }
                         }
                     }
                 }
-            }
-            if ((unsigned)fnext < (unsigned)M.nF) {
-                // both 128-byte lines a 112-byte record can touch
-                const char *a = reinterpret_cast<const char *>(g.frec + V.frec_off + fnext);
-                prefetch_l2(a);
-                prefetch_l2(a + sizeof(FaceRec) - 1);
-            }
-            // exclusive prefix of the two pair counts over the chunk
-            {
-                const int lane = tid & 31, wp = tid >> 5;
-                int a = cnt, b = hcnt;
+                if ((unsigned)fnext < (unsigned)M.nF) {
+                    // both 128-byte lines a 112-byte record can touch
+                    const char *a = reinterpret_cast<const char *>(g.frec + V.frec_off + fnext);
+                    prefetch_l2(a);
+                    prefetch_l2(a + sizeof(FaceRec) - 1);
+                }
+                // exclusive prefix of the row and ring pair counts over the chunk
+                {
+                    const int lane = tid & 31, wp = tid >> 5;
+                    int a = cnt, b = hcnt;
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int ya = __shfl_up_sync(0xffffffffu, a, o), yb = __shfl_up_sync(0xffffffffu, b, o);
-                    if (lane >= o) { a += ya; b += yb; }
-                }
-                if (lane == 31) { S.wsum[0][wp] = a; S.wsum[1][wp] = b; }
-                __syncthreads();
-                int oa = 0, ob = 0, ta = 0, tb = 0;
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int ya = __shfl_up_sync(0xffffffffu, a, o), yb = __shfl_up_sync(0xffffffffu, b, o);
+                        if (lane >= o) { a += ya; b += yb; }
+                    }
+                    if (lane == 31) { S.wsum[0][wp] = a; S.wsum[1][wp] = b; }
+                    __syncthreads();
+                    int oa = 0, ob = 0, ta = 0, tb = 0;
 #pragma unroll
-                for (int w = 0; w < NT / 32; ++w) {
-                    const int va = S.wsum[0][w], vb = S.wsum[1][w];
-                    if (w < wp) { oa += va; ob += vb; }
-                    ta += va; tb += vb;
+                    for (int w = 0; w < NT / 32; ++w) {
+                        const int va = S.wsum[0][w], vb = S.wsum[1][w];
+                        if (w < wp) { oa += va; ob += vb; }
+                        ta += va; tb += vb;
+                    }
+                    if (tid < CH) {
+                        S.start[tid] = oa + a - cnt;
+                        S.hstart[tid] = ob + b - hcnt;
+                        fill_blocks(blk, tid, oa + a - cnt, cnt);
+                        fill_blocks(hblk, tid, ob + b - hcnt, hcnt);
+                    }
+                    if (tid == 0) { S.totals[0] = ta; S.totals[1] = tb; S.item_ctr = 0; }
                 }
-                if (tid < CH) {
-                    S.start[tid] = oa + a - cnt;
-                    S.hstart[tid] = ob + b - hcnt;
-                    fill_blocks(blk, tid, oa + a - cnt, cnt);
-                    fill_blocks(hblk, tid, ob + b - hcnt, hcnt);
+                __syncthreads();
+                const int total = S.totals[0], htotal = S.totals[1];
+                raster_items<K, TT>(S, kbuf, qbuf + (tid >> 5) * WQ, blk, V, X0, Y0, nch, total, reach,
+                                    stage == ST_FRONT, g.stats != nullptr, n_pairs, n_exact, n_cand);
+                // (face, pixel) pairs of the ring: hard test only
+                for (int i = tid; i < htotal; i += NT) {
+                    const int f = pair_face(S.hstart, hblk, nch, i - (tid & 31), i);
+                    const int rc = S.hrect[f];
+                    int x, y;
+                    rect_xy(i - S.hstart[f], (rc >> 16) & 0xff, S.hdiv[f], x, y);
+                    x += (rc & 0xff) - 16;
+                    y += ((rc >> 8) & 0xff) - 16;
+                    if (x >= 0 && x < TT && y >= 0 && y < TT) continue;   // interior: decided by the peel
+                    const int si = (y + rho) * hs + (x + rho);
+                    if (S.sh[si] != 0) continue;
+                    const Pre &P = S.P[f];
+                    const float fx = (float)x + 0.5f, fy = (float)y + 0.5f;
+                    const float fmin = approx_fmin(P, fx, fy);
+                    if (fmin < -APPROX_EPS) continue;
+                    // clearly inside (margin far above the FP32 error of either test) or
+                    // decided by the exact fill-rule test
+                    if (fmin > APPROX_EPS || hard_test(S.F[f], (float)(X0 + x) + 0.5f, (float)(Y0 + y) + 0.5f))
+                        S.sh[si] = 1;
                 }
-                if (tid == 0) { S.totals[0] = ta; S.totals[1] = tb; S.item_ctr = 0; }
             }
+            ring = false;
             __syncthreads();
-            const int total = S.totals[0], htotal = S.totals[1];
-            raster_items<K, TT>(S, kbuf, qbuf + (tid >> 5) * WQ, blk, V, X0, Y0, nch, total, g.stats != nullptr,
-                                n_pairs, n_exact, n_cand);
-            // (face, pixel) pairs of the ring: hard test only
-            for (int i = tid; i < htotal; i += NT) {
-                const int f = pair_face(S.hstart, hblk, nch, i - (tid & 31), i);
-                const int rc = S.hrect[f];
-                int x, y;
-                rect_xy(i - S.hstart[f], (rc >> 16) & 0xff, S.hdiv[f], x, y);
-                x += (rc & 0xff) - 16;
-                y += ((rc >> 8) & 0xff) - 16;
-                if (x >= 0 && x < TT && y >= 0 && y < TT) continue;   // interior: decided by the peel
-                const int si = (y + rho) * hs + (x + rho);
-                if (S.sh[si] != 0) continue;
-                const Pre &P = S.P[f];
-                const float fx = (float)x + 0.5f, fy = (float)y + 0.5f;
-                const float fmin = approx_fmin(P, fx, fy);
-                if (fmin < -APPROX_EPS) continue;
-                // clearly inside (margin far above the FP32 error of either test) or
-                // decided by the exact fill-rule test
-                if (fmin > APPROX_EPS || hard_test(S.F[f], (float)(X0 + x) + 0.5f, (float)(Y0 + y) + 0.5f))
-                    S.sh[si] = 1;
+            if (stage == ST_FRONT) {
+                // S^H and E from the front fragments.  A hard key below 1/2 is in front of every
+                // soft one; at exactly 1/2 (the far plane) a soft fragment could tie, and the
+                // tile's pixels get all their layers instead
+                bool tie = false;
+#pragma unroll
+                for (int j = 0; j < PPT; ++j) {
+                    const int p = tid + j * NT, lx = p % TT, ly = p / TT;
+                    if (lx >= wlim || ly >= hlim) continue;
+                    const unsigned long long v = kbuf[kslot<TT>(lx, ly) * K];
+                    tie |= v != EMPTY && !(__uint_as_float((unsigned)(v >> 32)) < 0.5f);
+                    S.sh[(ly + rho) * hs + (lx + rho)] = v != EMPTY ? 1 : 0;
+                }
+                if (__syncthreads_or(tie)) {
+                    layered = true;
+                    stage = ST_LAYERS;
+                } else {
+                    halo_rows<TT>(S, hs);
+                    __syncthreads();
+                    edge_rows<TT>(g, S, rho, wlim, hlim);
+                    const bool any = tid < TT && S.eb[tid] != 0u;
+                    stage = __syncthreads_or(any) ? ST_LAYERS : ST_DONE;
+                    if (tid < TT) S.rm[tid] = S.eb[tid];
+                }
+                if (stage == ST_LAYERS)
+#pragma unroll
+                    for (int j = 0; j < PPT; ++j) {
+                        const int p = tid + j * NT, lx = p % TT, ly = p / TT;
+                        if (layered || row_bit(S.eb, lx, ly)) kbuf[kslot<TT>(lx, ly) * K] = EMPTY;
+                    }
+            } else {
+                stage = ST_DONE;
             }
         }
-        __syncthreads();
         // S^H of the tile's own pixels from the front slot
+        if (layered && !handed) {
 #pragma unroll
-        for (int j = 0; j < PPT; ++j) {
-            const int p = tid + j * NT;
-            const int lx = p % TT, ly = p / TT;
-            if (empty || lx >= wlim || ly >= hlim) continue;
-            const int ks = kslot<TT>(lx, ly) * K;
-            if (!BWD && g.kth) g.kth[V.slot_base + (long long)(Y0 + ly) * V.W + (X0 + lx)] = kbuf[ks + K - 1];
-            const unsigned long long v = kbuf[ks];
-            const bool sh = v != EMPTY && kept_hard(g, V, M, v, (float)(X0 + lx) + 0.5f, (float)(Y0 + ly) + 0.5f);
-            S.sh[(ly + rho) * hs + (lx + rho)] = sh ? 1 : 0;
+            for (int j = 0; j < PPT; ++j) {
+                const int p = tid + j * NT;
+                const int lx = p % TT, ly = p / TT;
+                if (empty || lx >= wlim || ly >= hlim) continue;
+                const unsigned long long v = kbuf[kslot<TT>(lx, ly) * K];
+                const bool sh = v != EMPTY && kept_hard(g, V, M, v, (float)(X0 + lx) + 0.5f, (float)(Y0 + ly) + 0.5f);
+                S.sh[(ly + rho) * hs + (lx + rho)] = sh ? 1 : 0;
+            }
+            __syncthreads();
+            if (!empty) {
+                halo_rows<TT>(S, hs);
+                __syncthreads();
+                edge_rows<TT>(g, S, rho, wlim, hlim);
+                __syncthreads();
+            }
+        }
+        // a forward without layer ids leaves each pixel's word for a re-rasterizing adjoint
+        if (!BWD && g.kth && !empty) {
+#pragma unroll
+            for (int j = 0; j < PPT; ++j) {
+                const int p = tid + j * NT, lx = p % TT, ly = p / TT;
+                if (lx >= wlim || ly >= hlim) continue;
+                const unsigned long long *slots = kbuf + kslot<TT>(lx, ly) * K;
+                unsigned long long w = slots[K - 1];
+                if (g.fronts) {
+                    const bool E = row_bit(S.eb, lx, ly), SH = row_bit(S.hb, lx, ly);
+                    w = (E ? w : SH ? slots[0] : EMPTY) & KTH_BITS;
+                    w |= (E ? KTH_E : 0ull) | (SH ? KTH_SH : 0ull);
+                }
+                g.kth[V.slot_base + (long long)(Y0 + ly) * V.W + (X0 + lx)] = w;
+            }
         }
     } else {
         // layers stored by the forward: S^H of the tile and of its ring is the hard flag
@@ -1705,26 +1864,16 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
         if (BWD && !some) return;
         empty = !some;
     }
-    __syncthreads();
-    if (g.edge_mode == 0 && !empty) {
-        // per halo row, the columns holding S^H = 0 and S^H = 1 (hs <= 48 fits 64 bits)
-        const int lane = tid & 31;
-        for (int row = tid >> 5; row < hs; row += NT / 32) {
-            unsigned long long b0 = 0ull, b1 = 0ull;
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                const int col = half * 32 + lane;
-                const unsigned char v = col < hs ? S.sh[row * hs + col] : (unsigned char)2;
-                b0 |= (unsigned long long)__ballot_sync(0xffffffffu, v == 0) << (32 * half);
-                b1 |= (unsigned long long)__ballot_sync(0xffffffffu, v == 1) << (32 * half);
-            }
-            if (lane == 0) { S.m0[row] = b0; S.m1[row] = b1; }
-        }
+    if (from_ids && !empty) {
+        __syncthreads();
+        halo_rows<TT>(S, hs);
+        __syncthreads();
+        edge_rows<TT>(g, S, rho, wlim, hlim);
         __syncthreads();
     }
 
     if constexpr (MODE == 2) {
-        n_layers = adjoint_queued<K, TT>(g, S, V, M, X0, Y0, rho, wlim, hlim);
+        n_layers = adjoint_queued<K, TT>(g, S, V, M, X0, Y0, wlim, hlim);
     } else if (empty) {
         // background: no layer, RGBA 0 (the loss's gradient 2 (0 - target))
         for (int j = 0; j < PPT; ++j) {
@@ -1765,7 +1914,7 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
             }
             if (!BWD && g.ids) {
                 // hard flags of the stored layers; the front one is S^H itself
-                hardbits = S.sh[(ly + rho) * hs + (lx + rho)] == 1 ? 1u : 0u;
+                hardbits = row_bit(S.hb, lx, ly) ? 1u : 0u;
 #pragma unroll
                 for (int k = 1; k < K; ++k) {
                     const unsigned long long v = kbuf[ks + k];
@@ -1782,11 +1931,11 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
             }
         }
         if constexpr (MODE == 1)
-            n_layers += adjoint_warp<K, TT>(g, S, V, M, X0, Y0, p, rho, in, ids);
+            n_layers += adjoint_warp<K, TT>(g, S, V, M, X0, Y0, p, in, ids);
         else if constexpr (BWD)
-            n_layers += adjoint_pixel<K, TT, EXTRA>(g, S, V, M, X0, Y0, lx, ly, rho, ids, glacc);
+            n_layers += adjoint_pixel<K, TT, EXTRA>(g, S, V, M, X0, Y0, lx, ly, ids, glacc);
         else
-            n_layers += finish_forward<K, TT, EXTRA>(g, S, V, M, X0, Y0, p, rho, in, ids, hardbits, single_chunk, l2acc);
+            n_layers += finish_forward<K, TT, EXTRA>(g, S, V, M, X0, Y0, p, in, ids, hardbits, single_chunk, l2acc);
     }
     if (!BWD && g.l2_loss) {
         // this tile's share of the fused L2 loss: warp sums, one atomic per warp
