@@ -209,28 +209,21 @@ static bool make_plan(const dressi_scene *sc, const dressi_view *views, int n_vi
 
 // ---------------------------------------------------------------------------
 // table upload: the tables travel as kernel parameters (no host-to-device copy,
-// so a whole pass can be captured into a CUDA graph)
+// so a whole pass can be captured into a CUDA graph), those of the vertex transform
+// where they fit
 // ---------------------------------------------------------------------------
-constexpr int BLOB_WORDS = 4000;
-struct Blob {
-    unsigned int n;
-    unsigned int w[BLOB_WORDS];
-};
-
-__global__ void k_upload(const __grid_constant__ Blob b, unsigned int *dst)
+__global__ void k_upload(const __grid_constant__ Tables<TABLE_WORDS> b, unsigned int *dst)
 {
-    for (unsigned int i = threadIdx.x; i < b.n; i += blockDim.x) dst[i] = b.w[i];
+    for (int i = threadIdx.x; i < b.n; i += blockDim.x) dst[i] = b.w[i];
 }
 
-static void upload(const void *src, size_t bytes, void *dst, cudaStream_t s)
+// tables too long for the vertex transform's parameter
+static void upload(const unsigned int *w, size_t words, unsigned int *d, cudaStream_t s)
 {
-    const unsigned int *w = static_cast<const unsigned int *>(src);
-    size_t words = bytes / 4;
-    unsigned int *d = static_cast<unsigned int *>(dst);
-    Blob b;
+    Tables<TABLE_WORDS> b;
     while (words > 0) {
-        const size_t n = std::min<size_t>(words, BLOB_WORDS);
-        b.n = (unsigned int)n;
+        const size_t n = std::min<size_t>(words, TABLE_WORDS);
+        b.n = (int)n;
         std::memcpy(b.w, w, n * 4);
         k_upload<<<1, 256, 0, s>>>(b, d);
         count_launch(1);
@@ -279,6 +272,8 @@ static Globals make_globals(const dressi_scene *sc, const dressi_params *p, cons
     g.adj_cur = reinterpret_cast<int *>(ws + L.adj_cur);
     g.adj = reinterpret_cast<int *>(ws + L.adj);
     g.scan_partial = reinterpret_cast<int *>(ws + L.scan_partial);
+    // the adjacency's scan runs before the normals are written, in their place (16 bytes a vertex)
+    g.scan_partial2 = reinterpret_cast<int *>(ws + L.nrm);
     g.sgrad = reinterpret_cast<float4 *>(ws + L.sgrad);
     g.ngrad = reinterpret_cast<float4 *>(ws + L.ngrad);
     g.status = status;
@@ -299,27 +294,38 @@ static Globals make_globals(const dressi_scene *sc, const dressi_params *p, cons
     return g;
 }
 
-// setup shared by both passes: tables, vertex transform, normals, binning
-static void run_setup(Globals &g, const Plan &P, char *ws, bool need_bins, cudaStream_t s)
+// setup shared by both passes: tables, vertex transform, normals, binning.  clr: arrays that
+// the vertex transform sets besides its own
+static void run_setup(Globals &g, const Plan &P, char *ws, bool need_bins, Clears clr, int n_clr, cudaStream_t s)
 {
     const Layout &L = P.lay;
-    // the view and mesh tables, adjacent in the workspace, in one upload
-    std::vector<unsigned char> tables(L.meshes + sizeof(MeshK) * P.meshes.size(), 0);
-    std::memcpy(tables.data() + L.views, P.views.data(), sizeof(ViewK) * P.views.size());
-    std::memcpy(tables.data() + L.meshes, P.meshes.data(), sizeof(MeshK) * P.meshes.size());
-    upload(tables.data(), tables.size(), ws + L.views, s);
+    const bool normals = g.shade_mode >= 2;
+    auto clear = [&](size_t off, size_t n) {
+        clr.p[n_clr] = reinterpret_cast<int *>(ws + off);
+        clr.n[n_clr] = (int)n;
+        clr.v[n_clr++] = 0;
+    };
+    if (normals) {
+        const size_t nv = (size_t)std::max<long long>(g.n_verts_total, 1);
+        clear(L.adj_off, nv + 1);
+        clear(L.adj_cur, nv);
+    }
+    if (g.persistent) {
+        clear(L.queue, 4);
+        clear(L.lpt_hist, LPT_BINS);
+    }
+    // the view and mesh tables, adjacent in the workspace
+    const size_t words = (L.meshes + sizeof(MeshK) * P.meshes.size()) / 4;
+    std::vector<unsigned> tables(words, 0u);
+    std::memcpy(reinterpret_cast<char *>(tables.data()) + L.views, P.views.data(), sizeof(ViewK) * P.views.size());
+    std::memcpy(reinterpret_cast<char *>(tables.data()) + L.meshes, P.meshes.data(), sizeof(MeshK) * P.meshes.size());
+    const bool fit = words <= (size_t)TABLE_WORDS;
+    if (!fit) upload(tables.data(), words, reinterpret_cast<unsigned *>(ws + L.views), s);
     // the vertex transform also writes the tile -> view table and, before the face table
     // counts into them, clears the tile counters
     g.zero_bins = need_bins ? 1 : 0;
-    launch_vertex(g, (int)P.views.size(), P.max_nv_view, s);
-    launch_face(g, (int)P.views.size(), P.max_nf_view, need_bins, s);
-    if (g.shade_mode >= 2) {
-        const size_t nv = (size_t)std::max<long long>(g.n_verts_total, 1);
-        cudaMemsetAsync(ws + L.adj_off, 0, sizeof(int) * (nv + 1), s);
-        cudaMemsetAsync(ws + L.adj_cur, 0, sizeof(int) * nv, s);
-        launch_normals(g, (int)P.meshes.size(), P.max_nf, P.max_nv, s);
-    }
-    if (need_bins) launch_bin(g, (int)P.views.size(), P.max_nf_view, s);
+    launch_vertex(g, (int)P.views.size(), P.max_nv_view, tables.data(), fit ? (int)words : 0, clr, s);
+    launch_faces(g, (int)P.views.size(), (int)P.meshes.size(), P.max_nf_view, P.max_nf, P.max_nv, need_bins, normals, s);
 }
 
 // Whether a pass without stored layer ids needs the layers behind the front one only inside the
@@ -334,22 +340,24 @@ static bool fronts_only(const dressi_params *p)
 
 // a forward that stores no layer ids leaves every pixel's word (K-th entry, or front layer with
 // E and S^H) in the workspace for a re-rasterizing adjoint; the flag says which, if any
-static void keep_kth(Globals &g, const Plan &P, const dressi_params *p, char *ws, cudaStream_t s)
+static Clears keep_kth(Globals &g, const Plan &P, const dressi_params *p, char *ws)
 {
     const bool keep = g.ids == nullptr;
     g.fronts = keep && fronts_only(p);
     g.kth = keep ? reinterpret_cast<unsigned long long *>(ws + P.lay.kth) : nullptr;
-    cudaMemsetAsync(ws + P.lay.kth_flag, keep ? (g.fronts ? 2 : 1) : 0, sizeof(int), s);
+    Clears clr;
+    clr.p[0] = reinterpret_cast<int *>(ws + P.lay.kth_flag);
+    clr.n[0] = 1;
+    clr.v[0] = keep ? (g.fronts ? KTH_FRONTS : KTH_LAST) : KTH_NONE;
+    return clr;
 }
 
 // the per-tile kernel, persistent (longest face list first when the lists exist) or
 // one CTA per tile
 static void run_tiles(Globals &g, const Plan &P, char *ws, bool bins_built, int pass, cudaStream_t s)
 {
-    if (g.persistent) {
-        cudaMemsetAsync(ws + P.lay.queue, 0, sizeof(int) * 4, s);
+    if (g.persistent) {   // the queue and the histogram are cleared by the setup or the adjoint's fill
         if (bins_built) {
-            cudaMemsetAsync(ws + P.lay.lpt_hist, 0, sizeof(int) * LPT_BINS, s);
             g.tile_order = reinterpret_cast<const int *>(ws + P.lay.tile_order);
             launch_lpt_order(g, s);
             const size_t n = sizeof(int) * (size_t)P.lay.total_tiles;
@@ -477,8 +485,7 @@ int dressi_forward(const dressi_scene *scene, const dressi_view *views, int32_t 
     Globals g = make_globals(scene, params, P, w, n_pix, dev_status);
     g.out = out_rgba;
     g.ids = layer_ids;
-    keep_kth(g, P, params, w, s);
-    run_setup(g, P, w, true, s);
+    run_setup(g, P, w, true, keep_kth(g, P, params, w), 1, s);
     run_tiles(g, P, w, true, 0, s);
     return cudaGetLastError() == cudaSuccess ? DRESSI_OK : DRESSI_ERR_LAUNCH;
 }
@@ -504,8 +511,7 @@ int dressi_forward_l2(const dressi_scene *scene, const dressi_view *views, int32
     g.l2_target = target;
     g.l2_grad = grad_rgba;
     g.l2_loss = loss_accum;
-    keep_kth(g, P, params, w, s);
-    run_setup(g, P, w, true, s);
+    run_setup(g, P, w, true, keep_kth(g, P, params, w), 1, s);
     run_tiles(g, P, w, true, 0, s);
     return cudaGetLastError() == cudaSuccess ? DRESSI_OK : DRESSI_ERR_LAUNCH;
 }
@@ -538,9 +544,12 @@ int dressi_forward_from_layers(const dressi_scene *scene, const dressi_view *vie
     Globals g = make_globals(scene, params, P, w, n_pix, dev_status);
     g.out = out_rgba;
     g.ids_in = layer_ids;
-    cudaMemsetAsync(w + P.lay.kth_flag, 0, sizeof(int), s);   // no K-th keys from this pass
+    Clears clr;   // no pixel words from this pass
+    clr.p[0] = g.kth_flag;
+    clr.n[0] = 1;
+    clr.v[0] = KTH_NONE;
     // vertex records, face table and normals (shading needs them), no binning
-    run_setup(g, P, w, false, s);
+    run_setup(g, P, w, false, clr, 1, s);
     run_tiles(g, P, w, false, 2, s);
     return cudaGetLastError() == cudaSuccess ? DRESSI_OK : DRESSI_ERR_LAUNCH;
 }
@@ -575,26 +584,43 @@ int dressi_backward_ex(const dressi_scene *scene, const dressi_view *views, int3
     g.gmvp = grad_mvp;
     g.glight = grad_light;
     g.gntex = params->shade_mode == 3 ? grad_ntex : nullptr;
-    if (g.gntex && P.n_texels > 0) cudaMemsetAsync(grad_ntex, 0, sizeof(float) * 4 * (size_t)P.n_texels, s);
-    if (grad_mvp) cudaMemsetAsync(grad_mvp, 0, sizeof(float) * 16 * (size_t)n_views, s);
-    if (grad_light) cudaMemsetAsync(grad_light, 0, sizeof(float) * 3 * (size_t)n_views, s);
     const long long nvt = scene->n_verts_total;
-    cudaMemsetAsync(grad_pos, 0, sizeof(float) * 3 * (size_t)nvt, s);
-    if (grad_col) cudaMemsetAsync(grad_col, 0, sizeof(float) * 3 * (size_t)nvt, s);
-    if (grad_tex && P.n_texels > 0) cudaMemsetAsync(grad_tex, 0, sizeof(float) * 4 * (size_t)P.n_texels, s);
-    cudaMemsetAsync(w + P.lay.sgrad, 0, sizeof(float4) * (size_t)std::max<long long>(P.lay.n_vrec, 1), s);
-    if (params->shade_mode >= 2)
-        cudaMemsetAsync(w + P.lay.ngrad, 0, sizeof(float4) * (size_t)std::max<long long>(nvt, 1), s);
     const bool tex_records = g.gtex && P.lay.tg_slots > 0;
     const bool gather = tex_records && params->texgrad_mode == 1;
     const bool inv_uv = tex_records && params->texgrad_mode == 2;
     if (!tex_records) g.texgrad_mode = 0;
-    if (gather) cudaMemsetAsync(w + P.lay.tg_keys, 0xff, sizeof(unsigned) * (size_t)P.lay.tg_slots, s);
-    if (inv_uv) cudaMemsetAsync(w + P.lay.inv_uv, 0xff, sizeof(int) * (size_t)P.n_texels, s);
-    g.fronts = !layer_ids && fronts_only(params);
+    // the outputs and accumulators, in one launch (a memset each costs a small call more than
+    // its bytes); past 16 MB a range goes by cudaMemsetAsync, which alone reaches the full rate
+    Fills f;
+    int nf = 0;
+    auto fill = [&](void *p, long long words, unsigned v = 0u) {
+        if (!p || words <= 0) return;
+        if (words >= (4 << 20)) {
+            cudaMemsetAsync(p, (int)(v & 0xff), sizeof(int) * (size_t)words, s);
+            return;
+        }
+        f.p[nf] = static_cast<unsigned *>(p);
+        f.n[nf] = words;
+        f.v[nf++] = v;
+    };
+    if (g.gntex) fill(grad_ntex, 4 * P.n_texels);
+    fill(grad_mvp, 16LL * n_views);
+    fill(grad_light, 3LL * n_views);
+    fill(grad_pos, 3 * nvt);
+    fill(grad_col, 3 * nvt);
+    fill(grad_tex, 4 * P.n_texels);
+    fill(w + P.lay.sgrad, 4 * P.lay.n_vrec);
+    if (params->shade_mode >= 2) fill(w + P.lay.ngrad, 4 * nvt);
+    if (gather) fill(w + P.lay.tg_keys, P.lay.tg_slots, 0xffffffffu);
+    if (inv_uv) fill(w + P.lay.inv_uv, P.n_texels, 0xffffffffu);
+    if (g.persistent) {
+        fill(w + P.lay.queue, 4);
+        fill(w + P.lay.lpt_hist, LPT_BINS);
+    }
+    launch_fill(f, s);
     // re-rasterizing after a forward on this workspace: its pixels' words, if it kept them
     if (params->reuse_setup && !layer_ids) g.kth = reinterpret_cast<unsigned long long *>(w + P.lay.kth);
-    if (!params->reuse_setup) run_setup(g, P, w, layer_ids == nullptr, s);
+    if (!params->reuse_setup) run_setup(g, P, w, layer_ids == nullptr, Clears(), 0, s);
     run_tiles(g, P, w, layer_ids == nullptr, 1, s);
     if (gather)
         launch_tex_gather(g, P.lay.tg_slots, P.n_texels, (int)P.meshes.size(), P.max_texels, w + P.lay.tg_scratch,

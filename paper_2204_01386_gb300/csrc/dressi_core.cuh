@@ -32,6 +32,12 @@ constexpr float EDGE_TIE_PX = 1e-3f;
 constexpr int FLAG_RANGE = 1 << 8;
 constexpr int FLAG_ODD = 1 << 9;    // the record's corner order is an odd permutation of the face's
 
+// a pixel's word from a forward without layer ids: nothing, the K-th (key, id) of every pixel, or
+// E and S^H with the K-th (key, id) where E = 1, else the front one (keys are below 2: the two top
+// bits are free)
+constexpr int KTH_NONE = 0, KTH_LAST = 0x01010101, KTH_FRONTS = 0x02020202;
+constexpr unsigned long long KTH_SH = 1ull << 63, KTH_E = 1ull << 62, KTH_BITS = KTH_E - 1;
+
 // ---------------------------------------------------------------------------
 // tables uploaded into the workspace
 // ---------------------------------------------------------------------------
@@ -128,7 +134,7 @@ struct Globals {
     int *adj_off;         // [n_verts_total + 1] vertex -> incident faces (CSR offsets)
     int *adj_cur;         // [n_verts_total] fill cursors
     int *adj;             // [3 * faces] incident face ids (mesh-local)
-    int *scan_partial;    // scratch of the device-wide scan
+    int *scan_partial, *scan_partial2;   // scratch of the device-wide scans (tile counts, adjacency)
     int *status;
     // scheduling of the per-tile kernel
     int persistent;       // 1: persistent CTAs pull tiles from *queue

@@ -6,15 +6,43 @@
 namespace dressi {
 struct Globals;
 void count_launch(int n);
-void launch_vertex(const Globals &g, int n_views, int max_nv, cudaStream_t s);
-void launch_normals(const Globals &g, int n_meshes, int max_nf, int max_nv, cudaStream_t s);
-void launch_face(const Globals &g, int n_views, int max_nf, bool count, cudaStream_t s);
-void launch_bin(const Globals &g, int n_views, int max_nf, cudaStream_t s);
+// words of view and mesh tables that one launch can carry as a parameter
+constexpr int TABLE_WORDS = 4000;
+template <int N>
+struct Tables {
+    int n;
+    alignas(8) unsigned w[N ? N : 2];
+};
+// small arrays of 32-bit words set by the vertex transform for the kernels after it
+struct Clears {
+    static constexpr int MAX = 5;
+    int *p[MAX] = {};
+    int n[MAX] = {}, v[MAX] = {};
+};
+// ranges of 32-bit words filled by one launch
+struct Fills {
+    static constexpr int MAX = 12;
+    unsigned *p[MAX] = {};
+    long long n[MAX] = {};
+    unsigned v[MAX] = {};
+};
+// exclusive prefix of n_in non-negative ints at src (0 past them) into n_out at dst
+struct ScanJob {
+    const int *src;
+    int *dst;
+    int n_in, n_out;
+    int *partial;   // scan_partials_needed(n_out) ints; receives the total behind the parts
+};
+void launch_vertex(const Globals &g, int n_views, int max_nv, const unsigned *tables, int words, const Clears &clr,
+                   cudaStream_t s);
+void launch_faces(const Globals &g, int n_views, int n_meshes, int max_nf_view, int max_nf, int max_nv, bool lists,
+                  bool normals, cudaStream_t s);
+void launch_fill(const Fills &f, cudaStream_t s);
 void launch_tile(const Globals &g, bool backward, cudaStream_t s);
 void launch_tile_shade(const Globals &g, cudaStream_t s);
 void launch_lpt_order(const Globals &g, cudaStream_t s);
 size_t texgather_scratch_bytes(long long slots, long long n_texels, size_t align);
-void launch_scan_inplace(int *a, int n, int *partial, cudaStream_t s);
+void launch_scans(const ScanJob *jobs, int n, cudaStream_t s);   // one or two, in the same launches
 int scan_partials_needed(long long n);
 void launch_inv_uv_apply(const Globals &g, long long n_texels, cudaStream_t s);
 void launch_tex_gather(const Globals &g, long long slots, long long n_texels, int n_meshes, int max_texels,

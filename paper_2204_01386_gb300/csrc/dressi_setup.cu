@@ -4,6 +4,9 @@
 #include "dressi_core.cuh"
 #include "dressi_launch.h"
 
+#include <algorithm>
+#include <cstring>
+
 namespace dressi {
 
 // ---------------------------------------------------------------------------
@@ -66,10 +69,29 @@ __device__ __forceinline__ DF df_recip(DF w)
     return quick_two_sum(r, __fmul_rn(e, r));
 }
 
-__global__ void k_vertex(Globals g)
+// The first kernel of a pass also uploads the tables (they travel as its parameter: no host-to-
+// device copy, so a pass can be captured into a CUDA graph) and clears the counters of the
+// kernels after it: a launch of its own costs a small call as much as its work (a 320-face,
+// 64 x 64 step is all launches).  TABLES: words of tables in the parameter (0: already uploaded).
+template <int TABLES>
+__global__ void k_vertex(Globals g, const __grid_constant__ Tables<TABLES> tab, Clears clr)
 {
-    const ViewK &V = g.views[blockIdx.y];
-    const MeshK &M = g.meshes[V.mesh];
+    const ViewK *views = g.views;
+    const MeshK *meshes = g.meshes;
+    const int nthreads = gridDim.x * gridDim.y * blockDim.x;
+    const int gtid = (blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x;
+    if (TABLES) {
+        unsigned *dst = reinterpret_cast<unsigned *>(const_cast<ViewK *>(g.views));
+        for (int i = gtid; i < tab.n; i += nthreads) dst[i] = tab.w[i];
+        // this kernel's own reads come from the parameter
+        views = reinterpret_cast<const ViewK *>(tab.w);
+        meshes = reinterpret_cast<const MeshK *>(tab.w + (reinterpret_cast<const unsigned *>(g.meshes) - dst));
+    }
+#pragma unroll
+    for (int q = 0; q < Clears::MAX; ++q)
+        for (int i = gtid; i < clr.n[q]; i += nthreads) clr.p[q][i] = clr.v[q];
+    const ViewK &V = views[blockIdx.y];
+    const MeshK &M = meshes[V.mesh];
     VRec *out = g.vrec + V.vrec_off;
     const long long nvt = g.n_verts_total;
     bool bad = false;
@@ -129,10 +151,12 @@ __device__ __forceinline__ bool face_vertices(const Globals &g, const MeshK &M, 
     return (unsigned)v[0] < (unsigned)M.nV && (unsigned)v[1] < (unsigned)M.nV && (unsigned)v[2] < (unsigned)M.nV;
 }
 
+// the vertex -> face adjacency of mesh m: PASS 0 counts, PASS 1 fills.  Runs in the extra grid rows
+// (one per mesh) of the face table and list fill kernels, which it does not depend on.
 template <int PASS>
-__global__ void k_adjacency(Globals g)
+__device__ __forceinline__ void adjacency(const Globals &g, int m)
 {
-    const MeshK &M = g.meshes[blockIdx.y];
+    const MeshK &M = g.meshes[m];
     for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < M.nF; f += gridDim.x * blockDim.x) {
         int v[3];
         if (!face_vertices(g, M, f, v)) continue;
@@ -143,6 +167,12 @@ __global__ void k_adjacency(Globals g)
             else g.adj[g.adj_off[gv] + atomicAdd(g.adj_cur + gv, 1)] = f;
         }
     }
+}
+
+template <int PASS>
+__global__ void k_adjacency(Globals g)
+{
+    adjacency<PASS>(g, blockIdx.y);
 }
 
 __global__ void k_normal_csr(Globals g)
@@ -266,6 +296,10 @@ __global__ void __launch_bounds__(256) k_face(Globals g)
     // each warp's 32 records (7 float4 each) go through shared memory so that the warp
     // writes its 3,584 contiguous bytes with full-line stores
     __shared__ float4 stage[256 / 32][32 * 7];
+    if (blockIdx.y >= g.n_views) {
+        adjacency<0>(g, blockIdx.y - g.n_views);
+        return;
+    }
     const ViewK V = g.views[blockIdx.y];   // copies: the fields stay in registers across the stores
     const MeshK M = g.meshes[V.mesh];
     const VRec *vr = g.vrec + V.vrec_off;
@@ -317,6 +351,10 @@ __global__ void __launch_bounds__(256) k_face(Globals g)
 // each face's tile rect comes packed from the face table kernel
 __global__ void k_bin(Globals g)
 {
+    if (blockIdx.y >= g.n_views) {
+        adjacency<1>(g, blockIdx.y - g.n_views);
+        return;
+    }
     const ViewK V = g.views[blockIdx.y];   // copies: the fields stay in registers across the stores
     const MeshK M = g.meshes[V.mesh];
     for (int f0 = blockIdx.x * blockDim.x; f0 < M.nF; f0 += gridDim.x * blockDim.x) {
@@ -383,11 +421,45 @@ __global__ void k_lpt_scatter(Globals g)
         order[atomicAdd(g.lpt_hist + lpt_bin(g.tile_count[t]), 1)] = t;
 }
 
+// the same order in one block (a launch instead of three): the histogram in shared memory
+__global__ void __launch_bounds__(LPT_BINS) k_lpt_single(Globals g)
+{
+    __shared__ int hist[LPT_BINS];
+    __shared__ int warp_sums[LPT_BINS / 32];
+    int *order = const_cast<int *>(g.tile_order);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    hist[tid] = 0;
+    __syncthreads();
+    for (int t = tid; t < g.total_tiles; t += LPT_BINS) atomicAdd(hist + lpt_bin(g.tile_count[t]), 1);
+    __syncthreads();
+    const int v = hist[tid];
+    int x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) warp_sums[warp] = x;
+    __syncthreads();
+    int before = 0;
+    for (int w = 0; w < warp; ++w) before += warp_sums[w];
+    hist[tid] = before + x - v;
+    __syncthreads();
+    for (int t = tid; t < g.total_tiles; t += LPT_BINS) order[atomicAdd(hist + lpt_bin(g.tile_count[t]), 1)] = t;
+}
+
 // ---------------------------------------------------------------------------
 // adjoint, per (view, vertex): (dX, dY, d(1/w)) -> clip -> object space
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ void normal_bwd(const Globals &g, int m);
+
+// grid rows: one per view, then (normals) one per mesh for the normals' share of the positions
 __global__ void k_vertex_bwd(Globals g)
 {
+    if (blockIdx.y >= g.n_views) {
+        normal_bwd(g, blockIdx.y - g.n_views);
+        return;
+    }
     const ViewK &V = g.views[blockIdx.y];
     const MeshK &M = g.meshes[V.mesh];
     const float4 *sg = g.sgrad + V.vrec_off;
@@ -441,9 +513,9 @@ __global__ void k_vertex_bwd(Globals g)
 
 // normals -> positions: dm_v = (dn_v - n_v (n_v . dn_v)) / |m_v|; per face
 // da = sum of dm over its corners; a = u x w gives du = w x da, dw = da x u
-__global__ void k_normal_bwd(Globals g)
+__device__ __forceinline__ void normal_bwd(const Globals &g, int m)
 {
-    const MeshK &M = g.meshes[blockIdx.y];
+    const MeshK &M = g.meshes[m];
     const long long nvt = g.n_verts_total;
     for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < M.nF; f += gridDim.x * blockDim.x) {
         const int *fv = g.faces + 3 * (M.face_off + f);
@@ -479,6 +551,27 @@ __global__ void k_normal_bwd(Globals g)
             atomicAdd(g.gpos + c * nvt + M.vert_off + v[2], gw[c]);
             atomicAdd(g.gpos + c * nvt + M.vert_off + v[0], -(gu[c] + gw[c]));
         }
+    }
+}
+
+__global__ void k_normal_bwd(Globals g) { normal_bwd(g, blockIdx.y); }
+
+// fills up to Fills::MAX ranges of 32-bit words in one launch (the adjoint's outputs and accumulators)
+__global__ void __launch_bounds__(256) k_fill(Fills f)
+{
+    const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+#pragma unroll
+    for (int q = 0; q < Fills::MAX; ++q) {
+        const unsigned v = f.v[q];
+        unsigned *p = f.p[q];
+        const long long n = f.n[q];
+        long long done = 0;
+        if ((reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+            const long long n4 = n >> 2;
+            for (long long i = t0; i < n4; i += stride) reinterpret_cast<uint4 *>(p)[i] = make_uint4(v, v, v, v);
+            done = n4 << 2;
+        }
+        for (long long i = done + t0; i < n; i += stride) p[i] = v;
     }
 }
 
@@ -524,46 +617,89 @@ static int grid_x(long long n, int block, int cap)
     return (int)b;
 }
 
-void launch_vertex(const Globals &g, int n_views, int max_nv, cudaStream_t s)
+constexpr int MAX_GRID_Y = 65535;
+
+template <int TABLES>
+static void launch_vertex_t(const Globals &g, dim3 grid, const unsigned *tables, int words, const Clears &clr,
+                            cudaStream_t s)
+{
+    Tables<TABLES> t;
+    t.n = words;
+    if (TABLES) std::memcpy(t.w, tables, sizeof(unsigned) * words);
+    k_vertex<TABLES><<<grid, 256, 0, s>>>(g, t, clr);
+    count_launch(1);
+}
+
+// the vertex transform; uploads the tables (words of them at tables) unless they are already there
+// (words 0), from a parameter as small as they allow: the launch copies all of it
+void launch_vertex(const Globals &g, int n_views, int max_nv, const unsigned *tables, int words, const Clears &clr,
+                   cudaStream_t s)
 {
     dim3 grid(grid_x(max_nv, 256, 1024), n_views);
-    k_vertex<<<grid, 256, 0, s>>>(g);
-    count_launch(1);
+    if (words == 0) launch_vertex_t<0>(g, grid, tables, words, clr, s);
+    else if (words <= 128) launch_vertex_t<128>(g, grid, tables, words, clr, s);
+    else launch_vertex_t<TABLE_WORDS>(g, grid, tables, words, clr, s);
 }
 
-void launch_normals(const Globals &g, int n_meshes, int max_nf, int max_nv, cudaStream_t s)
+// The per-face setup after the vertex transform: face table; with lists, the tile counts, their
+// prefix and the lists; with normals, the vertex -> face adjacency (counted beside the face
+// table, filled beside the lists) and the normals.  adj_off and adj_cur are cleared.
+void launch_faces(const Globals &g, int n_views, int n_meshes, int max_nf_view, int max_nf, int max_nv, bool lists,
+                  bool normals, cudaStream_t s)
 {
-    // adj_off and adj_cur are zeroed by the caller
-    dim3 gf(grid_x(max_nf, 256, 2048), n_meshes), gv(grid_x(max_nv, 256, 2048), n_meshes);
-    k_adjacency<0><<<gf, 256, 0, s>>>(g);
-    launch_scan_inplace(g.adj_off, (int)(g.n_verts_total + 1), g.scan_partial, s);
-    k_adjacency<1><<<gf, 256, 0, s>>>(g);
-    k_normal_csr<<<gv, 256, 0, s>>>(g);
-    count_launch(3);
-}
-
-void launch_face(const Globals &g, int n_views, int max_nf, bool count, cudaStream_t s)
-{
-    dim3 grid(grid_x(max_nf, 256, 2048), n_views);
-    if (count) k_face<true><<<grid, 256, 0, s>>>(g);
+    // (a launch holds 65,535 grid rows; views and meshes may be more together)
+    const bool merge = normals && n_views + n_meshes <= MAX_GRID_Y;
+    const dim3 grid(grid_x(std::max(max_nf_view, merge ? max_nf : 0), 256, 2048), n_views + (merge ? n_meshes : 0));
+    const dim3 grid_m(grid_x(max_nf, 256, 2048), n_meshes);
+    if (lists) k_face<true><<<grid, 256, 0, s>>>(g);
     else k_face<false><<<grid, 256, 0, s>>>(g);
     count_launch(1);
+    if (normals && !merge) {
+        k_adjacency<0><<<grid_m, 256, 0, s>>>(g);
+        count_launch(1);
+    }
+    // exclusive prefixes: tile_off[n] = total list entries
+    ScanJob jobs[2];
+    int nj = 0;
+    if (lists) jobs[nj++] = {g.tile_count, g.tile_off, g.total_tiles, g.total_tiles + 1, g.scan_partial};
+    if (normals) {
+        const int n = (int)(g.n_verts_total + 1);
+        jobs[nj++] = {g.adj_off, g.adj_off, n, n, g.scan_partial2};
+    }
+    if (nj) launch_scans(jobs, nj, s);
+    if (lists) {
+        k_bin<<<grid, 256, 0, s>>>(g);
+        count_launch(1);
+    }
+    if (normals && !(lists && merge)) {
+        k_adjacency<1><<<grid_m, 256, 0, s>>>(g);
+        count_launch(1);
+    }
+    if (normals) {
+        k_normal_csr<<<dim3(grid_x(max_nv, 256, 2048), n_meshes), 256, 0, s>>>(g);
+        count_launch(1);
+    }
 }
 
-// after launch_face(count = true): the counts' prefix and the lists
-void launch_bin(const Globals &g, int n_views, int max_nf, cudaStream_t s)
+void launch_fill(const Fills &f, cudaStream_t s)
 {
-    dim3 grid(grid_x(max_nf, 256, 2048), n_views);
-    // exclusive prefix of the tile counts: tile_off[n] = total list entries
-    cudaMemcpyAsync(g.tile_off, g.tile_count, sizeof(int) * (size_t)g.total_tiles, cudaMemcpyDeviceToDevice, s);
-    cudaMemsetAsync(g.tile_off + g.total_tiles, 0, sizeof(int), s);
-    launch_scan_inplace(g.tile_off, g.total_tiles + 1, g.scan_partial, s);
-    k_bin<<<grid, 256, 0, s>>>(g);
+    long long words = 0;
+    for (int q = 0; q < Fills::MAX; ++q) words = std::max(words, f.n[q]);
+    if (words == 0) return;
+    k_fill<<<grid_x(words / 4 + 1, 256, 152 * 16), 256, 0, s>>>(f);
     count_launch(1);
 }
+
+// one block up to LPT_SINGLE tiles: 16 rounds of its threads, against three launches of 2 to 7 us
+constexpr int LPT_SINGLE = 16 * LPT_BINS;
 
 void launch_lpt_order(const Globals &g, cudaStream_t s)
 {
+    if (g.total_tiles <= LPT_SINGLE) {
+        k_lpt_single<<<1, LPT_BINS, 0, s>>>(g);
+        count_launch(1);
+        return;
+    }
     const int grid = grid_x(g.total_tiles, 256, 1024);
     k_lpt_hist<<<grid, 256, 0, s>>>(g);
     k_lpt_scan<<<1, LPT_BINS, 0, s>>>(g);
@@ -574,12 +710,12 @@ void launch_lpt_order(const Globals &g, cudaStream_t s)
 void launch_vertex_bwd(const Globals &g, int n_views, int max_nv, int n_meshes, int max_nf, bool normals,
                        cudaStream_t s)
 {
-    dim3 grid(grid_x(max_nv, 256, 1024), n_views);
+    const bool merge = normals && n_views + n_meshes <= MAX_GRID_Y;
+    const dim3 grid(grid_x(std::max(max_nv, merge ? max_nf : 0), 256, 2048), n_views + (merge ? n_meshes : 0));
     k_vertex_bwd<<<grid, 256, 0, s>>>(g);
     count_launch(1);
-    if (normals) {
-        dim3 g2(grid_x(max_nf, 256, 2048), n_meshes);
-        k_normal_bwd<<<g2, 256, 0, s>>>(g);
+    if (normals && !merge) {
+        k_normal_bwd<<<dim3(grid_x(max_nf, 256, 2048), n_meshes), 256, 0, s>>>(g);
         count_launch(1);
     }
 }

@@ -26,7 +26,8 @@ constexpr int RS_ITEMS = 16;                      // items per thread per block
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;    // items per block
 constexpr int RS_BINS = 256;
 
-// --- device-wide exclusive scan of n non-negative ints (in place), three kernels ---
+// --- device-wide exclusive scans of non-negative ints: three kernels, or one block each ---
+// (grid rows: one per job, so that independent scans share their launches)
 // Sums saturate at INT_MAX (for non-negative terms min(a + b, INT_MAX) is still
 // associative), so a total past 2^31 - 1 reads as INT_MAX instead of wrapping.
 constexpr int SC_THREADS = 1024;
@@ -67,56 +68,100 @@ __device__ __forceinline__ int block_excl_scan(int v, int *warp_tot, int &total)
     return r;
 }
 
-__global__ void __launch_bounds__(SC_THREADS) k_scan_reduce(const int *a, int n, int *partial)
+struct ScanJobs {
+    ScanJob j[2];
+};
+
+__device__ __forceinline__ int scan_load(const ScanJob &J, int i) { return i < J.n_in ? J.src[i] : 0; }
+
+__global__ void __launch_bounds__(SC_THREADS) k_scan_reduce(ScanJobs jobs)
 {
     __shared__ int wt[32];
+    const ScanJob &J = jobs.j[blockIdx.y];
+    if (blockIdx.x * SC_TILE >= J.n_out) return;
     const int base = blockIdx.x * SC_TILE + threadIdx.x * SC_ITEMS;
     int s = 0;
 #pragma unroll
-    for (int j = 0; j < SC_ITEMS; ++j) s = sat_add(s, (base + j < n) ? a[base + j] : 0);
+    for (int j = 0; j < SC_ITEMS; ++j) s = sat_add(s, scan_load(J, base + j));
     int total;
     block_excl_scan(s, wt, total);
-    if (threadIdx.x == 0) partial[blockIdx.x] = total;
+    if (threadIdx.x == 0) J.partial[blockIdx.x] = total;
 }
 
-// exclusive scan of the partials in one block (nparts <= SC_TILE); partial[nparts] = total
-__global__ void __launch_bounds__(SC_THREADS) k_scan_partials(int *partial, int nparts)
+// exclusive scan of the partials in one block, SC_TILE at a time with a running carry;
+// partial[nparts] = total
+__global__ void __launch_bounds__(SC_THREADS) k_scan_partials(ScanJobs jobs)
 {
     __shared__ int wt[32];
-    const int base = threadIdx.x * SC_ITEMS;
-    int v[SC_ITEMS], s = 0;
+    const ScanJob &J = jobs.j[blockIdx.y];
+    const int nparts = (J.n_out + SC_TILE - 1) / SC_TILE;
+    int carry = 0;
+    for (int c0 = 0; c0 < nparts; c0 += SC_TILE) {
+        const int base = c0 + threadIdx.x * SC_ITEMS;
+        int v[SC_ITEMS], s = 0;
 #pragma unroll
-    for (int j = 0; j < SC_ITEMS; ++j) {
-        v[j] = (base + j < nparts) ? partial[base + j] : 0;
-        s = sat_add(s, v[j]);
-    }
-    int total;
-    int run = block_excl_scan(s, wt, total);
+        for (int j = 0; j < SC_ITEMS; ++j) {
+            v[j] = (base + j < nparts) ? J.partial[base + j] : 0;
+            s = sat_add(s, v[j]);
+        }
+        int total;
+        int run = sat_add(block_excl_scan(s, wt, total), carry);
 #pragma unroll
-    for (int j = 0; j < SC_ITEMS; ++j) {
-        if (base + j < nparts) partial[base + j] = run;
-        run = sat_add(run, v[j]);
+        for (int j = 0; j < SC_ITEMS; ++j) {
+            if (base + j < nparts) J.partial[base + j] = run;
+            run = sat_add(run, v[j]);
+        }
+        carry = sat_add(carry, total);
     }
-    if (threadIdx.x == 0) partial[nparts] = total;
+    if (threadIdx.x == 0) J.partial[nparts] = carry;
 }
 
-__global__ void __launch_bounds__(SC_THREADS) k_scan_down(int *a, int n, const int *partial)
+__global__ void __launch_bounds__(SC_THREADS) k_scan_down(ScanJobs jobs)
 {
     __shared__ int wt[32];
+    const ScanJob &J = jobs.j[blockIdx.y];
+    if (blockIdx.x * SC_TILE >= J.n_out) return;
     const int base = blockIdx.x * SC_TILE + threadIdx.x * SC_ITEMS;
     int v[SC_ITEMS], s = 0;
 #pragma unroll
     for (int j = 0; j < SC_ITEMS; ++j) {
-        v[j] = (base + j < n) ? a[base + j] : 0;
+        v[j] = scan_load(J, base + j);
         s = sat_add(s, v[j]);
     }
     int total;
-    int run = sat_add(block_excl_scan(s, wt, total), partial[blockIdx.x]);
+    int run = sat_add(block_excl_scan(s, wt, total), J.partial[blockIdx.x]);
 #pragma unroll
     for (int j = 0; j < SC_ITEMS; ++j) {
-        if (base + j < n) a[base + j] = run;
+        if (base + j < J.n_out) J.dst[base + j] = run;
         run = sat_add(run, v[j]);
     }
+}
+
+// the whole scan in one block, SC_TILE items at a time with a running carry (short arrays:
+// one launch instead of three); the total goes where the three-kernel scan leaves it
+__global__ void __launch_bounds__(SC_THREADS) k_scan_single(ScanJobs jobs)
+{
+    __shared__ int wt[32];
+    const ScanJob &J = jobs.j[blockIdx.x];
+    int carry = 0;
+    for (int c0 = 0; c0 < J.n_out; c0 += SC_TILE) {
+        const int base = c0 + threadIdx.x * SC_ITEMS;
+        int v[SC_ITEMS], s = 0;
+#pragma unroll
+        for (int j = 0; j < SC_ITEMS; ++j) {
+            v[j] = scan_load(J, base + j);
+            s = sat_add(s, v[j]);
+        }
+        int total;
+        int run = sat_add(block_excl_scan(s, wt, total), carry);
+#pragma unroll
+        for (int j = 0; j < SC_ITEMS; ++j) {
+            if (base + j < J.n_out) J.dst[base + j] = run;
+            run = sat_add(run, v[j]);
+        }
+        carry = sat_add(carry, total);
+    }
+    if (threadIdx.x == 0) J.partial[(J.n_out + SC_TILE - 1) / SC_TILE] = carry;
 }
 
 // --- stable LSD radix sort pass ---------------------------------------------------
@@ -254,44 +299,27 @@ static int grid_of(long long n, int block, int cap)
     return (int)b;
 }
 
-// the whole scan in one block, SC_TILE items at a time with a running carry (short arrays:
-// one launch instead of three); the total goes where the three-kernel scan leaves it
-__global__ void __launch_bounds__(SC_THREADS) k_scan_single(int *a, int n, int *total_out)
-{
-    __shared__ int wt[32];
-    int carry = 0;
-    for (int c0 = 0; c0 < n; c0 += SC_TILE) {
-        const int base = c0 + threadIdx.x * SC_ITEMS;
-        int v[SC_ITEMS], s = 0;
-#pragma unroll
-        for (int j = 0; j < SC_ITEMS; ++j) {
-            v[j] = (base + j < n) ? a[base + j] : 0;
-            s = sat_add(s, v[j]);
-        }
-        int total;
-        int run = sat_add(block_excl_scan(s, wt, total), carry);
-#pragma unroll
-        for (int j = 0; j < SC_ITEMS; ++j) {
-            if (base + j < n) a[base + j] = run;
-            run = sat_add(run, v[j]);
-        }
-        carry = sat_add(carry, total);
-    }
-    if (threadIdx.x == 0) *total_out = carry;
-}
+// one or two scans in the same launches: one block each up to SC_SINGLE items, where the serial
+// rounds of 4096 items (about 1.4 us each) cost less than two more launches
+constexpr int SC_SINGLE = 6 * SC_TILE;
 
-void launch_scan_inplace(int *a, int n, int *partial, cudaStream_t s)
+void launch_scans(const ScanJob *jobs, int n, cudaStream_t s)
 {
-    if (n <= 2 * SC_TILE) {
-        // partial[number of SC_TILE parts] = total, as k_scan_partials leaves it
-        k_scan_single<<<1, SC_THREADS, 0, s>>>(a, n, partial + (n + SC_TILE - 1) / SC_TILE);
+    ScanJobs J;
+    int longest = 0;
+    for (int i = 0; i < n; ++i) {
+        J.j[i] = jobs[i];
+        longest = std::max(longest, jobs[i].n_out);
+    }
+    if (longest <= SC_SINGLE) {
+        k_scan_single<<<n, SC_THREADS, 0, s>>>(J);
         count_launch(1);
         return;
     }
-    const int nparts = (n + SC_TILE - 1) / SC_TILE;
-    k_scan_reduce<<<nparts, SC_THREADS, 0, s>>>(a, n, partial);
-    k_scan_partials<<<1, SC_THREADS, 0, s>>>(partial, nparts);
-    k_scan_down<<<nparts, SC_THREADS, 0, s>>>(a, n, partial);
+    const dim3 grid((longest + SC_TILE - 1) / SC_TILE, n);
+    k_scan_reduce<<<grid, SC_THREADS, 0, s>>>(J);
+    k_scan_partials<<<dim3(1, n), SC_THREADS, 0, s>>>(J);
+    k_scan_down<<<grid, SC_THREADS, 0, s>>>(J);
     count_launch(3);
 }
 
@@ -336,7 +364,8 @@ void launch_tex_gather(const Globals &g, long long slots, long long n_texels, in
     for (int pass = 0; pass < passes; ++pass) {
         const int shift = 8 * pass;
         k_rs_hist<<<(int)nblocks, RS_THREADS, 0, s>>>(kin, cnt, slots, shift, hist, (int)nblocks);
-        launch_scan_inplace(hist, (int)hist_n, partial, s);
+        const ScanJob job = {hist, hist, (int)hist_n, (int)hist_n, partial};
+        launch_scans(&job, 1, s);
         if (pass == 0) {
             // the number of kept (valid) records is the scan's total
             cudaMemcpyAsync(count, partial + nparts, sizeof(int), cudaMemcpyDeviceToDevice, s);

@@ -51,11 +51,6 @@ constexpr int QN = NT / 32 * WQ;       // the CTA's warp queues
 constexpr int NBLK = 1024;             // pair blocks of 32 with a table entry (32,768 items)
 // the raster's passes (tile_body)
 constexpr int ST_FRONT = 0, ST_LAYERS = 1, ST_DONE = 2;
-// a pixel's word from a forward without layer ids: nothing, the K-th (key, id) of every pixel, or
-// E and S^H with the K-th (key, id) where E = 1, else the front one (keys are below 2: the two top
-// bits are free)
-constexpr int KTH_NONE = 0, KTH_LAST = 0x01010101, KTH_FRONTS = 0x02020202;
-constexpr unsigned long long KTH_SH = 1ull << 63, KTH_E = 1ull << 62, KTH_BITS = KTH_E - 1;
 
 // conservative tile-local data of a staged face: edge equations in pixels relative to
 // the tile origin (FP32, a few 1e-6 px of error) and the smallest corner depth.  12 words:
