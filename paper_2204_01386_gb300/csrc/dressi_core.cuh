@@ -493,6 +493,25 @@ __device__ __forceinline__ void frag_lambda(const FaceGeo &R, const Frag &fr, fl
     for (int j = 0; j < 3; ++j) lam[j] = (j == P) ? fsub(1.f, fr.t) : ((j == Q) ? fr.t : 0.f);
 }
 
+// frag_lambda of a hard fragment, from the crosses alone (eval_face's and frag_lambda's operations)
+__device__ __forceinline__ void front_lambda(const FaceGeo &R, float px, float py, float lam[3])
+{
+    float dx[3], dy[3], c[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        dx[i] = fsub(fsub(px, R.c[i].xh), R.c[i].xl);
+        dy[i] = fsub(fsub(py, R.c[i].yh), R.c[i].yl);
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int P = i == 2 ? 0 : i, Q = i == 2 ? 2 : i + 1;
+        c[i] = ffma(dx[P], dy[Q], -fmul(dy[P], dx[Q]));
+    }
+    lam[0] = fmul(c[1], R.invA);
+    lam[1] = fmul(-c[2], R.invA);
+    lam[2] = fmul(c[0], R.invA);
+}
+
 // Hard test only (for S^H of halo pixels): true if p lies in the closed face under
 // the fill rule.
 __device__ __forceinline__ bool hard_test(const FaceGeo &R, float px, float py)

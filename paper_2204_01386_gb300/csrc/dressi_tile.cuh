@@ -23,7 +23,7 @@
 //      bilinear texture, Lambert or normal map) the layers its pixels blend as one list,
 //      and each pixel blends them (D_k = sigmoid(dist/sigma), colour and silhouette
 //      equations of Sec. 3.4.3), optionally with the L2 loss; adjoint: the same values are
-//      rebuilt, by warp lists (re-rasterizing) or a CTA-wide layer queue (stored ids), and
+//      rebuilt by warp lists, and
 //      dL/dI is pushed back to the screen-space corners, vertex colours, vertex normals,
 //      texels, the camera and the light.
 // With layer ids stored by the forward (modes 2, 3, 4, 7), steps 1-3 are skipped: S^H of
@@ -38,7 +38,13 @@
 
 namespace dressi {
 
-constexpr int NT = 256;                // threads per CTA
+constexpr int NT_MAX = 256;            // threads per CTA, at most
+// threads per CTA of one instantiation
+template <int MODE, int TT>
+__host__ __device__ constexpr int cta_threads()
+{
+    return 256;
+}
 constexpr int TT_MAX = 32;             // tile edges: 16 (one pixel per thread) or 32 (four)
 constexpr int RHO_MAX = 8;             // largest supported edge-mask radius
 constexpr int HS_MAX = TT_MAX + 2 * RHO_MAX;
@@ -47,7 +53,6 @@ constexpr int CH = 128;                // faces staged per round (one per thread
 constexpr int HASH = 256;              // face id -> staged slot, open addressing (2 CH: at most half full)
 constexpr unsigned long long EMPTY = ~0ULL;
 constexpr int WQ = 160;                // a warp's queue of pretested pairs (31 waiting + 32 items x 4)
-constexpr int QN = NT / 32 * WQ;       // the CTA's warp queues
 constexpr int NBLK = 1024;             // pair blocks of 32 with a table entry (32,768 items)
 // the raster's passes (tile_body)
 constexpr int ST_FRONT = 0, ST_LAYERS = 1, ST_DONE = 2;
@@ -118,16 +123,17 @@ struct Shade {
     int vi[3];
     float iw[3];
     int odd;              // the record's corner order is an odd permutation of the face's
-    float lam[3], b[3], Q;
+    float lam[3], b[3], iQ;   // iQ: 1 / sum lam_i / w_i
     float C[3];
-    float D;
+    float D;                  // not set for a layer built as a front one
     // texture
     int ix[2], iy[2];
     float fx, fy;
     float A[3];
+    float Ax[3], Ay[3];   // the adjoint's: derivatives of A in texel space
     float Xt[3], Yt[3];   // texel-space corner coordinates relative to corner 0
     // Lambert
-    float n[3], mlen, ndl;
+    float n[3], il, ndl;  // il: 1 / length of the interpolated normal (0 for none)
     float np[3];          // the shading normal: n, or the normal-mapped n' (shade_mode 3)
 };
 
@@ -153,9 +159,11 @@ __device__ __forceinline__ float4 load_ntexel(const Globals &g, long long idx)
     return __ldg(reinterpret_cast<const float4 *>(g.ntex) + idx);
 }
 
+// i modulo n (REPEAT wrap): the integer division, some 25 instructions, only outside [0, n)
 __device__ __forceinline__ int wrapi(int i, int n)
 {
-    int m = i % n;
+    if ((unsigned)i < (unsigned)n) return i;
+    const int m = i % n;
     return m < 0 ? m + n : m;
 }
 
@@ -248,24 +256,24 @@ __device__ __forceinline__ void nmap_eval(const Globals &g, const MeshK &M, cons
     for (int c = 0; c < 3; ++c) N.np[c] = fmul(mp[c], iml);
 }
 
-// b, C, D and the sampling state of one layer from S.vi, S.iw, S.lam and dist.  Every
+// b, C and the sampling state of one layer from S.vi, S.iw and S.lam.  Every
 // operation is rounded as written (no contraction left to the compiler), so the kernels
 // that shade a layer -- forward, forward from stored layers, adjoint -- agree bit for bit.
-// The reciprocals of the barycentric sum and of the normal's length, and the sigmoid's
-// exponential and division, are the fast hardware approximations (a few ulp, far inside the
-// 1e-5 image tolerance): this function runs for every shaded layer in every pass.
-// X: the kernel has the normal map compiled in (the kernels without it stay lean)
-template <bool X>
-__device__ __forceinline__ void shade(const Globals &g, const ViewK &V, const MeshK &M, float dist, Shade &S)
+// The reciprocals of the barycentric sum and of the normal's length are the fast hardware
+// approximations (a few ulp, far inside the 1e-5 image tolerance): this function runs for
+// every shaded layer in every pass.
+// X: the kernel has the normal map compiled in (the kernels without it stay lean); ADJ: for an
+// adjoint, which takes the texel derivatives with the texels at hand instead of loading them
+// again.
+template <bool X, bool ADJ>
+__device__ __forceinline__ void shade(const Globals &g, const ViewK &V, const MeshK &M, Shade &S)
 {
     float q[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) q[i] = fmul(S.lam[i], S.iw[i]);
-    S.Q = fadd(fadd(q[0], q[1]), q[2]);
-    const float iQ = __fdividef(1.f, S.Q);   // 2 ulp
+    S.iQ = __fdividef(1.f, fadd(fadd(q[0], q[1]), q[2]));   // 2 ulp
 #pragma unroll
-    for (int i = 0; i < 3; ++i) S.b[i] = fmul(q[i], iQ);
-    S.D = sigmoidf_stable(fmul(dist, V.inv_sigma_px));
+    for (int i = 0; i < 3; ++i) S.b[i] = fmul(q[i], S.iQ);
     const long long nvt = g.n_verts_total;
     if (g.shade_mode == 0) {
 #pragma unroll
@@ -286,8 +294,8 @@ __device__ __forceinline__ void shade(const Globals &g, const ViewK &V, const Me
     int x0, y0;
     texcoord(S.b, u, (float)M.tex_w, x0, S.fx, S.Xt);
     texcoord(S.b, v, (float)M.tex_h, y0, S.fy, S.Yt);
-    S.ix[0] = wrapi(x0, M.tex_w); S.ix[1] = wrapi(x0 + 1, M.tex_w);
-    S.iy[0] = wrapi(y0, M.tex_h); S.iy[1] = wrapi(y0 + 1, M.tex_h);
+    S.ix[0] = wrapi(x0, M.tex_w); S.ix[1] = S.ix[0] + 1 < M.tex_w ? S.ix[0] + 1 : 0;
+    S.iy[0] = wrapi(y0, M.tex_h); S.iy[1] = S.iy[0] + 1 < M.tex_h ? S.iy[0] + 1 : 0;
     const long long tb = M.tex_off;
     const float4 t00 = load_texel(g, tb + (long long)S.iy[0] * M.tex_w + S.ix[0]);
     const float4 t10 = load_texel(g, tb + (long long)S.iy[0] * M.tex_w + S.ix[1]);
@@ -298,6 +306,14 @@ __device__ __forceinline__ void shade(const Globals &g, const ViewK &V, const Me
     S.A[0] = ffma(w11, t11.x, ffma(w01, t01.x, ffma(w10, t10.x, fmul(w00, t00.x))));
     S.A[1] = ffma(w11, t11.y, ffma(w01, t01.y, ffma(w10, t10.y, fmul(w00, t00.y))));
     S.A[2] = ffma(w11, t11.z, ffma(w01, t01.z, ffma(w10, t10.z, fmul(w00, t00.z))));
+    if (ADJ) {
+        S.Ax[0] = gy * (t10.x - t00.x) + S.fy * (t11.x - t01.x);
+        S.Ax[1] = gy * (t10.y - t00.y) + S.fy * (t11.y - t01.y);
+        S.Ax[2] = gy * (t10.z - t00.z) + S.fy * (t11.z - t01.z);
+        S.Ay[0] = gx * (t01.x - t00.x) + S.fx * (t11.x - t10.x);
+        S.Ay[1] = gx * (t01.y - t00.y) + S.fx * (t11.y - t10.y);
+        S.Ay[2] = gx * (t01.z - t00.z) + S.fx * (t11.z - t10.z);
+    }
     if (g.shade_mode == 1) {
         S.C[0] = S.A[0]; S.C[1] = S.A[1]; S.C[2] = S.A[2];
         return;
@@ -311,9 +327,8 @@ __device__ __forceinline__ void shade(const Globals &g, const ViewK &V, const Me
         m[2] = ffma(S.b[i], nv.z, m[2]);
     }
     const float m2 = ffma(m[0], m[0], ffma(m[1], m[1], fmul(m[2], m[2])));
-    const float il = m2 > 0.f ? rsqrtf(m2) : 0.f;   // 2 ulp
-    S.mlen = fmul(m2, il);
-    S.n[0] = fmul(m[0], il); S.n[1] = fmul(m[1], il); S.n[2] = fmul(m[2], il);
+    S.il = m2 > 0.f ? rsqrtf(m2) : 0.f;   // 2 ulp
+    S.n[0] = fmul(m[0], S.il); S.n[1] = fmul(m[1], S.il); S.n[2] = fmul(m[2], S.il);
     S.np[0] = S.n[0]; S.np[1] = S.n[1]; S.np[2] = S.n[2];
     if (X && g.shade_mode == 3) {
         NMap N;
@@ -332,18 +347,37 @@ struct Layer {
     Shade S;
 };
 
-template <bool X>
-__device__ __forceinline__ bool layer_build(const Globals &g, const ViewK &V, const MeshK &M, int id,
-                                            float px, float py, Layer &L)
+// front (warp-uniform): the layer is a hard one of which the colour alone is wanted (a pixel outside
+// the edge mask shows its front layer's): its barycentrics are the area ratios, and the distance,
+// the candidate and hard tests and the coverage D are left out.
+template <bool X, bool ADJ>
+__device__ __forceinline__ bool layer_eval(const Globals &g, const ViewK &V, const MeshK &M, float px, float py,
+                                           bool front, Layer &L)
 {
-    if (!face_get(g, V, M, id, L.R)) return false;
-    if (!eval_face(L.R, px, py, V.r_px, V.half_inv_S, L.fr)) return false;
-    frag_lambda(L.R, L.fr, L.S.lam);
+    if (front) {
+        front_lambda(L.R, px, py, L.S.lam);
+        L.fr.hard = 1;
+        L.fr.feat = 0;
+        L.fr.t = 0.f;
+        L.S.D = 0.f;
+    } else {
+        if (!eval_face(L.R, px, py, V.r_px, V.half_inv_S, L.fr)) return false;
+        frag_lambda(L.R, L.fr, L.S.lam);
+        // the exponential and the division are the fast hardware forms (a few ulp)
+        L.S.D = sigmoidf_stable(fmul(L.fr.dist, V.inv_sigma_px));
+    }
 #pragma unroll
     for (int i = 0; i < 3; ++i) { L.S.vi[i] = L.R.vi[i]; L.S.iw[i] = L.R.iw[i]; }
     L.S.odd = (L.R.flags & FLAG_ODD) != 0;
-    shade<X>(g, V, M, L.fr.dist, L.S);
+    shade<X, ADJ>(g, V, M, L.S);
     return true;
+}
+
+template <bool X, bool ADJ>
+__device__ __forceinline__ bool layer_build(const Globals &g, const ViewK &V, const MeshK &M, int id,
+                                            float px, float py, bool front, Layer &L)
+{
+    return face_get(g, V, M, id, L.R) && layer_eval<X, ADJ>(g, V, M, px, py, front, L);
 }
 
 // ---------------------------------------------------------------------------
@@ -364,8 +398,8 @@ __device__ __forceinline__ bool layer_adjoint(const Globals &g, const ViewK &V, 
     float dx[3], dy[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        dx[i] = (px - R.c[i].xh) - R.c[i].xl;
-        dy[i] = (py - R.c[i].yh) - R.c[i].yl;
+        dx[i] = fsub(fsub(px, R.c[i].xh), R.c[i].xl);   // as eval_face formed them
+        dy[i] = fsub(fsub(py, R.c[i].yh), R.c[i].yl);
     }
     float gX[3] = {0.f, 0.f, 0.f}, gY[3] = {0.f, 0.f, 0.f}, gW[3] = {0.f, 0.f, 0.f};
     const float o = (R.flags & 1) ? 1.f : -1.f;
@@ -380,7 +414,7 @@ __device__ __forceinline__ bool layer_adjoint(const Globals &g, const ViewK &V, 
             if (ft == a) {
                 // F = o cross(V_b - V_a, p - V_a) / |V_b - V_a|
                 const float ex = dx[a] - dx[b], ey = dy[a] - dy[b];
-                const float il = 1.f / sqrtf(ex * ex + ey * ey);
+                const float il = fabsf(R.invL[a]);
                 const float c = ex * dy[a] - ey * dx[a];
                 const float il3 = il * il * il;
                 const float gex = o * (dy[a] * il - c * ex * il3);
@@ -391,10 +425,11 @@ __device__ __forceinline__ bool layer_adjoint(const Globals &g, const ViewK &V, 
             }
             if (ft == 3 + a) {
                 // dist = -|p - V_a|
-                const float l = sqrtf(dx[a] * dx[a] + dy[a] * dy[a]);
+                const float l = -L.fr.dist;
                 if (l > 0.f) {
-                    gX[a] += gdist * dx[a] / l;
-                    gY[a] += gdist * dy[a] / l;
+                    const float s = gdist / l;
+                    gX[a] += s * dx[a];
+                    gY[a] += s * dy[a];
                 }
             }
         }
@@ -422,7 +457,7 @@ __device__ __forceinline__ bool layer_adjoint(const Globals &g, const ViewK &V, 
             } else {
                 const float sl = fmaxf(S.ndl, 0.f);
                 gA[0] = gC[0] * sl; gA[1] = gC[1] * sl; gA[2] = gC[2] * sl;
-                if (S.ndl > 0.f && S.mlen > 0.f) {
+                if (S.ndl > 0.f && S.il > 0.f) {
                     const float gs = gC[0] * S.A[0] + gC[1] * S.A[1] + gC[2] * S.A[2];
                     if (EXTRA && gl) {
                         // C = A max(0, n.l): dL/dl = (gC . A) n (n' with a normal map)
@@ -503,9 +538,8 @@ __device__ __forceinline__ bool layer_adjoint(const Globals &g, const ViewK &V, 
                         }
                     }
                     const float nd = S.n[0] * gn[0] + S.n[1] * gn[1] + S.n[2] * gn[2];
-                    const float il = 1.f / S.mlen;
-                    const float gm[3] = {(gn[0] - S.n[0] * nd) * il, (gn[1] - S.n[1] * nd) * il,
-                                         (gn[2] - S.n[2] * nd) * il};
+                    const float gm[3] = {(gn[0] - S.n[0] * nd) * S.il, (gn[1] - S.n[1] * nd) * S.il,
+                                         (gn[2] - S.n[2] * nd) * S.il};
 #pragma unroll
                     for (int i = 0; i < 3; ++i) {
                         const long long gi = M.vert_off + S.vi[i];
@@ -539,14 +573,8 @@ __device__ __forceinline__ bool layer_adjoint(const Globals &g, const ViewK &V, 
                 atomicAdd(gt + i01, make_float4(w01 * gA[0], w01 * gA[1], w01 * gA[2], 0.f));
                 atomicAdd(gt + i11, make_float4(w11 * gA[0], w11 * gA[1], w11 * gA[2], 0.f));
             }
-            const float4 t00 = load_texel(g, i00), t10 = load_texel(g, i10), t01 = load_texel(g, i01),
-                         t11 = load_texel(g, i11);
-            const float gx = gA[0] * ((1.f - S.fy) * (t10.x - t00.x) + S.fy * (t11.x - t01.x)) +
-                             gA[1] * ((1.f - S.fy) * (t10.y - t00.y) + S.fy * (t11.y - t01.y)) +
-                             gA[2] * ((1.f - S.fy) * (t10.z - t00.z) + S.fy * (t11.z - t01.z));
-            const float gy = gA[0] * ((1.f - S.fx) * (t01.x - t00.x) + S.fx * (t11.x - t10.x)) +
-                             gA[1] * ((1.f - S.fx) * (t01.y - t00.y) + S.fx * (t11.y - t10.y)) +
-                             gA[2] * ((1.f - S.fx) * (t01.z - t00.z) + S.fx * (t11.z - t10.z));
+            const float gx = gA[0] * S.Ax[0] + gA[1] * S.Ax[1] + gA[2] * S.Ax[2];
+            const float gy = gA[0] * S.Ay[0] + gA[1] * S.Ay[1] + gA[2] * S.Ay[2];
             // x = sum b_i X_i - 1/2; adding a constant to every gb_i is invisible to the
             // perspective step below (sum b = 1), so corner offsets from corner 0 are used
             // (the normal map, sampled at the same texel coordinates, adds gxn, gyn)
@@ -555,11 +583,10 @@ __device__ __forceinline__ bool layer_adjoint(const Globals &g, const ViewK &V, 
         }
         // perspective-correct barycentrics: b_i = q_i / Q, q_i = lam_i / w_i
         const float bdot = S.b[0] * gb[0] + S.b[1] * gb[1] + S.b[2] * gb[2];
-        const float iQ = 1.f / S.Q;
         float glam[3];
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            const float gq = (gb[i] - bdot) * iQ;
+            const float gq = (gb[i] - bdot) * S.iQ;
             glam[i] = gq * S.iw[i];
             gW[i] += gq * S.lam[i];
         }
@@ -660,15 +687,13 @@ struct Smem {
     // every mode
     int view, totals[2], next;
     int item_ctr;        // raster: the next (face, row segment) item of the chunk a warp takes
-    int qn[2];           // the stored-ids adjoint: its layer ring's items queued / taken
     unsigned long long m0[HS_MAX], m1[HS_MAX];   // per halo row: columns with S^H = 0 / 1
     unsigned eb[TT_MAX], hb[TT_MAX];   // per tile row: pixels with E = 1, with S^H = 1
     unsigned rm[TT_MAX];               // per tile row: pixels that the raster pass serves
     unsigned char sh[HS_MAX * HS_MAX];
     // the raster (forward and re-rasterizing adjoint) only: the modes from stored layer
-    // ids are launched with the shared memory up to F (the stored-ids adjoint adds its
-    // layer queues there, adj_smem_bytes), leaving the rest of the SM's unified L1 / shared storage
-    // to the L1 cache
+    // ids are launched with the shared memory up to F, leaving the rest of the SM's unified
+    // L1 / shared storage to the L1 cache
     FaceGeo F[CH];       // the staged chunk's faces (geometric part)
     int fid[CH];         // their face ids
     Pre P[CH];
@@ -679,7 +704,7 @@ struct Smem {
     unsigned rdiv[CH];   // rounded-up 2^32 / (segments per rect row), 0 for one (rect_xy)
     unsigned hdiv[CH];   // the same for the ring rect's width
     int2 hash[HASH];     // (face id, slot) of the last staged chunk
-    int wsum[2][NT / 32];
+    int wsum[2][NT_MAX / 32];
 };
 
 __device__ __forceinline__ unsigned long long pack_frag(float key, int id)
@@ -778,8 +803,49 @@ __device__ __forceinline__ bool kept_hard(const Globals &g, const ViewK &V, cons
            eval_face<false>(R, px, py, V.r_px, V.half_inv_S, fr) && fr.hard;
 }
 
+// halo_rows from stored layers: S^H of the tile and of its ring is the hard flag of every pixel's
+// front layer (a non-negative id: hard; bit 31: soft).  A warp takes rows, and issues all its
+// loads before the first result is used.  Returns whether this thread saw a layer in the tile.
+template <int TT, int NT>
+__device__ __forceinline__ bool halo_from_ids(const Globals &g, Smem &S, const ViewK &V, int X0, int Y0, int rho)
+{
+    constexpr int ROWS = (TT + 2 * RHO_MAX) / (NT / 32), HALVES = TT + 2 * RHO_MAX > 32 ? 2 : 1;
+    const int hs = TT + 2 * rho, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int f[ROWS][HALVES];
+    unsigned in = 0u;
+#pragma unroll
+    for (int u = 0; u < ROWS; ++u)
+#pragma unroll
+        for (int h = 0; h < HALVES; ++h) {
+            const int row = warp + u * (NT / 32), col = lane + 32 * h;
+            const int X = X0 - rho + col, Y = Y0 - rho + row;
+            f[u][h] = -1;
+            if (row < hs && col < hs && X >= 0 && Y >= 0 && X < V.W && Y < V.H) {
+                f[u][h] = __ldg(g.ids_in + V.pix_off + (long long)Y * V.W + X);
+                in |= 1u << (u * HALVES + h);
+            }
+        }
+    bool any = false;
+#pragma unroll
+    for (int u = 0; u < ROWS; ++u) {
+        const int row = warp + u * (NT / 32);
+        if (row >= hs) break;
+        unsigned long long b0 = 0ull, b1 = 0ull;
+#pragma unroll
+        for (int h = 0; h < HALVES; ++h) {
+            const bool here = (in >> (u * HALVES + h)) & 1u;
+            const int col = lane + 32 * h;
+            b0 |= (unsigned long long)__ballot_sync(0xffffffffu, here && f[u][h] < 0) << (32 * h);
+            b1 |= (unsigned long long)__ballot_sync(0xffffffffu, here && f[u][h] >= 0) << (32 * h);
+            any |= f[u][h] != -1 && row >= rho && row < TT + rho && col >= rho && col < TT + rho;
+        }
+        if (lane == 0) { S.m0[row] = b0; S.m1[row] = b1; }
+    }
+    return any;
+}
+
 // per halo row, the columns holding S^H = 0 and S^H = 1 (hs <= 48 fits 64 bits)
-template <int TT>
+template <int TT, int NT>
 __device__ __forceinline__ void halo_rows(Smem &S, int hs)
 {
     const int lane = threadIdx.x & 31;
@@ -892,7 +958,7 @@ __device__ __forceinline__ bool pixel_weights(const Globals &g, const ViewK &V, 
 #pragma unroll 1
         for (int k = 0; k < nl; ++k) {
             Layer L;
-            if (layer_build<EXTRA>(g, V, M, ids[k], px, py, L)) {
+            if (layer_build<EXTRA, true>(g, V, M, ids[k], px, py, false, L)) {
                 Dk[k] = L.S.D;
                 Ck[k][0] = L.S.C[0]; Ck[k][1] = L.S.C[1]; Ck[k][2] = L.S.C[2];
             }
@@ -933,7 +999,7 @@ __device__ __forceinline__ unsigned adjoint_pixel(const Globals &g, const Smem &
         const bool any = gDl != 0.f || gCl[0] != 0.f || gCl[1] != 0.f || gCl[2] != 0.f;
         Layer L;
         const long long slot = (V.slot_base + (long long)Y * V.W + X) * K + k;
-        if (any && layer_build<EXTRA>(g, V, M, ids[k], px, py, L)) {
+        if (any && layer_build<EXTRA, true>(g, V, M, ids[k], px, py, false, L)) {
             ++layers;
             if (layer_adjoint<EXTRA>(g, V, M, L, px, py, gCl, gDl, slot, gl)) stored |= 1u << k;
         }
@@ -999,49 +1065,54 @@ __device__ __forceinline__ unsigned finish_forward(const Globals &g, const Smem 
     float Cs[3] = {0.f, 0.f, 0.f}, C1[3] = {0.f, 0.f, 0.f};
     float Ds = 0.f, prod = 1.f;
     unsigned layers = 0;
-    for (int w = 0; w * 32 < tot; ++w) {
+    // a warp without edge-masked pixels (most) needs no list: each lane shades its own front layer
+    const bool anyE = __any_sync(FULL, E);
+    const int passes = anyE ? (tot + 31) >> 5 : (tot > 0 ? 1 : 0);
+    for (int w = 0; w < passes; ++w) {
         const int i = w * 32 + lane;
-        // the pixel (lane) whose layers include list entry i: the last one starting at or before it
-        int o = 0;
+        int o = lane, id = ids[0];
+        bool act = cnt > 0;
+        if (anyE) {
+            // the pixel (lane) whose layers include list entry i: the last one starting at or before it
+            o = 0;
 #pragma unroll
-        for (int st = 16; st > 0; st >>= 1)
-            if (__shfl_sync(FULL, off, o + st) <= i) o += st;
-        const int k = i - __shfl_sync(FULL, off, o);
-        int id = 0x7fffffff;
+            for (int st = 16; st > 0; st >>= 1)
+                if (__shfl_sync(FULL, off, o + st) <= i) o += st;
+            const int k = i - __shfl_sync(FULL, off, o);
+            id = 0x7fffffff;
 #pragma unroll
-        for (int kk = 0; kk < K; ++kk) {
-            const int v = __shfl_sync(FULL, ids[kk], o);
-            if (kk == k) id = v;
+            for (int kk = 0; kk < K; ++kk) {
+                const int v = __shfl_sync(FULL, ids[kk], o);
+                if (kk == k) id = v;
+            }
+            act = i < tot;
         }
         float C[3] = {0.f, 0.f, 0.f}, D = 0.f;
         int live = 0;
-        if (i < tot) {
+        if (act) {
             // re-evaluate the layer at its pixel (from shared memory when the whole tile
             // list was staged at once): distance and barycentrics, then the shading
             const int po = p - lane + o;
             const float px = (float)(X0 + po % TT) + 0.5f, py = (float)(Y0 + po / TT) + 0.5f;
             const int slot = single_chunk ? find_slot(S, id) : -1;
-            FaceRec R;
+            Layer L;
             bool ok;
             if (slot >= 0) {
-                face_complete(g, V, id, S.F[slot], R);
-                ok = (R.flags & FLAG_LIVE) != 0;
+                face_complete(g, V, id, S.F[slot], L.R);
+                ok = (L.R.flags & FLAG_LIVE) != 0;
             } else {
-                ok = face_get(g, V, M, id, R);
+                ok = face_get(g, V, M, id, L.R);
             }
-            Frag fr;
-            if (ok && eval_face(R, px, py, V.r_px, V.half_inv_S, fr)) {
-                Shade Sh;
-                frag_lambda(R, fr, Sh.lam);
-#pragma unroll
-                for (int q = 0; q < 3; ++q) { Sh.vi[q] = R.vi[q]; Sh.iw[q] = R.iw[q]; }
-                Sh.odd = (R.flags & FLAG_ODD) != 0;
-                shade<EXTRA>(g, V, M, fr.dist, Sh);
-                C[0] = Sh.C[0]; C[1] = Sh.C[1]; C[2] = Sh.C[2];
-                D = Sh.D;
+            if (ok && layer_eval<EXTRA, false>(g, V, M, px, py, !anyE, L)) {
+                C[0] = L.S.C[0]; C[1] = L.S.C[1]; C[2] = L.S.C[2];
+                D = L.S.D;
                 live = 1;
                 ++layers;
             }
+        }
+        if (!anyE) {
+            C1[0] = C[0]; C1[1] = C[1]; C1[2] = C[2];
+            break;
         }
         // this pixel's layers among the entries of this pass, in layer order
 #pragma unroll
@@ -1081,33 +1152,32 @@ __device__ __forceinline__ unsigned finish_forward(const Globals &g, const Smem 
     return layers;
 }
 
-// The re-rasterizing adjoint of one round of pixels (one per thread; lanes outside the
-// image take part with no layer), warp-collective like the forward's shading: a warp
-// rebuilds the layers its edge-masked pixels blend (for D_k, C_k) as one list, each
-// pixel forms dL/dC_k, dL/dD_k (blend_weights), and the warp then rebuilds and
-// back-propagates the layers with a gradient as a second list.
+// The adjoint of one round of pixels (one per thread; lanes outside the image take part with
+// no layer), warp-collective like the forward's shading: a warp rebuilds the layers its
+// edge-masked pixels blend (for D_k, C_k) as one list, each pixel forms dL/dC_k, dL/dD_k
+// (blend_weights), and the warp then rebuilds and back-propagates the layers with a gradient
+// as a second list.  A warp without edge-masked pixels (most) needs neither list nor shuffles:
+// each lane back-propagates its own front layer.  Nothing here waits for another warp: a
+// CTA-wide layer queue, which this replaced for the stored-ids adjoint, filled its lanes
+// better at the silhouettes but held all warps at its barriers.
+// ids: a pixel's layers (0x7fffffff none); outside the edge mask only the front one is read.
 template <int K, int TT>
 __device__ __forceinline__ unsigned adjoint_warp(const Globals &g, const Smem &S, const ViewK &V, const MeshK &M,
-                                                 int X0, int Y0, int p, bool in, const int (&ids)[K])
+                                                 int X0, int Y0, int p, bool in, const int (&ids)[K], float4 gi4)
 {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int lx = p % TT, ly = p / TT;
     int nl = 0;
     bool E = false, SH = false, active = false;
-    float4 gi4 = make_float4(0.f, 0.f, 0.f, 0.f);
     if (in) {
 #pragma unroll
         for (int k = 0; k < K; ++k) nl += (ids[k] != 0x7fffffff) ? 1 : 0;
-        if (nl > 0) {
-            gi4 = __ldg(reinterpret_cast<const float4 *>(g.gin) + V.pix_off + (long long)(Y0 + ly) * V.W + (X0 + lx));
-            active = gi4.x != 0.f || gi4.y != 0.f || gi4.z != 0.f || gi4.w != 0.f;
-            if (active) {
-                SH = row_bit(S.hb, lx, ly);
-                E = row_bit(S.eb, lx, ly);
-            }
-        }
+        active = nl > 0 && (gi4.x != 0.f || gi4.y != 0.f || gi4.z != 0.f || gi4.w != 0.f);
+        SH = row_bit(S.hb, lx, ly);
+        E = active && row_bit(S.eb, lx, ly);
     }
+    const bool anyE = __any_sync(FULL, E);   // else every layer is a pixel's front one
     // list entry i of a warp list with per-lane counts cnt (exclusive offsets off):
     // the owning lane
     auto owner = [&](int off, int i) {
@@ -1133,9 +1203,9 @@ __device__ __forceinline__ unsigned adjoint_warp(const Globals &g, const Smem &S
 #pragma unroll
     for (int k = 0; k < K; ++k) { Dk[k] = 0.f; Ck[k][0] = Ck[k][1] = Ck[k][2] = 0.f; }
     {
-        const int cnt = (active && E) ? nl : 0;
-        int tot;
-        const int off = scan(cnt, tot);
+        const int cnt = E ? nl : 0;
+        int tot = 0, off = 0;
+        if (anyE) off = scan(cnt, tot);
         for (int w = 0; w * 32 < tot; ++w) {
             const int i = w * 32 + lane;
             const int o = owner(off, i);
@@ -1150,7 +1220,7 @@ __device__ __forceinline__ unsigned adjoint_warp(const Globals &g, const Smem &S
             if (i < tot) {
                 const int po = p - lane + o;
                 Layer L;
-                if (layer_build<false>(g, V, M, id, (float)(X0 + po % TT) + 0.5f, (float)(Y0 + po / TT) + 0.5f, L)) {
+                if (layer_build<false, false>(g, V, M, id, (float)(X0 + po % TT) + 0.5f, (float)(Y0 + po / TT) + 0.5f, false, L)) {
                     C[0] = L.S.C[0]; C[1] = L.S.C[1]; C[2] = L.S.C[2];
                     D = L.S.D;
                 }
@@ -1184,203 +1254,45 @@ __device__ __forceinline__ unsigned adjoint_warp(const Globals &g, const Smem &S
     // pass 2: the adjoints of the layers with a gradient
     unsigned layers = 0;
     {
-        int tot;
-        const int off = scan(__popc(want), tot);
-        for (int w = 0; w * 32 < tot; ++w) {
-            const int i = w * 32 + lane;
-            const int o = owner(off, i);
-            const int j = i - __shfl_sync(FULL, off, o);   // the owner's j-th layer with a gradient
-            const unsigned wm = __shfl_sync(FULL, want, o);
-            int k = 0;
+        int tot = 0, off = 0;
+        if (anyE) off = scan(__popc(want), tot);
+        const int passes = anyE ? (tot + 31) >> 5 : 1;
+        for (int w = 0; w < passes; ++w) {
+            int o = lane, k = 0, id = ids[0];
+            float gC[3] = {gCk[0][0], gCk[0][1], gCk[0][2]}, gD = 0.f;
+            bool act = want != 0u;
+            if (anyE) {
+                const int i = w * 32 + lane;
+                o = owner(off, i);
+                const int j = i - __shfl_sync(FULL, off, o);   // the owner's j-th layer with a gradient
+                const unsigned wm = __shfl_sync(FULL, want, o);
 #pragma unroll
-            for (int kk = 0, seen = 0; kk < K; ++kk)
-                if ((wm >> kk) & 1u) {
-                    if (seen == j) k = kk;
-                    ++seen;
+                for (int kk = 0, seen = 0; kk < K; ++kk)
+                    if ((wm >> kk) & 1u) {
+                        if (seen == j) k = kk;
+                        ++seen;
+                    }
+#pragma unroll
+                for (int kk = 0; kk < K; ++kk) {
+                    const int v = __shfl_sync(FULL, ids[kk], o);
+                    const float a0 = __shfl_sync(FULL, gCk[kk][0], o), a1 = __shfl_sync(FULL, gCk[kk][1], o),
+                                a2 = __shfl_sync(FULL, gCk[kk][2], o), b = __shfl_sync(FULL, gDk[kk], o);
+                    if (kk == k) { id = v; gC[0] = a0; gC[1] = a1; gC[2] = a2; gD = b; }
                 }
-            int id = 0x7fffffff;
-            float gC[3] = {0.f, 0.f, 0.f}, gD = 0.f;
-#pragma unroll
-            for (int kk = 0; kk < K; ++kk) {
-                const int v = __shfl_sync(FULL, ids[kk], o);
-                const float a0 = __shfl_sync(FULL, gCk[kk][0], o), a1 = __shfl_sync(FULL, gCk[kk][1], o),
-                            a2 = __shfl_sync(FULL, gCk[kk][2], o), b = __shfl_sync(FULL, gDk[kk], o);
-                if (kk == k) { id = v; gC[0] = a0; gC[1] = a1; gC[2] = a2; gD = b; }
+                act = i < tot;
             }
-            if (i < tot) {
+            if (act) {
                 const int po = p - lane + o;
                 const int Xo = X0 + po % TT, Yo = Y0 + po / TT;
                 const float px = (float)Xo + 0.5f, py = (float)Yo + 0.5f;
                 const long long slot = (V.slot_base + (long long)Yo * V.W + Xo) * K + k;
                 Layer L;
-                if (layer_build<false>(g, V, M, id, px, py, L)) {
+                if (layer_build<false, true>(g, V, M, id, px, py, !anyE, L)) {
                     ++layers;
                     layer_adjoint<false>(g, V, M, L, px, py, gC, gD, slot, nullptr);
                 }
             }
         }
-    }
-    return layers;
-}
-
-// The adjoint from stored layer ids, by layer rather than by pixel.  A layer rebuilt
-// from its face id (record, distance, barycentrics, shading) is the costliest step, and
-// by pixel it would run with the lanes of background, single-layer and gradient-free
-// pixels idle.  Each round of NT pixels (one per thread) instead
-//   1. queues, for an edge-masked pixel, each of its layers for the blend (D_k, C_k);
-//      a pixel outside the mask queues its front layer's adjoint directly
-//      (dL/dC = dL/dRGB when S^H = 1);
-//   2. rebuilds the queued layers with all threads into a (pixel, layer) table;
-//   3. forms each edge-masked pixel's dL/dC_k, dL/dD_k from the table (blend_weights)
-//      and queues its layers with a gradient;
-//   4. rebuilds and back-propagates the queued adjoints, whole multiples of NT at a
-//      time (the rest waits for the next round; the last round takes all).
-// Steps 2 and 3 are skipped in a round without edge-masked pixels.  The adjoint ring
-// holds fewer than NT leftovers plus one round's K NT items.
-template <int K>
-__host__ __device__ constexpr int adj_ring() { return NT * (K + 1); }
-__host__ __device__ constexpr size_t adj_ring_off() { return (offsetof(Smem, F) + 15) / 16 * 16; }
-template <int K>
-__host__ __device__ constexpr size_t adj_smem_bytes()
-{
-    // adjoint ring (dL/dC, dL/dD | face id, pixel and layer), blend table, blend queue
-    return adj_ring_off() + (sizeof(float4) + sizeof(int2)) * adj_ring<K>() + sizeof(float4) * NT * K +
-           sizeof(unsigned short) * NT * K;
-}
-
-template <int K, int TT>
-__device__ __forceinline__ unsigned adjoint_queued(const Globals &g, Smem &S, const ViewK &V, const MeshK &M,
-                                                   int X0, int Y0, int wlim, int hlim)
-{
-    constexpr int PPT = TT * TT / NT;
-    constexpr int QC = adj_ring<K>();
-    float4 *qg = reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(&S) + adj_ring_off());
-    int2 *qi = reinterpret_cast<int2 *>(qg + QC);        // (face id, pixel | layer << 10)
-    float4 *dc = reinterpret_cast<float4 *>(qi + QC);    // [thread][layer]: (C_k, D_k)
-    unsigned short *bq = reinterpret_cast<unsigned short *>(dc + NT * K);   // thread | layer << 8
-    const int tid = threadIdx.x, lane = tid & 31;
-    unsigned layers = 0;
-    // S.qn[0]: adjoint items queued, S.qn[1]: taken (both zero at the tile's start);
-    // S.totals[0]: blend items of the round
-    if (tid == 0) S.totals[0] = 0;
-    __syncthreads();
-
-    // warp-aggregated reservation of c slots on counter *ctr: returns this lane's first slot
-    auto reserve = [&](int *ctr, int c) {
-        int incl = c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        int base = 0;
-        if (lane == 31 && incl > 0) base = atomicAdd(ctr, incl);
-        return __shfl_sync(0xffffffffu, base, 31) + incl - c;
-    };
-    auto push_adj = [&](int base, int id, int p, int k, float c0, float c1, float c2, float d) {
-        const int q = base % QC;
-        qg[q] = make_float4(c0, c1, c2, d);
-        qi[q] = make_int2(id, p | (k << 10));
-    };
-
-    for (int j = 0; j < PPT; ++j) {
-        const int p = tid + j * NT;
-        const int lx = p % TT, ly = p / TT;
-        const int X = X0 + lx, Y = Y0 + ly;
-        const long long pix = V.pix_off + (long long)Y * V.W + X;
-        const bool in = lx < wlim && ly < hlim;
-        // step 1
-        int nl = 0, id0 = 0;
-        bool E = false, front = false;
-        float4 gi4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (in) {
-            // the layer ids and dL/dI together: one load latency instead of two in a row
-            int idk[K];
-#pragma unroll
-            for (int k = 0; k < K; ++k) idk[k] = __ldg(g.ids_in + (long long)k * g.n_pix + pix);
-            gi4 = __ldg(reinterpret_cast<const float4 *>(g.gin) + pix);
-#pragma unroll
-            for (int k = 0; k < K; ++k) nl += idk[k] != -1 ? 1 : 0;
-            if (nl > 0 && (gi4.x != 0.f || gi4.y != 0.f || gi4.z != 0.f || gi4.w != 0.f)) {
-                E = row_bit(S.eb, lx, ly);
-                // outside the mask the pixel is its front layer's colour where S^H = 1
-                front = !E && row_bit(S.hb, lx, ly) && (gi4.x != 0.f || gi4.y != 0.f || gi4.z != 0.f);
-                id0 = idk[0] & 0x7fffffff;
-            }
-        }
-        {
-            const int b = reserve(&S.totals[0], E ? nl : 0);
-            for (int k = 0; k < (E ? nl : 0); ++k) bq[b + k] = (unsigned short)(tid | (k << 8));
-            const int a = reserve(&S.qn[0], front ? 1 : 0);
-            if (front) push_adj(a, id0, p, 0, gi4.x, gi4.y, gi4.z, 0.f);
-        }
-        __syncthreads();
-        const int nb = S.totals[0];
-        if (nb > 0) {
-            // step 2: the blend table
-            for (int i = tid; i < nb; i += NT) {
-                const int it = bq[i];
-                const int o = it & 255, k = it >> 8;
-                const int po = o + j * NT;
-                const int Xo = X0 + po % TT, Yo = Y0 + po / TT;
-                const long long pixo = V.pix_off + (long long)Yo * V.W + Xo;
-                const int id = __ldg(g.ids_in + (long long)k * g.n_pix + pixo) & 0x7fffffff;
-                Layer L;
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (layer_build<false>(g, V, M, id, (float)Xo + 0.5f, (float)Yo + 0.5f, L))
-                    v = make_float4(L.S.C[0], L.S.C[1], L.S.C[2], L.S.D);
-                dc[o * K + k] = v;
-            }
-            __syncthreads();
-            // every thread has read the blend count; the next round's reservations
-            // come after this round's last barrier
-            if (tid == 0) S.totals[0] = 0;
-            // step 3
-            float gCk[K][3], gDk[K];
-            unsigned want = 0u;
-            int ids[K];
-            if (E) {
-                float Dk[K], Ck[K][3];
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    gDk[k] = 0.f; gCk[k][0] = gCk[k][1] = gCk[k][2] = 0.f;
-                    const float4 v = k < nl ? dc[tid * K + k] : make_float4(0.f, 0.f, 0.f, 0.f);
-                    Ck[k][0] = v.x; Ck[k][1] = v.y; Ck[k][2] = v.z; Dk[k] = v.w;
-                }
-                blend_weights<K>(Dk, Ck, nl, gi4, gCk, gDk);
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    ids[k] = k < nl ? __ldg(g.ids_in + (long long)k * g.n_pix + pix) & 0x7fffffff : 0;
-                    if (k < nl && (gDk[k] != 0.f || gCk[k][0] != 0.f || gCk[k][1] != 0.f || gCk[k][2] != 0.f))
-                        want |= 1u << k;
-                }
-            }
-            int a = reserve(&S.qn[0], __popc(want));
-#pragma unroll
-            for (int k = 0; k < K; ++k)
-                if ((want >> k) & 1u) push_adj(a++, ids[k], p, k, gCk[k][0], gCk[k][1], gCk[k][2], gDk[k]);
-            __syncthreads();
-        }
-        // step 4
-        const int head = S.qn[1], n = S.qn[0] - head;
-        const int m = (j == PPT - 1) ? n : n / NT * NT;
-        for (int i = tid; i < m; i += NT) {
-            const int q = (head + i) % QC;
-            const float4 gg = qg[q];
-            const int2 it = qi[q];
-            const int pp = it.y & 1023, k = it.y >> 10;
-            const int Xq = X0 + pp % TT, Yq = Y0 + pp / TT;
-            const float px = (float)Xq + 0.5f, py = (float)Yq + 0.5f;
-            const float gCl[3] = {gg.x, gg.y, gg.z};
-            const long long slot = (V.slot_base + (long long)Yq * V.W + Xq) * K + k;
-            Layer L;
-            if (layer_build<false>(g, V, M, it.x, px, py, L)) {
-                ++layers;
-                layer_adjoint<false>(g, V, M, L, px, py, gCl, gg.w, slot, nullptr);
-            }
-        }
-        __syncthreads();   // the items taken are free and every thread has read the counters
-        if (tid == 0) S.qn[1] = head + m;
     }
     return layers;
 }
@@ -1520,20 +1432,17 @@ __device__ __forceinline__ void raster_items(Smem &S, unsigned long long *kbuf, 
 template <int K, int MODE, int TT>
 __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned long long *kbuf, const int t)
 {
+    constexpr int NT = cta_threads<MODE, TT>();
     constexpr int PPT = TT * TT / NT;   // pixels per thread in the per-pixel phases
     // after the K-lists: the candidate queue and the two pair-block tables
     unsigned *qbuf = reinterpret_cast<unsigned *>(kbuf + TT * TT * K);
-    unsigned char *blk = reinterpret_cast<unsigned char *>(qbuf + QN);
+    unsigned char *blk = reinterpret_cast<unsigned char *>(qbuf + NT / 32 * WQ);
     unsigned char *hblk = blk + NBLK;
     // the adjoints with extras: each thread's share of dL/dlight, after the part of the
     // shared memory the kernel uses (the header alone when it reads stored layers)
     float(*gl_slots)[3] = reinterpret_cast<float(*)[3]>(
         MODE == 4 ? reinterpret_cast<unsigned char *>(&S) + offsetof(Smem, F) : hblk + NBLK);
-    if (threadIdx.x == 0) {
-        S.view = g.tile_view[t];
-        S.qn[0] = 0;
-        S.qn[1] = 0;
-    }
+    if (threadIdx.x == 0) S.view = g.tile_view[t];
     __syncthreads();
     const ViewK &V = g.views[S.view];
     const MeshK &M = g.meshes[V.mesh];
@@ -1544,10 +1453,6 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
     const int hs = TT + 2 * rho;
     const int wlim = min(TT, V.W - X0), hlim = min(TT, V.H - Y0);   // tile part inside the image
 
-    for (int i = tid; i < hs * hs; i += NT) {
-        const int hx = X0 - rho + i % hs, hy = Y0 - rho + i / hs;
-        S.sh[i] = (hx >= 0 && hy >= 0 && hx < V.W && hy < V.H) ? 0 : 2;
-    }
     constexpr bool EXTRA = MODE >= 4;
     constexpr bool BWD = MODE == 1 || MODE == 2 || MODE == 4 || MODE == 5;
     constexpr bool from_ids = MODE == 2 || MODE == 3 || MODE == 4 || MODE == 7;
@@ -1560,6 +1465,11 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
     unsigned n_pairs = 0, n_exact = 0, n_cand = 0, n_layers = 0;
     float l2acc = 0.f;   // the fused L2 loss: this thread's sum of squares
     if (!from_ids) {
+        for (int row = tid >> 5; row < hs; row += NT / 32)
+            for (int col = tid & 31; col < hs; col += 32) {
+                const int hx = X0 - rho + col, hy = Y0 - rho + row;
+                S.sh[row * hs + col] = (hx >= 0 && hy >= 0 && hx < V.W && hy < V.H) ? 0 : 2;
+            }
         const long long lb = g.tile_off[t], le = g.tile_off[t + 1];
         const bool fallback = le > g.list_cap;
         const int n = fallback ? M.nF : (int)(le - lb);
@@ -1775,7 +1685,7 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
                     layered = true;
                     stage = ST_LAYERS;
                 } else {
-                    halo_rows<TT>(S, hs);
+                    halo_rows<TT, NT>(S, hs);
                     __syncthreads();
                     edge_rows<TT>(g, S, rho, wlim, hlim);
                     const bool any = tid < TT && S.eb[tid] != 0u;
@@ -1805,7 +1715,7 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
             }
             __syncthreads();
             if (!empty) {
-                halo_rows<TT>(S, hs);
+                halo_rows<TT, NT>(S, hs);
                 __syncthreads();
                 edge_rows<TT>(g, S, rho, wlim, hlim);
                 __syncthreads();
@@ -1830,46 +1740,18 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
     } else {
         // layers stored by the forward: S^H of the tile and of its ring is the hard flag
         // of every pixel's stored front layer (a non-negative id: hard; bit 31: soft)
-        bool any = false;   // some pixel of the tile itself holds a layer
-        // every load of the thread's share is issued before the first result is used
-        constexpr int HI = (HS_MAX * HS_MAX + NT - 1) / NT;
-        int fl[HI];
-        unsigned loaded = 0u;   // bit u: entry u is inside the halo and the image
-#pragma unroll
-        for (int u = 0; u < HI; ++u) {
-            const int i = tid + u * NT;
-            fl[u] = -1;
-            if (i < hs * hs && S.sh[i] != 2) {
-                const int hx = i % hs - rho, hy = i / hs - rho;
-                fl[u] = __ldg(g.ids_in + V.pix_off + (long long)(Y0 + hy) * V.W + (X0 + hx));
-                loaded |= 1u << u;
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < HI; ++u) {
-            if (!((loaded >> u) & 1u)) continue;
-            const int i = tid + u * NT;
-            const int hx = i % hs - rho, hy = i / hs - rho;
-            S.sh[i] = fl[u] >= 0 ? 1 : 0;
-            any |= fl[u] != -1 && hx >= 0 && hy >= 0 && hx < TT && hy < TT;
-        }
         // an adjoint over a tile whose pixels hold no layer has nothing to propagate; a
         // forward over it writes the background
-        const bool some = __syncthreads_or(any);
+        const bool some = __syncthreads_or(halo_from_ids<TT, NT>(g, S, V, X0, Y0, rho));
         if (BWD && !some) return;
         empty = !some;
     }
     if (from_ids && !empty) {
-        __syncthreads();
-        halo_rows<TT>(S, hs);
-        __syncthreads();
         edge_rows<TT>(g, S, rho, wlim, hlim);
         __syncthreads();
     }
 
-    if constexpr (MODE == 2) {
-        n_layers = adjoint_queued<K, TT>(g, S, V, M, X0, Y0, wlim, hlim);
-    } else if (empty) {
+    if (empty) {
         // background: no layer, RGBA 0 (the loss's gradient 2 (0 - target))
         for (int j = 0; j < PPT; ++j) {
             const int p = tid + j * NT;
@@ -1888,13 +1770,45 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
                 l2acc += dx * dx + dy * dy + dz * dz + dw * dw;
             }
         }
+    } else if constexpr (MODE == 2) {
+        // the adjoint from stored ids: a round's front ids and dL/dI are loaded under the round
+        // before it
+        int id0 = -1;
+        float4 gi = make_float4(0.f, 0.f, 0.f, 0.f);
+        auto fetch = [&](int j) {
+            const int p = tid + j * NT, lx = p % TT, ly = p / TT;
+            id0 = -1;
+            if (row_bit(S.eb, lx, ly) || row_bit(S.hb, lx, ly)) {   // bits of pixels in the image
+                const long long pix = V.pix_off + (long long)(Y0 + ly) * V.W + (X0 + lx);
+                id0 = __ldg(g.ids_in + pix);
+                gi = __ldg(reinterpret_cast<const float4 *>(g.gin) + pix);
+            }
+        };
+        fetch(0);
+        for (int j = 0; j < PPT; ++j) {
+            const int p = tid + j * NT, lx = p % TT, ly = p / TT;
+            int ids[K];
+            ids[0] = id0 == -1 ? 0x7fffffff : (id0 & 0x7fffffff);
+            const float4 gj = gi;
+            if (j + 1 < PPT) fetch(j + 1);
+            const bool E = row_bit(S.eb, lx, ly);
+#pragma unroll
+            for (int k = 1; k < K; ++k) {
+                ids[k] = 0x7fffffff;
+                if (E) {
+                    const int id = __ldg(g.ids_in + (long long)k * g.n_pix + V.pix_off + (long long)(Y0 + ly) * V.W + (X0 + lx));
+                    if (id != -1) ids[k] = id & 0x7fffffff;
+                }
+            }
+            n_layers += adjoint_warp<K, TT>(g, S, V, M, X0, Y0, p, lx < wlim && ly < hlim, ids, gj);
+        }
     } else for (int j = 0; j < PPT; ++j) {
         const int p = tid + j * NT;
         const int lx = p % TT, ly = p / TT;
         const bool in = lx < wlim && ly < hlim;
-        // the forward's shading and the re-rasterizing adjoint are warp-collective: every
+        // the forward's shading and the adjoint without extras are warp-collective: every
         // lane takes part
-        if (BWD && MODE != 1 && !in) continue;
+        if (BWD && EXTRA && !in) continue;
         int ids[K];
         unsigned hardbits = 0u;
 #pragma unroll
@@ -1919,15 +1833,22 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
             }
         } else {
             const long long pix = V.pix_off + (long long)(Y0 + ly) * V.W + (X0 + lx);
+            // a pixel outside the edge mask shows its front layer, where S^H = 1 (the inverse UV
+            // samples every front layer)
+            const bool E = row_bit(S.eb, lx, ly), SH = row_bit(S.hb, lx, ly);
 #pragma unroll
             for (int k = 0; k < K; ++k) {
+                if (!(E || (k == 0 && SH)) && MODE != 4) continue;
                 const int id = __ldg(g.ids_in + (long long)k * g.n_pix + pix);
                 ids[k] = id == -1 ? 0x7fffffff : (id & 0x7fffffff);
             }
         }
-        if constexpr (MODE == 1)
-            n_layers += adjoint_warp<K, TT>(g, S, V, M, X0, Y0, p, in, ids);
-        else if constexpr (BWD)
+        if constexpr (MODE == 1) {
+            float4 gi4 = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (in && (row_bit(S.eb, lx, ly) || row_bit(S.hb, lx, ly)))
+                gi4 = __ldg(reinterpret_cast<const float4 *>(g.gin) + V.pix_off + (long long)(Y0 + ly) * V.W + (X0 + lx));
+            n_layers += adjoint_warp<K, TT>(g, S, V, M, X0, Y0, p, in, ids, gi4);
+        } else if constexpr (BWD)
             n_layers += adjoint_pixel<K, TT, EXTRA>(g, S, V, M, X0, Y0, lx, ly, ids, glacc);
         else
             n_layers += finish_forward<K, TT, EXTRA>(g, S, V, M, X0, Y0, p, in, ids, hardbits, single_chunk, l2acc);
@@ -1960,20 +1881,22 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
     }
 }
 
-// one CTA per tile.  CTAs per SM (measured best): four for the forward (64 registers),
-// for the layer-queued adjoint from stored ids (64, a few spills: more warps beat the
-// registers for its gathers; five, at 48 registers, spill too much) and for the adjoint
-// that re-rasterizes, which holds both the raster and the adjoint state (64 registers and
-// spills, but four CTAs beat three at 80 registers by 4 % on the 2048^2 views); three for
-// the instantiations with the normal map, the light gradient and the inverse UV.
+// one CTA per tile.  CTAs per SM, measured (us; 24 views of 512^2 of 20,480 faces unless said):
+//   forward                   4 (64 registers) 611, 3: 679 -- issue bound, warps beat registers
+//   adjoint from stored ids   2 (128) 375, 3: 380, 4: 409, 5: 498 -- at 64 registers it spills 400
+//                             bytes a thread, two thirds of its L1 requests
+//   re-rasterizing adjoint    3 (80) 709, 4: 748, 2: 718 (two 2048^2 views, 1.31 M faces)
+//   forward from stored ids   4: 147, 3: 164, 5: 155, 6: 161
+//   with the extras           adjoint from ids 2: 138, 3: 148; forward 4: 162, 3: 172 (normal map,
+//                             6 x 384^2); the other two as their plain forms
 template <int MODE, int TT>
 constexpr int tile_min_ctas()
 {
-    return (MODE == 4 || MODE >= 6) ? 3 : 4;
+    return (MODE == 2 || MODE == 4) ? 2 : (MODE == 1 || MODE == 5) ? 3 : 4;
 }
 
 template <int K, int MODE, int TT>
-__global__ void __launch_bounds__(NT, tile_min_ctas<MODE, TT>()) k_tile(Globals g)
+__global__ void __launch_bounds__(cta_threads<MODE, TT>(), tile_min_ctas<MODE, TT>()) k_tile(Globals g)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem &S = *reinterpret_cast<Smem *>(smem_raw);
@@ -1984,7 +1907,7 @@ __global__ void __launch_bounds__(NT, tile_min_ctas<MODE, TT>()) k_tile(Globals 
 // persistent: as many CTAs as fit on the GPU pull tiles from one queue, in the
 // order of g.tile_order (longest face list first) when it is given
 template <int K, int MODE, int TT>
-__global__ void __launch_bounds__(NT, tile_min_ctas<MODE, TT>()) k_tile_persistent(Globals g)
+__global__ void __launch_bounds__(cta_threads<MODE, TT>(), tile_min_ctas<MODE, TT>()) k_tile_persistent(Globals g)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem &S = *reinterpret_cast<Smem *>(smem_raw);
@@ -2006,18 +1929,16 @@ constexpr size_t tile_smem_bytes()
     // from stored ids: the first part of Smem; otherwise Smem, the K-lists, the
     // candidate queue, the two pair-block tables; the adjoints with extras add the
     // per-thread dL/dlight slots
-    return (MODE == 2   ? adj_smem_bytes<K>()
-            : MODE == 3 || MODE == 4 || MODE == 7
+    return (MODE == 2 || MODE == 3 || MODE == 4 || MODE == 7
                 ? offsetof(Smem, F)
-                : sizeof(Smem) + sizeof(unsigned long long) * TT * TT * K + sizeof(unsigned) * QN + 2 * NBLK) +
-           (MODE == 4 || MODE == 5 ? sizeof(float) * 3 * NT : 0);
+                : sizeof(Smem) + sizeof(unsigned long long) * TT * TT * K +
+                      sizeof(unsigned) * WQ * cta_threads<MODE, TT>() / 32 + 2 * NBLK) +
+           (MODE == 4 || MODE == 5 ? sizeof(float) * 3 * cta_threads<MODE, TT>() : 0);
 }
 // four forward CTAs of the default configuration (K = 3, 16 px tiles) per SM: 228 KB of
 // shared memory per SM, 1 KB of it reserved per CTA
 static_assert(4 * (tile_smem_bytes<3, 0, 16>() + 1024) <= 228 * 1024, "K = 3 forward tiles no longer fit four CTAs per SM");
 static_assert(4 * (tile_smem_bytes<3, 0, 32>() + 1024) <= 228 * 1024, "K = 3, 32 px forward tiles no longer fit four CTAs per SM");
-static_assert(4 * (tile_smem_bytes<3, 2, 32>() + 1024) <= 228 * 1024,
-              "K = 3 adjoint from stored ids no longer fits four CTAs per SM");
 
 constexpr int LAUNCH_MAX_DEVICES = 64;
 
@@ -2031,6 +1952,7 @@ static void launch_kk(const Globals &g, cudaStream_t s)
     static std::atomic<bool> ready[LAUNCH_MAX_DEVICES];
     static int per_sm_of[LAUNCH_MAX_DEVICES], sms_of[LAUNCH_MAX_DEVICES];
     static std::mutex mu;
+    constexpr int NT = cta_threads<MODE, TT>();
     const size_t smem = tile_smem_bytes<K, MODE, TT>();
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
