@@ -291,7 +291,7 @@ __device__ __forceinline__ void bin_walk(const Globals &g, const ViewK &V, int f
 // binning (the lists' lengths).
 // ---------------------------------------------------------------------------
 template <bool COUNT>
-__global__ void __launch_bounds__(256) k_face(Globals g)
+__global__ void __launch_bounds__(256, 4) k_face(Globals g)
 {
     // each warp's 32 records (7 float4 each) go through shared memory so that the warp
     // writes its 3,584 contiguous bytes with full-line stores
@@ -453,11 +453,25 @@ __global__ void __launch_bounds__(LPT_BINS) k_lpt_single(Globals g)
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void normal_bwd(const Globals &g, int m);
 
-// grid rows: one per view, then (normals) one per mesh for the normals' share of the positions
+// dL/dcolour from its float4 accumulator (ngrad) to the planes
+__device__ __forceinline__ void color_bwd(const Globals &g)
+{
+    const long long nvt = g.n_verts_total;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nvt; i += (long long)gridDim.x * blockDim.x) {
+        const float4 c = g.ngrad[i];
+        g.gcol[i] = c.x;
+        g.gcol[nvt + i] = c.y;
+        g.gcol[2 * nvt + i] = c.z;
+    }
+}
+
+// grid rows: one per view, then (normals) one per mesh for the normals' share of the positions, or
+// (vertex colours) one for their planes
 __global__ void k_vertex_bwd(Globals g)
 {
     if (blockIdx.y >= g.n_views) {
-        normal_bwd(g, blockIdx.y - g.n_views);
+        if (g.gcol) color_bwd(g);
+        else normal_bwd(g, blockIdx.y - g.n_views);
         return;
     }
     const ViewK &V = g.views[blockIdx.y];
@@ -555,6 +569,7 @@ __device__ __forceinline__ void normal_bwd(const Globals &g, int m)
 }
 
 __global__ void k_normal_bwd(Globals g) { normal_bwd(g, blockIdx.y); }
+__global__ void k_color_bwd(Globals g) { color_bwd(g); }
 
 // fills up to Fills::MAX ranges of 32-bit words in one launch (the adjoint's outputs and accumulators)
 __global__ void __launch_bounds__(256) k_fill(Fills f)
@@ -710,10 +725,16 @@ void launch_lpt_order(const Globals &g, cudaStream_t s)
 void launch_vertex_bwd(const Globals &g, int n_views, int max_nv, int n_meshes, int max_nf, bool normals,
                        cudaStream_t s)
 {
-    const bool merge = normals && n_views + n_meshes <= MAX_GRID_Y;
-    const dim3 grid(grid_x(std::max(max_nv, merge ? max_nf : 0), 256, 2048), n_views + (merge ? n_meshes : 0));
+    const int rows = normals ? n_meshes : g.gcol ? 1 : 0;
+    const bool merge = rows > 0 && n_views + rows <= MAX_GRID_Y;
+    const long long wide = !merge ? 0 : normals ? max_nf : g.n_verts_total;
+    const dim3 grid(grid_x(std::max<long long>(max_nv, wide), 256, 2048), n_views + (merge ? rows : 0));
     k_vertex_bwd<<<grid, 256, 0, s>>>(g);
     count_launch(1);
+    if (g.gcol && !merge) {
+        k_color_bwd<<<grid_x(g.n_verts_total, 256, 2048), 256, 0, s>>>(g);
+        count_launch(1);
+    }
     if (normals && !merge) {
         k_normal_bwd<<<dim3(grid_x(max_nf, 256, 2048), n_meshes), 256, 0, s>>>(g);
         count_launch(1);

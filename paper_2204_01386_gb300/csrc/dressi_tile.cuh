@@ -297,6 +297,11 @@ __device__ __forceinline__ void shade(const Globals &g, const ViewK &V, const Me
     S.ix[0] = wrapi(x0, M.tex_w); S.ix[1] = S.ix[0] + 1 < M.tex_w ? S.ix[0] + 1 : 0;
     S.iy[0] = wrapi(y0, M.tex_h); S.iy[1] = S.iy[0] + 1 < M.tex_h ? S.iy[0] + 1 : 0;
     const long long tb = M.tex_off;
+    if (ADJ && g.grad_prefetch) {
+        // the texel gradient's lines, wanted by the reductions at the end of this layer
+        prefetch_l2(g.gtex + 4 * (tb + (long long)S.iy[0] * M.tex_w + S.ix[0]));
+        prefetch_l2(g.gtex + 4 * (tb + (long long)S.iy[1] * M.tex_w + S.ix[0]));
+    }
     const float4 t00 = load_texel(g, tb + (long long)S.iy[0] * M.tex_w + S.ix[0]);
     const float4 t10 = load_texel(g, tb + (long long)S.iy[0] * M.tex_w + S.ix[1]);
     const float4 t01 = load_texel(g, tb + (long long)S.iy[1] * M.tex_w + S.ix[0]);
@@ -443,11 +448,12 @@ __device__ __forceinline__ bool layer_adjoint(const Globals &g, const ViewK &V, 
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
                 const long long gi = M.vert_off + S.vi[i];
+                // dL/dcolour in the normals' accumulator, which this mode does not use: one 16-byte
+                // reduction per corner instead of three 4-byte ones (16 views of 224^2, K = 5:
+                // see k_vertex_bwd, which writes the planes)
+                if (g.gcol) atomicAdd(g.ngrad + gi, make_float4(S.b[i] * gC[0], S.b[i] * gC[1], S.b[i] * gC[2], 0.f));
 #pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    if (g.gcol) atomicAdd(g.gcol + c * nvt + gi, S.b[i] * gC[c]);
-                    gb[i] = fmaf(gC[c], __ldg(g.col + c * nvt + gi), gb[i]);
-                }
+                for (int c = 0; c < 3; ++c) gb[i] = fmaf(gC[c], __ldg(g.col + c * nvt + gi), gb[i]);
             }
         } else {
             float gA[3];
