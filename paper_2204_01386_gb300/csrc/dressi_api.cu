@@ -56,7 +56,7 @@ struct Plan {
     std::vector<MeshK> meshes;
     Layout lay;
     int max_nv = 0, max_nf = 0, max_nv_view = 0, max_nf_view = 0, max_texels = 0;
-    long long n_texels = 0, n_faces = 0;
+    long long n_texels = 0, n_faces = 0, view_faces = 0, view_pixels = 0;
 };
 
 static bool check_params(const dressi_params *p)
@@ -158,6 +158,8 @@ static bool make_plan(const dressi_scene *sc, const dressi_view *views, int n_vi
         if (nt > 0x7fffffff) return false;
         tiles = (int)nt;
     }
+    P.view_faces = view_faces;
+    P.view_pixels = view_pixels;
     Layout &L = P.lay;
     L.n_vrec = vrec;
     L.total_tiles = tiles;
@@ -310,10 +312,8 @@ static void run_setup(Globals &g, const Plan &P, char *ws, bool need_bins, Clear
         clear(L.adj_off, nv + 1);
         clear(L.adj_cur, nv);
     }
-    if (g.persistent) {
-        clear(L.queue, 4);
-        clear(L.lpt_hist, LPT_BINS);
-    }
+    if (g.persistent || g.fronts == 2) clear(L.queue, 4);
+    if (g.persistent) clear(L.lpt_hist, LPT_BINS);
     // the view and mesh tables, adjacent in the workspace
     const size_t words = (L.meshes + sizeof(MeshK) * P.meshes.size()) / 4;
     std::vector<unsigned> tables(words, 0u);
@@ -338,17 +338,42 @@ static bool fronts_only(const dressi_params *p)
     return p->edge_mode != 1 && !inv_uv && p->r < 2.f;
 }
 
+// Where the front fragments come from: the face table kernel, where a face's lane visits its pixels
+// with the record at hand, if the faces are small and enough of them to fill the GPU; else the
+// tiles' own rasters.  Face table + forward tile kernel, us, from the tiles / from the face table:
+//   1,280 x 720, 81,920 faces (11 pixels per face)      6 + 108 / 14 + 63
+//   4 views of 768^2, 32,000 faces each (18)            8 + 238 / 44 + 128
+//   8 views of 512^2, 20,480 faces each (13)           11 + 296 / 38 + 164
+//   2 views of 2048^2, 1.31 M faces (3)               106 + 1094 / 165 + 554
+//   256^2, 20,480 faces (3)                             6 + 56 / 9 + 30
+//   256^2, 5,120 faces (13)                             6 + 53 / 24 + 37   (and a launch and a fill)
+//   8 views of 512^2, 5,120 faces each (51)             8 + 223 / 169 + 128
+//   8 views of 512^2, 1,280 faces each (205)           10 + 195 / 398 + 108
+constexpr long long FRONT_MIN_FACES = 16384;
+constexpr long long FRONT_MAX_PX = 24;   // view pixels per face
+
+static void choose_fronts(Globals &g, const Plan &P, bool only, char *ws, cudaStream_t s)
+{
+    g.fronts = only ? 1 : 0;
+    if (!only || P.view_faces < FRONT_MIN_FACES || P.view_pixels > FRONT_MAX_PX * P.view_faces) return;
+    g.fronts = 2;
+    g.big = reinterpret_cast<int2 *>(ws + P.lay.lists);   // before the lists are written
+    g.big_cap = (int)(P.lay.list_cap / 2);
+    g.big_n = reinterpret_cast<int *>(ws + P.lay.queue) + 1;
+    cudaMemsetAsync(ws + P.lay.kth, WORD_FILL, sizeof(unsigned long long) * (size_t)P.view_pixels, s);
+}
+
 // a forward that stores no layer ids leaves every pixel's word (K-th entry, or front layer with
 // E and S^H) in the workspace for a re-rasterizing adjoint; the flag says which, if any
-static Clears keep_kth(Globals &g, const Plan &P, const dressi_params *p, char *ws)
+static Clears keep_kth(Globals &g, const Plan &P, const dressi_params *p, char *ws, cudaStream_t s)
 {
     const bool keep = g.ids == nullptr;
-    g.fronts = keep && fronts_only(p);
     g.kth = keep ? reinterpret_cast<unsigned long long *>(ws + P.lay.kth) : nullptr;
+    choose_fronts(g, P, keep && fronts_only(p), ws, s);
     Clears clr;
     clr.p[0] = reinterpret_cast<int *>(ws + P.lay.kth_flag);
     clr.n[0] = 1;
-    clr.v[0] = keep ? (g.fronts ? KTH_FRONTS : KTH_LAST) : KTH_NONE;
+    clr.v[0] = !keep ? KTH_NONE : g.fronts ? KTH_FRONTS : KTH_LAST;
     return clr;
 }
 
@@ -485,7 +510,7 @@ int dressi_forward(const dressi_scene *scene, const dressi_view *views, int32_t 
     Globals g = make_globals(scene, params, P, w, n_pix, dev_status);
     g.out = out_rgba;
     g.ids = layer_ids;
-    run_setup(g, P, w, true, keep_kth(g, P, params, w), 1, s);
+    run_setup(g, P, w, true, keep_kth(g, P, params, w, s), 1, s);
     run_tiles(g, P, w, true, 0, s);
     return cudaGetLastError() == cudaSuccess ? DRESSI_OK : DRESSI_ERR_LAUNCH;
 }
@@ -511,7 +536,7 @@ int dressi_forward_l2(const dressi_scene *scene, const dressi_view *views, int32
     g.l2_target = target;
     g.l2_grad = grad_rgba;
     g.l2_loss = loss_accum;
-    run_setup(g, P, w, true, keep_kth(g, P, params, w), 1, s);
+    run_setup(g, P, w, true, keep_kth(g, P, params, w, s), 1, s);
     run_tiles(g, P, w, true, 0, s);
     return cudaGetLastError() == cudaSuccess ? DRESSI_OK : DRESSI_ERR_LAUNCH;
 }
@@ -626,9 +651,22 @@ int dressi_backward_ex(const dressi_scene *scene, const dressi_view *views, int3
         fill(w + P.lay.lpt_hist, LPT_BINS);
     }
     launch_fill(f, s);
-    // re-rasterizing after a forward on this workspace: its pixels' words, if it kept them
-    if (params->reuse_setup && !layer_ids) g.kth = reinterpret_cast<unsigned long long *>(w + P.lay.kth);
-    if (!params->reuse_setup) run_setup(g, P, w, layer_ids == nullptr, Clears(), 0, s);
+    const bool only = !layer_ids && fronts_only(params);
+    if (params->reuse_setup) {
+        // re-rasterizing after a forward on this workspace: its pixels' words, if it kept them
+        g.fronts = only ? 1 : 0;
+        if (!layer_ids) g.kth = reinterpret_cast<unsigned long long *>(w + P.lay.kth);
+    } else {
+        Clears clr;
+        choose_fronts(g, P, only, w, s);
+        if (g.fronts == 2) {
+            g.kth = reinterpret_cast<unsigned long long *>(w + P.lay.kth);
+            clr.p[0] = g.kth_flag;
+            clr.n[0] = 1;
+            clr.v[0] = KTH_RAW;
+        }
+        run_setup(g, P, w, layer_ids == nullptr, clr, g.fronts == 2 ? 1 : 0, s);
+    }
     run_tiles(g, P, w, layer_ids == nullptr, 1, s);
     if (gather)
         launch_tex_gather(g, P.lay.tg_slots, P.n_texels, (int)P.meshes.size(), P.max_texels, w + P.lay.tg_scratch,

@@ -32,11 +32,25 @@ constexpr float EDGE_TIE_PX = 1e-3f;
 constexpr int FLAG_RANGE = 1 << 8;
 constexpr int FLAG_ODD = 1 << 9;    // the record's corner order is an odd permutation of the face's
 
-// a pixel's word from a forward without layer ids: nothing, the K-th (key, id) of every pixel, or
-// E and S^H with the K-th (key, id) where E = 1, else the front one (keys are below 2: the two top
-// bits are free)
-constexpr int KTH_NONE = 0, KTH_LAST = 0x01010101, KTH_FRONTS = 0x02020202;
-constexpr unsigned long long KTH_SH = 1ull << 63, KTH_E = 1ull << 62, KTH_BITS = KTH_E - 1;
+// An empty K-list slot.
+constexpr unsigned long long EMPTY = ~0ULL;
+// A pixel's word in the workspace (*kth_flag says which): nothing; KTH_LAST the K-th (key, id) of every
+// pixel; KTH_RAW its front hard (key, id), WORD_NONE for none, as the face table kernel left it;
+// KTH_FRONTS the same, but E, S^H and the K-th (key, id) (all ones: none) where E = 1.  Keys of these
+// forms are below 2 (r < 2 screens): the two top bits are free.  WORD_NONE is one byte repeated
+// (it is filled in), above every hard key.
+constexpr int KTH_NONE = 0, KTH_LAST = 1, KTH_RAW = 2, KTH_FRONTS = 3;
+constexpr int WORD_FILL = 0x3f;
+constexpr unsigned long long WORD_NONE = 0x3f3f3f3f3f3f3f3full;
+constexpr unsigned long long WORD_SH = 1ull << 63, WORD_E = 1ull << 62, WORD_BITS = WORD_E - 1;
+__device__ __forceinline__ bool word_hard(unsigned long long w)   // S^H
+{
+    return (w & WORD_E) ? (w & WORD_SH) != 0 : w != WORD_NONE;
+}
+__device__ __forceinline__ bool word_tie(unsigned long long w)   // a front layer at the far plane, undecided
+{
+    return !(w & WORD_E) && w != WORD_NONE && !(__uint_as_float((unsigned)(w >> 32)) < 0.5f);
+}
 
 // ---------------------------------------------------------------------------
 // tables uploaded into the workspace
@@ -150,7 +164,11 @@ struct Globals {
     // rasterizes nothing where the mask is empty
     unsigned long long *kth;
     int *kth_flag;
-    int fronts;           // layers beyond the front one are only needed inside the edge mask
+    int fronts;           // layers beyond the front one are only needed inside the edge mask: the front
+                          // ones come 1 from the tiles' rasters, 2 from the face table kernel (in kth)
+    int2 *big;            // faces left to k_front_big (view, face), in the tile lists' place
+    int big_cap;
+    int *big_n;
     int zero_bins;        // the vertex transform clears tile_count and tile_cursor
     // forward
     float *out;
@@ -189,6 +207,12 @@ __device__ __forceinline__ bool lex_less(float axh, float axl, float ayh, float 
     if (axl != bxl) return axl < bxl;
     if (ayh != byh) return ayh < byh;
     return ayl < byl;
+}
+
+__device__ __forceinline__ unsigned long long pack_frag(float key, int id)
+{
+    const unsigned int kb = __float_as_uint(key) & 0x7fffffffu;   // keys are >= 0; folds -0 into +0
+    return ((unsigned long long)kb << 32) | (unsigned int)id;
 }
 
 __device__ __forceinline__ float fsub(float a, float b) { return __fsub_rn(a, b); }

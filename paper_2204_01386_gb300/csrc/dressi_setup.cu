@@ -285,17 +285,159 @@ __device__ __forceinline__ void bin_walk(const Globals &g, const ViewK &V, int f
 }
 
 // ---------------------------------------------------------------------------
+// front words: the front hard (key, id) of every pixel, by 64-bit atomicMin in the order of the
+// faces, for passes that need more layers only inside the edge mask.  A small face covers a few
+// pixels; visiting them from the face (a dozen pixel tests, the record at hand) replaces its
+// staging, bounding boxes and shared-memory lists in each of the tiles that its grown box touches
+// (measured on both sides of the line that chooses it: FRONT_MIN_FACES, dressi_api.cu).  A lane
+// visits a face's rows, cut to the covered interval: two 2048^2 views of 1.31 M faces 165 us with
+// the table, which alone takes 106; a warp-wide list of all box pixels took 198, and on 21-pixel
+// faces 84 instead of 44 us (its batches look up face, record and pixel for each pair).
+// ---------------------------------------------------------------------------
+constexpr int FRONT_LANE = 512;   // pixels of a bounding box that its face's lane visits alone
+constexpr int FRONT_BIG = 4096;   // pixels of a bounding box left to k_front_big
+
+// the pixel centres inside the face's bounding box (grown by a margin over the corners' low parts)
+__device__ __forceinline__ bool front_rect(const ViewK &V, const FaceGeo &R, int &x0, int &y0, int &w, int &h)
+{
+    const float M = 0.01f;
+    x0 = max(0, (int)ceilf(fminf(R.c[0].xh, fminf(R.c[1].xh, R.c[2].xh)) - 0.5f - M));
+    y0 = max(0, (int)ceilf(fminf(R.c[0].yh, fminf(R.c[1].yh, R.c[2].yh)) - 0.5f - M));
+    w = min(V.W - 1, (int)floorf(fmaxf(R.c[0].xh, fmaxf(R.c[1].xh, R.c[2].xh)) - 0.5f + M)) - x0 + 1;
+    h = min(V.H - 1, (int)floorf(fmaxf(R.c[0].yh, fmaxf(R.c[1].yh, R.c[2].yh)) - 0.5f + M)) - y0 + 1;
+    return w > 0 && h > 0;
+}
+
+__device__ __forceinline__ void front_pixel(const ViewK &V, const FaceGeo &R, int f, int x, int y, unsigned long long *words)
+{
+    Frag fr;
+    if (eval_face<false>(R, (float)x + 0.5f, (float)y + 0.5f, 0.f, V.half_inv_S, fr, true))
+        atomicMin(words + (long long)y * V.W + x, pack_frag(fr.key, f));
+}
+
+// a face's pixels by its own lane: each row of the box cut to where the three cross products, linear
+// along the row, are above -FRONT_SLACK px (a division-free half-plane per edge), and the pixels
+// left tested exactly.  Where the crosses' rounding could reach the slack (corners far outside
+// the box, or an edge far shorter than the face), the whole rows are tested.
+constexpr float FRONT_SLACK = 2e-3f;
+
+__device__ __forceinline__ void front_lane(const ViewK &V, const FaceGeo &R, int f, int x0, int y0, int w, int h,
+                                           unsigned long long *words)
+{
+    float dx[3], slope[3], inv[3], eps[3], sgn[3];
+    float ext = (float)h, sharp = 0.f;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        dx[i] = ((float)x0 + 0.5f - R.c[i].xh) - R.c[i].xl;
+        ext = fmaxf(ext, fmaxf(fabsf(dx[i]), fabsf((float)y0 + 0.5f - R.c[i].yh) + (float)h));
+        sharp = fmaxf(sharp, fabsf(R.invL[i]));
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int P = i == 2 ? 0 : i, Q = i == 2 ? 2 : i + 1;
+        sgn[i] = R.invL[i] > 0.f ? 1.f : -1.f;
+        // d cross / d x = dy_Q - dy_P; a level edge keeps or drops a whole row
+        const float sl = sgn[i] * ((R.c[P].yh - R.c[Q].yh) + (R.c[P].yl - R.c[Q].yl));
+        slope[i] = fabsf(sl) < 1e-9f ? 1e-9f : sl;
+        inv[i] = __fdividef(1.f, slope[i]);
+        eps[i] = __fdividef(FRONT_SLACK, fabsf(R.invL[i]));
+    }
+    const bool cut = 1.2e-7f * ext * ext * sharp <= 0.5f * FRONT_SLACK;
+    for (int y = y0; y < y0 + h; ++y) {
+        float lo = 0.f, hi = (float)(w - 1);
+        if (cut) {
+            float dy[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) dy[i] = ((float)y + 0.5f - R.c[i].yh) - R.c[i].yl;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const int P = i == 2 ? 0 : i, Q = i == 2 ? 2 : i + 1;
+                const float c = sgn[i] * (dx[P] * dy[Q] - dy[P] * dx[Q]);
+                const float t = -(c + eps[i]) * inv[i];
+                if (slope[i] > 0.f) lo = fmaxf(lo, t);
+                else hi = fminf(hi, t);
+            }
+        }
+        if (!(lo <= hi)) continue;
+        const int k1 = (int)floorf(hi);
+        for (int k = (int)ceilf(lo); k <= k1; ++k) front_pixel(V, R, f, x0 + k, y, words);
+    }
+}
+
+// the larger of the warp's 32 staged faces (stride 7 float4; c: box pixels of this lane's face f, 0 for none): their
+// pixels as one list, 32 at a time with full lanes.  A list entry's face is found by the bits of
+// the faces that start in its batch.
+__device__ __forceinline__ void front_warp(const ViewK &V, const float4 *recs, int f0, int c, int x0, int y0, int w,
+                                           unsigned long long *words, int2 *slot)
+{
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    int incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += v;
+    }
+    const int total = __shfl_sync(FULL, incl, 31), first = incl - c;
+    const unsigned some = __ballot_sync(FULL, c > 0);
+    // the faces with pixels packed to the front: first | lane, and the box
+    const int rank = __popc(some & ((1u << lane) - 1u));
+    if (c > 0) slot[rank] = make_int2(first, lane);
+    __syncwarp();
+    int nb = -1;
+    for (int b0 = 0; b0 < total; b0 += 32) {
+        const unsigned starts = __reduce_or_sync(FULL, (c > 0 && (unsigned)(first - b0) < 32u) ? 1u << (first - b0) : 0u);
+        const int idx = nb + __popc(starts & (0xffffffffu >> (31 - lane)));
+        nb += __popc(starts);
+        const int2 e = slot[max(idx, 0)];
+        const int fx = __shfl_sync(FULL, x0, e.y), fy = __shfl_sync(FULL, y0, e.y), fw = __shfl_sync(FULL, w, e.y);
+        if (b0 + lane < total) {
+            const int k = b0 + lane - e.x;
+            // k / w: both are small integers, the quotient of the floats is off by at most one
+            int q = (int)__fdividef((float)k + 0.5f, (float)fw);
+            int r = k - q * fw;
+            if (r < 0) { --q; r += fw; }
+            else if (r >= fw) { ++q; r -= fw; }
+            front_pixel(V, *reinterpret_cast<const FaceGeo *>(recs + e.y * 7), f0 + e.y, fx + r, fy + q, words);
+        }
+    }
+    __syncwarp();
+}
+
+// the faces with larger boxes, from the list that k_face left: a warp takes a band of a face's rows
+__global__ void __launch_bounds__(256) k_front_big(Globals g)
+{
+    const int n = min(*g.big_n, g.big_cap);
+    if (n == 0) return;
+    const int warps = gridDim.x * (blockDim.x >> 5), lane = threadIdx.x & 31;
+    const int bands = max(1, min(64, warps / n));
+    for (long long it = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < (long long)n * bands; it += warps) {
+        const int2 e = g.big[it / bands];
+        const int band = (int)(it % bands);
+        const ViewK &V = g.views[e.x];
+        const FaceGeo &R = *reinterpret_cast<const FaceGeo *>(g.frec + V.frec_off + e.y);
+        int x0, y0, w, h;
+        if (!front_rect(V, R, x0, y0, w, h)) continue;
+        const int r0 = (int)((long long)h * band / bands), r1 = (int)((long long)h * (band + 1) / bands);
+        for (int y = y0 + r0; y < y0 + r1; ++y)
+            for (int x = x0 + lane; x < x0 + w; x += 32) front_pixel(V, R, e.y, x, y, g.kth + V.slot_base);
+    }
+}
+
+// ---------------------------------------------------------------------------
 // face table: the record of every (view, face) -- screen corners, canonical edges,
 // lengths, area, flags -- built once per call and read by binning, staging,
 // shading and the adjoint (112 bytes each).  COUNT: also the tile counts of the
 // binning (the lists' lengths).
 // ---------------------------------------------------------------------------
-template <bool COUNT>
-__global__ void __launch_bounds__(256, 4) k_face(Globals g)
+// FRONT: also the front words of the faces' pixels.
+template <bool COUNT, bool FRONT>
+__global__ void __launch_bounds__(256, FRONT ? 3 : 4) k_face(Globals g)
 {
     // each warp's 32 records (7 float4 each) go through shared memory so that the warp
     // writes its 3,584 contiguous bytes with full-line stores
     __shared__ float4 stage[256 / 32][32 * 7];
+    __shared__ int2 slots[FRONT ? 256 : 1];
     if (blockIdx.y >= g.n_views) {
         adjacency<0>(g, blockIdx.y - g.n_views);
         return;
@@ -335,6 +477,29 @@ __global__ void __launch_bounds__(256, 4) k_face(Globals g)
             const int nrec = max(0, min(32, M.nF - wf0));
             float4 *dst = reinterpret_cast<float4 *>(g.frec + V.frec_off + wf0);
             for (int i = lane; i < nrec * 7; i += 32) dst[i] = ws[i];
+        }
+        if (FRONT) {
+            int x0 = 0, y0 = 0, w = 0, h = 0, c = 0;
+            if (live && front_rect(V, R, x0, y0, w, h)) {
+                c = w * h;
+                if (c <= FRONT_LANE) {
+                    c = 0;
+                    front_lane(V, R, f, x0, y0, w, h, g.kth + V.slot_base);
+                } else if ((long long)w * h > FRONT_BIG) {
+                    const int q = atomicAdd(g.big_n, 1);
+                    if (q < g.big_cap) {
+                        g.big[q] = make_int2(blockIdx.y, f);
+                        c = 0;
+                    } else {
+                        // no room: here after all, row by row
+                        c = 0;
+                        for (int y = y0; y < y0 + h; ++y)
+                            for (int x = x0; x < x0 + w; ++x) front_pixel(V, R, f, x, y, g.kth + V.slot_base);
+                    }
+                }
+            }
+            if (__any_sync(0xffffffffu, c > 0))
+                front_warp(V, ws, f0 + (threadIdx.x & ~31), c, x0, y0, w, g.kth + V.slot_base, slots + (threadIdx.x & ~31));
         }
         __syncwarp();   // the staged records are read before the next iteration writes them
         if (COUNT) {
@@ -666,9 +831,14 @@ void launch_faces(const Globals &g, int n_views, int n_meshes, int max_nf_view, 
     const bool merge = normals && n_views + n_meshes <= MAX_GRID_Y;
     const dim3 grid(grid_x(std::max(max_nf_view, merge ? max_nf : 0), 256, 2048), n_views + (merge ? n_meshes : 0));
     const dim3 grid_m(grid_x(max_nf, 256, 2048), n_meshes);
-    if (lists) k_face<true><<<grid, 256, 0, s>>>(g);
-    else k_face<false><<<grid, 256, 0, s>>>(g);
+    if (lists && g.fronts == 2) k_face<true, true><<<grid, 256, 0, s>>>(g);
+    else if (lists) k_face<true, false><<<grid, 256, 0, s>>>(g);
+    else k_face<false, false><<<grid, 256, 0, s>>>(g);
     count_launch(1);
+    if (lists && g.fronts == 2) {
+        k_front_big<<<152 * 4, 256, 0, s>>>(g);   // before the tile lists are written
+        count_launch(1);
+    }
     if (normals && !merge) {
         k_adjacency<0><<<grid_m, 256, 0, s>>>(g);
         count_launch(1);

@@ -51,7 +51,6 @@ constexpr int HS_MAX = TT_MAX + 2 * RHO_MAX;
 constexpr float APPROX_EPS = 1e-3f;    // pixel slack of the tile-local (approximate) edge equations
 constexpr int CH = 128;                // faces staged per round (one per thread)
 constexpr int HASH = 256;              // face id -> staged slot, open addressing (2 CH: at most half full)
-constexpr unsigned long long EMPTY = ~0ULL;
 constexpr int WQ = 160;                // a warp's queue of pretested pairs (31 waiting + 32 items x 4)
 constexpr int NBLK = 1024;             // pair blocks of 32 with a table entry (32,768 items)
 // the raster's passes (tile_body)
@@ -713,12 +712,6 @@ struct Smem {
     int wsum[2][NT_MAX / 32];
 };
 
-__device__ __forceinline__ unsigned long long pack_frag(float key, int id)
-{
-    const unsigned int kb = __float_as_uint(key) & 0x7fffffffu;   // keys are >= 0; folds -0 into +0
-    return ((unsigned long long)kb << 32) | (unsigned int)id;
-}
-
 // The K-list slots of tile pixel (x, y) start at kbuf + kslot(x, y) K.  Each row is rotated
 // by 5 y columns: with K = 3 (24-byte slot groups) the 8-byte bank pair of a pixel's group
 // is then 3 x + 15 y mod 16, so both access patterns of the raster spread over the banks --
@@ -848,6 +841,35 @@ __device__ __forceinline__ bool halo_from_ids(const Globals &g, Smem &S, const V
         if (lane == 0) { S.m0[row] = b0; S.m1[row] = b1; }
     }
     return any;
+}
+
+// halo_rows from the face table kernel's words: S^H of the tile and of its ring is whether a hard
+// fragment covers the pixel.  (A forward's neighbour tiles may meanwhile give their edge-masked
+// pixels' words the K-th entry: word_hard is the same before and after.)  Bit 0 of the result: this thread saw one in the tile or its ring;
+// bit 1: one of the tile at key 1/2 or more (the far plane, where a soft one could tie).
+template <int TT, int NT>
+__device__ __forceinline__ int halo_from_words(const Globals &g, Smem &S, const ViewK &V, int X0, int Y0, int rho)
+{
+    const int hs = TT + 2 * rho, lane = threadIdx.x & 31;
+    int got = 0;
+    for (int row = threadIdx.x >> 5; row < hs; row += NT / 32) {
+        const int Y = Y0 - rho + row;
+        unsigned long long b0 = 0ull, b1 = 0ull;
+#pragma unroll
+        for (int h = 0; h < (TT + 2 * RHO_MAX > 32 ? 2 : 1); ++h) {
+            const int col = lane + 32 * h, X = X0 - rho + col;
+            const bool here = col < hs && X >= 0 && Y >= 0 && X < V.W && Y < V.H;
+            unsigned long long w = WORD_NONE;
+            if (here) w = g.kth[V.slot_base + (long long)Y * V.W + X];
+            const bool sh = word_hard(w);
+            if (sh) got |= 1;
+            if (word_tie(w) && row >= rho && row < TT + rho && col >= rho && col < TT + rho) got |= 2;
+            b0 |= (unsigned long long)__ballot_sync(0xffffffffu, here && !sh) << (32 * h);
+            b1 |= (unsigned long long)__ballot_sync(0xffffffffu, here && sh) << (32 * h);
+        }
+        if (lane == 0) { S.m0[row] = b0; S.m1[row] = b1; }
+    }
+    return got;
 }
 
 // per halo row, the columns holding S^H = 0 and S^H = 1 (hs <= 48 fits 64 bits)
@@ -1468,14 +1490,13 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
     bool single_chunk = false;
     bool empty = false;   // a forward over a tile that no face reaches
     bool handed = false;  // E, S^H and the front layers come from the forward's words
+    bool raw = false;     // the front layers come from the face table kernel's words
     unsigned n_pairs = 0, n_exact = 0, n_cand = 0, n_layers = 0;
     float l2acc = 0.f;   // the fused L2 loss: this thread's sum of squares
     if (!from_ids) {
-        for (int row = tid >> 5; row < hs; row += NT / 32)
-            for (int col = tid & 31; col < hs; col += 32) {
-                const int hx = X0 - rho + col, hy = Y0 - rho + row;
-                S.sh[row * hs + col] = (hx >= 0 && hy >= 0 && hx < V.W && hy < V.H) ? 0 : 2;
-            }
+        // what a front pass or the forward left in the workspace
+        const int words = BWD && g.kth ? *g.kth_flag : KTH_NONE;
+        raw = BWD ? words == KTH_RAW : g.fronts == 2;
         const long long lb = g.tile_off[t], le = g.tile_off[t + 1];
         const bool fallback = le > g.list_cap;
         const int n = fallback ? M.nF : (int)(le - lb);
@@ -1485,39 +1506,69 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
         // a forward over such a tile has no layer and S^H = 0 in the tile and its ring (no
         // face comes within the binning radius), so E = 0 or no layer to blend: background
         empty = n == 0;
-        // what the forward left in the workspace for a re-rasterizing adjoint
-        const int words = BWD && g.kth ? *g.kth_flag : 0;
-        handed = words == KTH_FRONTS;
         bool layered = !g.fronts;   // the K layers of every pixel are wanted
         int stage = g.fronts ? ST_FRONT : ST_LAYERS;
-        if (!empty)   // 16-byte stores (TT^2 K is even; kbuf is 16-byte aligned)
+        if (BWD && words == KTH_FRONTS) {
+            // E, S^H and the front layers as the forward found them
+            int got = 0;
+#pragma unroll
+            for (int j = 0; j < PPT; ++j) {
+                const int p = tid + j * NT, lx = p % TT, ly = p / TT;
+                unsigned long long w = WORD_NONE;
+                if (lx < wlim && ly < hlim) w = g.kth[V.slot_base + (long long)(Y0 + ly) * V.W + (X0 + lx)];
+                const bool E = (w & WORD_E) != 0, SH = word_hard(w);
+                row_masks<TT>(S.eb, p, E);
+                row_masks<TT>(S.hb, p, SH);
+                row_masks<TT>(S.rm, p, E);
+                got |= (E || SH ? 1 : 0) | (E ? 2 : 0) | (word_tie(w) ? 4 : 0);
+            }
+            // only front layers outside the edge mask, and nothing at all: done
+            if (!__syncthreads_or(got)) return;
+            handed = !__syncthreads_or(got & 4);   // a tile with far-plane ties is decided again
+            if (handed) stage = __syncthreads_or(got & 2) ? ST_LAYERS : ST_DONE;
+            else if (tid < TT_MAX) S.rm[tid] = 0xffffffffu;
+        } else if (tid < TT_MAX) {
+            S.rm[tid] = 0xffffffffu;
+        }
+        if (!raw && !handed)
+            for (int row = tid >> 5; row < hs; row += NT / 32)
+                for (int col = tid & 31; col < hs; col += 32) {
+                    const int hx = X0 - rho + col, hy = Y0 - rho + row;
+                    S.sh[row * hs + col] = (hx >= 0 && hy >= 0 && hx < V.W && hy < V.H) ? 0 : 2;
+                }
+        if (raw && !empty) {
+            const int got = halo_from_words<TT, NT>(g, S, V, X0, Y0, rho);
+            // no hard fragment near: S^H = 0 and E = 0 (or nothing to blend), the background
+            if (!__syncthreads_or(got)) {
+                if (BWD) return;
+                empty = true;
+            } else if (__syncthreads_or(got & 2)) {
+                layered = true;
+                stage = ST_LAYERS;
+                for (int row = tid >> 5; row < hs; row += NT / 32)
+                    for (int col = tid & 31; col < hs; col += 32)
+                        S.sh[row * hs + col] = (S.m1[row] >> col & 1ull) ? 1 : (S.m0[row] >> col & 1ull) ? 0 : 2;
+            } else {
+                edge_rows<TT>(g, S, rho, wlim, hlim);
+                const bool any = tid < TT && S.eb[tid] != 0u;
+                stage = __syncthreads_or(any) ? ST_LAYERS : ST_DONE;
+                if (tid < TT) S.rm[tid] = S.eb[tid];
+                __syncthreads();
+            }
+        }
+        if (!empty && stage != ST_DONE)   // 16-byte stores (TT^2 K is even; kbuf is 16-byte aligned)
             for (int i = tid; i < TT * TT * K / 2; i += NT)
                 reinterpret_cast<ulonglong2 *>(kbuf)[i] = make_ulonglong2(EMPTY, EMPTY);
-        if (tid < TT_MAX) S.rm[tid] = 0xffffffffu;
-        if (handed) {
-            bool any = false, some = false;
+        if (handed && stage != ST_DONE) {
+            // an edge-masked pixel's K-th entry seeds its list (see KTH_LAST below)
             __syncthreads();   // after the clearing stores
 #pragma unroll
             for (int j = 0; j < PPT; ++j) {
                 const int p = tid + j * NT, lx = p % TT, ly = p / TT;
-                bool E = false, SH = false;
-                if (lx < wlim && ly < hlim) {
-                    const unsigned long long w = g.kth[V.slot_base + (long long)(Y0 + ly) * V.W + (X0 + lx)];
-                    E = (w & KTH_E) != 0;
-                    SH = (w & KTH_SH) != 0;
-                    const unsigned long long v = w & KTH_BITS;
-                    // an edge-masked pixel's K-th entry seeds its list; else the front layer
-                    if (v != KTH_BITS) kbuf[kslot<TT>(lx, ly) * K + (E ? K - 1 : 0)] = v;
-                }
-                row_masks<TT>(S.eb, p, E);
-                row_masks<TT>(S.hb, p, SH);
-                row_masks<TT>(S.rm, p, E);
-                any |= E;
-                some |= E || SH;
+                if (!row_bit(S.eb, lx, ly)) continue;
+                const unsigned long long w = g.kth[V.slot_base + (long long)(Y0 + ly) * V.W + (X0 + lx)] & WORD_BITS;
+                if (w != WORD_BITS) kbuf[kslot<TT>(lx, ly) * K + K - 1] = w;
             }
-            // only front layers outside the edge mask, and nothing at all: done
-            if (!__syncthreads_or(some)) return;
-            stage = __syncthreads_or(any) ? ST_LAYERS : ST_DONE;
         } else if (words == KTH_LAST) {
             // the forward's K-th (key, id) of every pixel as a first entry of its K-list: it
             // is the K-th smallest of the pixel's candidates, so it stays in the last slot and
@@ -1541,8 +1592,8 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
         // 2048^2 views of a 1.31 M-face mesh 127 -> 45 M pairs and 53 -> 8 M exact evaluations, the
         // forward 1667 -> 1130 us, the adjoint 1541 -> 764 us (four 768^2 views of 32,000 faces:
         // 310 -> 244 and 350 -> 217 us).
-        bool ring = rho > 0 && !handed;
-        single_chunk = n <= CH;
+        bool ring = rho > 0 && !handed && !raw;
+        single_chunk = n <= CH && stage != ST_DONE;   // all of the list staged (and hashed) at once
         // the id -> slot hash serves the forward's shading of a tile staged in one chunk
         const bool use_hash = !BWD && single_chunk;
         while (stage != ST_DONE && !empty) {
@@ -1709,7 +1760,7 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
             }
         }
         // S^H of the tile's own pixels from the front slot
-        if (layered && !handed) {
+        if (layered) {
 #pragma unroll
             for (int j = 0; j < PPT; ++j) {
                 const int p = tid + j * NT;
@@ -1728,7 +1779,7 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
             }
         }
         // a forward without layer ids leaves each pixel's word for a re-rasterizing adjoint
-        if (!BWD && g.kth && !empty) {
+        if (!BWD && g.kth && !empty && !(raw && layered)) {
 #pragma unroll
             for (int j = 0; j < PPT; ++j) {
                 const int p = tid + j * NT, lx = p % TT, ly = p / TT;
@@ -1737,8 +1788,8 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
                 unsigned long long w = slots[K - 1];
                 if (g.fronts) {
                     const bool E = row_bit(S.eb, lx, ly), SH = row_bit(S.hb, lx, ly);
-                    w = (E ? w : SH ? slots[0] : EMPTY) & KTH_BITS;
-                    w |= (E ? KTH_E : 0ull) | (SH ? KTH_SH : 0ull);
+                    if (raw && !E) continue;   // the front word is there
+                    w = E ? (w & WORD_BITS) | WORD_E | (SH ? WORD_SH : 0ull) : SH ? slots[0] : WORD_NONE;
                 }
                 g.kth[V.slot_base + (long long)(Y0 + ly) * V.W + (X0 + lx)] = w;
             }
@@ -1822,9 +1873,13 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
         if (!in) {
         } else if (!from_ids) {
             const int ks = kslot<TT>(lx, ly) * K;
+            // the front layer of a pixel outside the edge mask, where the tile did not raster it
+            const bool front = (raw || handed) && !row_bit(S.rm, lx, ly);
+            unsigned long long word = EMPTY;
+            if (front && row_bit(S.hb, lx, ly)) word = g.kth[V.slot_base + (long long)(Y0 + ly) * V.W + (X0 + lx)];
 #pragma unroll
             for (int k = 0; k < K; ++k) {
-                const unsigned long long v = kbuf[ks + k];
+                const unsigned long long v = front ? (k == 0 ? word : EMPTY) : kbuf[ks + k];
                 ids[k] = (v == EMPTY) ? 0x7fffffff : (int)(unsigned int)(v & 0xffffffffu);
             }
             if (!BWD && g.ids) {

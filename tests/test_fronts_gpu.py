@@ -71,3 +71,23 @@ def test_far_plane_ties_without_ids(tile):
         m = pixel_mesh(v, [f[i] for i in order], W, H, z=1.0, col=np.random.default_rng(1).random((6, 3)).astype(np.float32))
         s = pixel_scene(m, W, H, K=3, r=2.0 / W, sigma=0.3 / W, delta=2.0 / W, shade_mode=0)
         _check(s, tile, 1)
+
+
+@pytest.mark.parametrize("tile,schedule", [(16, 1), (32, 2)])
+@pytest.mark.parametrize("K,edge", [(1, 0), (3, 0), (3, 2)])
+@pytest.mark.parametrize("W,H", [(257, 193), (1040, 611)])
+def test_fronts_from_the_face_table(tile, schedule, K, edge, W, H):
+    """Scenes of 32,768 faces and more, small ones beside some that fill the view (their boxes are
+    above and below the size that gets warps of its own)."""
+    pos, f = synth.icosphere(6)
+    g = np.random.default_rng(5)
+    big = np.array([[-3, -2, -3], [3, -2, -3], [0, 3, -3], [-0.3, 0.2, 1.3], [0.3, 0.1, 1.3], [0.1, 0.6, 1.2],
+                    [-0.05, -0.3, 1.4], [0.05, -0.33, 1.4], [0.0, -0.2, 1.4]], np.float64)
+    n = pos.shape[0]
+    m = synth.Mesh(np.concatenate([synth.displace(pos, 0.1, 3), big]).astype(np.float32),
+                   np.concatenate([f, [[n, n + 1, n + 2], [n + 3, n + 4, n + 5], [n + 6, n + 7, n + 8]]]).astype(np.int32),
+                   col=g.random((n + 9, 3)).astype(np.float32))
+    r = 2.0 / max(W, H)
+    views = [synth.View(synth.camera_mvp(e, W, H), 0, W, H) for e in ((0, 0, 3), (0.5, 0.4, 2.9))]
+    s = synth.Scene("front_words", [m], views, synth.Params(K=K, r=r, sigma=r / 7, delta=r, edge_mode=edge))
+    _check(s, tile, schedule)
