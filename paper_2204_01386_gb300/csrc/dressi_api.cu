@@ -216,6 +216,7 @@ static bool make_plan(const dressi_scene *sc, const dressi_view *views, int n_vi
 // ---------------------------------------------------------------------------
 __global__ void k_upload(const __grid_constant__ Tables<TABLE_WORDS> b, unsigned int *dst)
 {
+    grid_wait();
     for (int i = threadIdx.x; i < b.n; i += blockDim.x) dst[i] = b.w[i];
 }
 
@@ -227,7 +228,7 @@ static void upload(const unsigned int *w, size_t words, unsigned int *d, cudaStr
         const size_t n = std::min<size_t>(words, TABLE_WORDS);
         b.n = (int)n;
         std::memcpy(b.w, w, n * 4);
-        k_upload<<<1, 256, 0, s>>>(b, d);
+        launch(k_upload, 1, 256, 0, s, b, d);
         count_launch(1);
         w += n;
         d += n;

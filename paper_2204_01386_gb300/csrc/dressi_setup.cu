@@ -76,6 +76,7 @@ __device__ __forceinline__ DF df_recip(DF w)
 template <int TABLES>
 __global__ void k_vertex(Globals g, const __grid_constant__ Tables<TABLES> tab, Clears clr)
 {
+    grid_wait();
     const ViewK *views = g.views;
     const MeshK *meshes = g.meshes;
     const int nthreads = gridDim.x * gridDim.y * blockDim.x;
@@ -172,11 +173,13 @@ __device__ __forceinline__ void adjacency(const Globals &g, int m)
 template <int PASS>
 __global__ void k_adjacency(Globals g)
 {
+    grid_wait();
     adjacency<PASS>(g, blockIdx.y);
 }
 
 __global__ void k_normal_csr(Globals g)
 {
+    grid_wait();
     const MeshK &M = g.meshes[blockIdx.y];
     const long long nvt = g.n_verts_total;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < M.nV; i += gridDim.x * blockDim.x) {
@@ -407,6 +410,7 @@ __device__ __forceinline__ void front_warp(const ViewK &V, const float4 *recs, i
 // the faces with larger boxes, from the list that k_face left: a warp takes a band of a face's rows
 __global__ void __launch_bounds__(256) k_front_big(Globals g)
 {
+    grid_wait();
     const int n = min(*g.big_n, g.big_cap);
     if (n == 0) return;
     const int warps = gridDim.x * (blockDim.x >> 5), lane = threadIdx.x & 31;
@@ -434,6 +438,7 @@ __global__ void __launch_bounds__(256) k_front_big(Globals g)
 template <bool COUNT, bool FRONT>
 __global__ void __launch_bounds__(256, FRONT ? 3 : 4) k_face(Globals g)
 {
+    grid_wait();
     // each warp's 32 records (7 float4 each) go through shared memory so that the warp
     // writes its 3,584 contiguous bytes with full-line stores
     __shared__ float4 stage[256 / 32][32 * 7];
@@ -516,6 +521,7 @@ __global__ void __launch_bounds__(256, FRONT ? 3 : 4) k_face(Globals g)
 // each face's tile rect comes packed from the face table kernel
 __global__ void k_bin(Globals g)
 {
+    grid_wait();
     if (blockIdx.y >= g.n_views) {
         adjacency<1>(g, blockIdx.y - g.n_views);
         return;
@@ -549,12 +555,14 @@ __device__ __forceinline__ int lpt_bin(int count) { return LPT_BINS - 1 - min(co
 
 __global__ void k_lpt_hist(Globals g)
 {
+    grid_wait();
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.total_tiles; t += gridDim.x * blockDim.x)
         atomicAdd(g.lpt_hist + lpt_bin(g.tile_count[t]), 1);
 }
 
 __global__ void __launch_bounds__(LPT_BINS) k_lpt_scan(Globals g)
 {
+    grid_wait();
     __shared__ int warp_sums[LPT_BINS / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int v = g.lpt_hist[tid];
@@ -581,6 +589,7 @@ __global__ void __launch_bounds__(LPT_BINS) k_lpt_scan(Globals g)
 
 __global__ void k_lpt_scatter(Globals g)
 {
+    grid_wait();
     int *order = const_cast<int *>(g.tile_order);
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.total_tiles; t += gridDim.x * blockDim.x)
         order[atomicAdd(g.lpt_hist + lpt_bin(g.tile_count[t]), 1)] = t;
@@ -589,6 +598,7 @@ __global__ void k_lpt_scatter(Globals g)
 // the same order in one block (a launch instead of three): the histogram in shared memory
 __global__ void __launch_bounds__(LPT_BINS) k_lpt_single(Globals g)
 {
+    grid_wait();
     __shared__ int hist[LPT_BINS];
     __shared__ int warp_sums[LPT_BINS / 32];
     int *order = const_cast<int *>(g.tile_order);
@@ -634,6 +644,7 @@ __device__ __forceinline__ void color_bwd(const Globals &g)
 // (vertex colours) one for their planes
 __global__ void k_vertex_bwd(Globals g)
 {
+    grid_wait();
     if (blockIdx.y >= g.n_views) {
         if (g.gcol) color_bwd(g);
         else normal_bwd(g, blockIdx.y - g.n_views);
@@ -733,12 +744,13 @@ __device__ __forceinline__ void normal_bwd(const Globals &g, int m)
     }
 }
 
-__global__ void k_normal_bwd(Globals g) { normal_bwd(g, blockIdx.y); }
-__global__ void k_color_bwd(Globals g) { color_bwd(g); }
+__global__ void k_normal_bwd(Globals g) { grid_wait(); normal_bwd(g, blockIdx.y); }
+__global__ void k_color_bwd(Globals g) { grid_wait(); color_bwd(g); }
 
 // fills up to Fills::MAX ranges of 32-bit words in one launch (the adjoint's outputs and accumulators)
 __global__ void __launch_bounds__(256) k_fill(Fills f)
 {
+    grid_wait();
     const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
 #pragma unroll
     for (int q = 0; q < Fills::MAX; ++q) {
@@ -758,6 +770,7 @@ __global__ void __launch_bounds__(256) k_fill(Fills f)
 // L2 loss helper
 __global__ void k_l2(const float *out, const float *tgt, long long n, float *grad, float *loss)
 {
+    grid_wait();
     float acc = 0.f;
     const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -806,7 +819,7 @@ static void launch_vertex_t(const Globals &g, dim3 grid, const unsigned *tables,
     Tables<TABLES> t;
     t.n = words;
     if (TABLES) std::memcpy(t.w, tables, sizeof(unsigned) * words);
-    k_vertex<TABLES><<<grid, 256, 0, s>>>(g, t, clr);
+    launch(k_vertex<TABLES>, grid, 256, 0, s, g, t, clr);
     count_launch(1);
 }
 
@@ -831,16 +844,16 @@ void launch_faces(const Globals &g, int n_views, int n_meshes, int max_nf_view, 
     const bool merge = normals && n_views + n_meshes <= MAX_GRID_Y;
     const dim3 grid(grid_x(std::max(max_nf_view, merge ? max_nf : 0), 256, 2048), n_views + (merge ? n_meshes : 0));
     const dim3 grid_m(grid_x(max_nf, 256, 2048), n_meshes);
-    if (lists && g.fronts == 2) k_face<true, true><<<grid, 256, 0, s>>>(g);
-    else if (lists) k_face<true, false><<<grid, 256, 0, s>>>(g);
-    else k_face<false, false><<<grid, 256, 0, s>>>(g);
+    if (lists && g.fronts == 2) launch(k_face<true, true>, grid, 256, 0, s, g);
+    else if (lists) launch(k_face<true, false>, grid, 256, 0, s, g);
+    else launch(k_face<false, false>, grid, 256, 0, s, g);
     count_launch(1);
     if (lists && g.fronts == 2) {
-        k_front_big<<<152 * 4, 256, 0, s>>>(g);   // before the tile lists are written
+        launch(k_front_big, 152 * 4, 256, 0, s, g);   // before the tile lists are written
         count_launch(1);
     }
     if (normals && !merge) {
-        k_adjacency<0><<<grid_m, 256, 0, s>>>(g);
+        launch(k_adjacency<0>, grid_m, 256, 0, s, g);
         count_launch(1);
     }
     // exclusive prefixes: tile_off[n] = total list entries
@@ -853,15 +866,15 @@ void launch_faces(const Globals &g, int n_views, int n_meshes, int max_nf_view, 
     }
     if (nj) launch_scans(jobs, nj, s);
     if (lists) {
-        k_bin<<<grid, 256, 0, s>>>(g);
+        launch(k_bin, grid, 256, 0, s, g);
         count_launch(1);
     }
     if (normals && !(lists && merge)) {
-        k_adjacency<1><<<grid_m, 256, 0, s>>>(g);
+        launch(k_adjacency<1>, grid_m, 256, 0, s, g);
         count_launch(1);
     }
     if (normals) {
-        k_normal_csr<<<dim3(grid_x(max_nv, 256, 2048), n_meshes), 256, 0, s>>>(g);
+        launch(k_normal_csr, dim3(grid_x(max_nv, 256, 2048), n_meshes), 256, 0, s, g);
         count_launch(1);
     }
 }
@@ -871,7 +884,7 @@ void launch_fill(const Fills &f, cudaStream_t s)
     long long words = 0;
     for (int q = 0; q < Fills::MAX; ++q) words = std::max(words, f.n[q]);
     if (words == 0) return;
-    k_fill<<<grid_x(words / 4 + 1, 256, 152 * 16), 256, 0, s>>>(f);
+    launch(k_fill, grid_x(words / 4 + 1, 256, 152 * 16), 256, 0, s, f);
     count_launch(1);
 }
 
@@ -881,14 +894,14 @@ constexpr int LPT_SINGLE = 16 * LPT_BINS;
 void launch_lpt_order(const Globals &g, cudaStream_t s)
 {
     if (g.total_tiles <= LPT_SINGLE) {
-        k_lpt_single<<<1, LPT_BINS, 0, s>>>(g);
+        launch(k_lpt_single, 1, LPT_BINS, 0, s, g);
         count_launch(1);
         return;
     }
     const int grid = grid_x(g.total_tiles, 256, 1024);
-    k_lpt_hist<<<grid, 256, 0, s>>>(g);
-    k_lpt_scan<<<1, LPT_BINS, 0, s>>>(g);
-    k_lpt_scatter<<<grid, 256, 0, s>>>(g);
+    launch(k_lpt_hist, grid, 256, 0, s, g);
+    launch(k_lpt_scan, 1, LPT_BINS, 0, s, g);
+    launch(k_lpt_scatter, grid, 256, 0, s, g);
     count_launch(3);
 }
 
@@ -899,21 +912,21 @@ void launch_vertex_bwd(const Globals &g, int n_views, int max_nv, int n_meshes, 
     const bool merge = rows > 0 && n_views + rows <= MAX_GRID_Y;
     const long long wide = !merge ? 0 : normals ? max_nf : g.n_verts_total;
     const dim3 grid(grid_x(std::max<long long>(max_nv, wide), 256, 2048), n_views + (merge ? rows : 0));
-    k_vertex_bwd<<<grid, 256, 0, s>>>(g);
+    launch(k_vertex_bwd, grid, 256, 0, s, g);
     count_launch(1);
     if (g.gcol && !merge) {
-        k_color_bwd<<<grid_x(g.n_verts_total, 256, 2048), 256, 0, s>>>(g);
+        launch(k_color_bwd, grid_x(g.n_verts_total, 256, 2048), 256, 0, s, g);
         count_launch(1);
     }
     if (normals && !merge) {
-        k_normal_bwd<<<dim3(grid_x(max_nf, 256, 2048), n_meshes), 256, 0, s>>>(g);
+        launch(k_normal_bwd, dim3(grid_x(max_nf, 256, 2048), n_meshes), 256, 0, s, g);
         count_launch(1);
     }
 }
 
 void launch_l2(const float *out, const float *tgt, long long n, float *grad, float *loss, cudaStream_t s)
 {
-    k_l2<<<grid_x(n, 256, 152 * 8), 256, 0, s>>>(out, tgt, n, grad, loss);
+    launch(k_l2, grid_x(n, 256, 152 * 8), 256, 0, s, out, tgt, n, grad, loss);
     count_launch(1);
 }
 

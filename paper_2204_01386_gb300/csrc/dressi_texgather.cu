@@ -76,6 +76,7 @@ __device__ __forceinline__ int scan_load(const ScanJob &J, int i) { return i < J
 
 __global__ void __launch_bounds__(SC_THREADS) k_scan_reduce(ScanJobs jobs)
 {
+    grid_wait();
     __shared__ int wt[32];
     const ScanJob &J = jobs.j[blockIdx.y];
     if (blockIdx.x * SC_TILE >= J.n_out) return;
@@ -92,6 +93,7 @@ __global__ void __launch_bounds__(SC_THREADS) k_scan_reduce(ScanJobs jobs)
 // partial[nparts] = total
 __global__ void __launch_bounds__(SC_THREADS) k_scan_partials(ScanJobs jobs)
 {
+    grid_wait();
     __shared__ int wt[32];
     const ScanJob &J = jobs.j[blockIdx.y];
     const int nparts = (J.n_out + SC_TILE - 1) / SC_TILE;
@@ -118,6 +120,7 @@ __global__ void __launch_bounds__(SC_THREADS) k_scan_partials(ScanJobs jobs)
 
 __global__ void __launch_bounds__(SC_THREADS) k_scan_down(ScanJobs jobs)
 {
+    grid_wait();
     __shared__ int wt[32];
     const ScanJob &J = jobs.j[blockIdx.y];
     if (blockIdx.x * SC_TILE >= J.n_out) return;
@@ -141,6 +144,7 @@ __global__ void __launch_bounds__(SC_THREADS) k_scan_down(ScanJobs jobs)
 // one launch instead of three); the total goes where the three-kernel scan leaves it
 __global__ void __launch_bounds__(SC_THREADS) k_scan_single(ScanJobs jobs)
 {
+    grid_wait();
     __shared__ int wt[32];
     const ScanJob &J = jobs.j[blockIdx.x];
     int carry = 0;
@@ -175,6 +179,7 @@ __device__ __forceinline__ int rs_count(const int *count, long long cap)
 __global__ void __launch_bounds__(RS_THREADS) k_rs_hist(const unsigned *keys, const int *count, long long cap,
                                                         int shift, int *hist, int nblocks)
 {
+    grid_wait();
     __shared__ int h[RS_BINS];
     const int n = rs_count(count, cap);
     const long long base = (long long)blockIdx.x * RS_TILE;
@@ -200,6 +205,7 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const unsigned *keys_
                                                            const int *offs, int nblocks, unsigned *keys_out,
                                                            int *vals_out)
 {
+    grid_wait();
     __shared__ int run[RS_BINS];                     // next free position of each digit
     __shared__ int wcnt[RS_THREADS / 32][RS_BINS];   // per-warp digit counts of a round
     const int n = rs_count(count, cap);
@@ -247,6 +253,7 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const unsigned *keys_
 // first[key] = the first sorted position holding key (the table starts at -1)
 __global__ void k_tg_first(const unsigned *keys, const int *count, int *first)
 {
+    grid_wait();
     const int n = *count;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const unsigned k = keys[i];
@@ -256,6 +263,7 @@ __global__ void k_tg_first(const unsigned *keys, const int *count, int *first)
 
 __global__ void k_tex_gather(Globals g, const unsigned *keys, const int *vals, const int *count, const int *first)
 {
+    grid_wait();
     const MeshK &M = g.meshes[blockIdx.y];
     const long long n_tex = (long long)M.tex_w * M.tex_h;
     const int n = *count;
@@ -312,14 +320,14 @@ void launch_scans(const ScanJob *jobs, int n, cudaStream_t s)
         longest = std::max(longest, jobs[i].n_out);
     }
     if (longest <= SC_SINGLE) {
-        k_scan_single<<<n, SC_THREADS, 0, s>>>(J);
+        launch(k_scan_single, n, SC_THREADS, 0, s, J);
         count_launch(1);
         return;
     }
     const dim3 grid((longest + SC_TILE - 1) / SC_TILE, n);
-    k_scan_reduce<<<grid, SC_THREADS, 0, s>>>(J);
-    k_scan_partials<<<dim3(1, n), SC_THREADS, 0, s>>>(J);
-    k_scan_down<<<grid, SC_THREADS, 0, s>>>(J);
+    launch(k_scan_reduce, grid, SC_THREADS, 0, s, J);
+    launch(k_scan_partials, dim3(1, n), SC_THREADS, 0, s, J);
+    launch(k_scan_down, grid, SC_THREADS, 0, s, J);
     count_launch(3);
 }
 
@@ -363,14 +371,14 @@ void launch_tex_gather(const Globals &g, long long slots, long long n_texels, in
     int *vout = vA;
     for (int pass = 0; pass < passes; ++pass) {
         const int shift = 8 * pass;
-        k_rs_hist<<<(int)nblocks, RS_THREADS, 0, s>>>(kin, cnt, slots, shift, hist, (int)nblocks);
+        launch(k_rs_hist, (int)nblocks, RS_THREADS, 0, s, kin, cnt, slots, shift, hist, (int)nblocks);
         const ScanJob job = {hist, hist, (int)hist_n, (int)hist_n, partial};
         launch_scans(&job, 1, s);
         if (pass == 0) {
             // the number of kept (valid) records is the scan's total
             cudaMemcpyAsync(count, partial + nparts, sizeof(int), cudaMemcpyDeviceToDevice, s);
         }
-        k_rs_scatter<<<(int)nblocks, RS_THREADS, 0, s>>>(kin, vin, cnt, slots, shift, hist, (int)nblocks, kout, vout);
+        launch(k_rs_scatter, (int)nblocks, RS_THREADS, 0, s, kin, vin, cnt, slots, shift, hist, (int)nblocks, kout, vout);
         count_launch(2);
         cnt = count;
         kin = kout;
@@ -379,9 +387,9 @@ void launch_tex_gather(const Globals &g, long long slots, long long n_texels, in
         vout = (vout == vA) ? vB : vA;
     }
     cudaMemsetAsync(first, 0xff, sizeof(int) * (size_t)std::max<long long>(n_texels, 1), s);
-    k_tg_first<<<grid_of(slots, 256, 152 * 16), 256, 0, s>>>(kin, count, first);
+    launch(k_tg_first, grid_of(slots, 256, 152 * 16), 256, 0, s, kin, count, first);
     dim3 grid(grid_of(max_texels, 256, 4096), n_meshes);
-    k_tex_gather<<<grid, 256, 0, s>>>(g, kin, vin, count, first);
+    launch(k_tex_gather, grid, 256, 0, s, g, kin, vin, count, first);
     count_launch(2);
 }
 
@@ -392,6 +400,7 @@ void launch_tex_gather(const Globals &g, long long slots, long long n_texels, in
 // ---------------------------------------------------------------------------
 __global__ void k_inv_uv_apply(Globals g, long long n_texels)
 {
+    grid_wait();
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n_texels;
          t += (long long)gridDim.x * blockDim.x) {
         const int s = g.inv_uv[t];
@@ -404,7 +413,7 @@ __global__ void k_inv_uv_apply(Globals g, long long n_texels)
 void launch_inv_uv_apply(const Globals &g, long long n_texels, cudaStream_t s)
 {
     const long long blocks = std::min<long long>((n_texels + 255) / 256, 152LL * 32);
-    k_inv_uv_apply<<<(int)std::max<long long>(blocks, 1), 256, 0, s>>>(g, n_texels);
+    launch(k_inv_uv_apply, (int)std::max<long long>(blocks, 1), 256, 0, s, g, n_texels);
     count_launch(1);
 }
 

@@ -1959,6 +1959,7 @@ constexpr int tile_min_ctas()
 template <int K, int MODE, int TT>
 __global__ void __launch_bounds__(cta_threads<MODE, TT>(), tile_min_ctas<MODE, TT>()) k_tile(Globals g)
 {
+    grid_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem &S = *reinterpret_cast<Smem *>(smem_raw);
     unsigned long long *kbuf = reinterpret_cast<unsigned long long *>(smem_raw + sizeof(Smem));
@@ -1970,6 +1971,7 @@ __global__ void __launch_bounds__(cta_threads<MODE, TT>(), tile_min_ctas<MODE, T
 template <int K, int MODE, int TT>
 __global__ void __launch_bounds__(cta_threads<MODE, TT>(), tile_min_ctas<MODE, TT>()) k_tile_persistent(Globals g)
 {
+    grid_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem &S = *reinterpret_cast<Smem *>(smem_raw);
     unsigned long long *kbuf = reinterpret_cast<unsigned long long *>(smem_raw + sizeof(Smem));
@@ -2038,9 +2040,9 @@ static void launch_kk(const Globals &g, cudaStream_t s)
     }
     if (g.persistent) {
         const int grid = std::min(g.total_tiles, per_sm * sms);
-        k_tile_persistent<K, MODE, TT><<<grid, NT, smem, s>>>(g);
+        launch(k_tile_persistent<K, MODE, TT>, grid, NT, smem, s, g);
     } else {
-        k_tile<K, MODE, TT><<<g.total_tiles, NT, smem, s>>>(g);
+        launch(k_tile<K, MODE, TT>, g.total_tiles, NT, smem, s, g);
     }
 }
 
