@@ -36,6 +36,7 @@ static void launch_tile_profiled(const Globals &g, int pass, cudaStream_t s)
     const bool bwd = pass == 1;
     cudaEvent_t b = g_prof[bwd ? 2 : 0], e = g_prof[bwd ? 3 : 1];
     if (b) cudaEventRecord(b, s);
+    if (g.heavy) launch_tile_heavy(g, s);
     if (pass == 2) launch_tile_shade(g, s);
     else launch_tile(g, bwd, s);
     if (e) cudaEventRecord(e, s);
@@ -55,6 +56,7 @@ struct Plan {
     std::vector<ViewK> views;
     std::vector<MeshK> meshes;
     Layout lay;
+    int dense = 0;   // faces per tile, the densest view's
     int max_nv = 0, max_nf = 0, max_nv_view = 0, max_nf_view = 0, max_texels = 0;
     long long n_texels = 0, n_faces = 0, view_faces = 0, view_pixels = 0;
 };
@@ -154,6 +156,7 @@ static bool make_plan(const dressi_scene *sc, const dressi_view *views, int n_vi
         view_faces += mk.nF;
         P.max_nv_view = std::max(P.max_nv_view, mk.nV);
         P.max_nf_view = std::max(P.max_nf_view, mk.nF);
+        P.dense = std::max(P.dense, (int)(mk.nF / ((long long)k.tiles_x * k.tiles_y)));
         long long nt = (long long)tiles + (long long)k.tiles_x * k.tiles_y;
         if (nt > 0x7fffffff) return false;
         tiles = (int)nt;
@@ -313,6 +316,7 @@ static void run_setup(Globals &g, const Plan &P, char *ws, bool need_bins, Clear
         clear(L.adj_off, nv + 1);
         clear(L.adj_cur, nv);
     }
+    if (g.heavy) clear(L.sgrad, 1);
     if (g.persistent || g.fronts == 2) clear(L.queue, 4);
     if (g.persistent) clear(L.lpt_hist, LPT_BINS);
     // the view and mesh tables, adjacent in the workspace
@@ -364,6 +368,19 @@ static void choose_fronts(Globals &g, const Plan &P, bool only, char *ws, cudaSt
     cudaMemsetAsync(ws + P.lay.kth, WORD_FILL, sizeof(unsigned long long) * (size_t)P.view_pixels, s);
 }
 
+// Views of more faces than this per tile may have tiles that outlast the others (long_list): a
+// forward lists them, in the adjoint's vertex accumulators (free until then), for k_tile_heavy.  The
+// launch and the listing cost some 4 us where there turn out to be none.
+constexpr int HEAVY_FACES_PER_TILE = 256;
+
+static void allow_heavy(Globals &g, const Plan &P, char *ws)
+{
+    // its tiles take one raster pass: the in-tile front pass is followed by a second one
+    if (g.fronts == 1 || P.dense < HEAVY_FACES_PER_TILE) return;
+    g.heavy_cap = (int)std::min<long long>(HEAVY_MAX, 4 * P.lay.n_vrec - 1);
+    if (g.heavy_cap > 0) g.heavy = reinterpret_cast<int *>(ws + P.lay.sgrad);
+}
+
 // a forward that stores no layer ids leaves every pixel's word (K-th entry, or front layer with
 // E and S^H) in the workspace for a re-rasterizing adjoint; the flag says which, if any
 static Clears keep_kth(Globals &g, const Plan &P, const dressi_params *p, char *ws, cudaStream_t s)
@@ -371,6 +388,7 @@ static Clears keep_kth(Globals &g, const Plan &P, const dressi_params *p, char *
     const bool keep = g.ids == nullptr;
     g.kth = keep ? reinterpret_cast<unsigned long long *>(ws + P.lay.kth) : nullptr;
     choose_fronts(g, P, keep && fronts_only(p), ws, s);
+    allow_heavy(g, P, ws);
     Clears clr;
     clr.p[0] = reinterpret_cast<int *>(ws + P.lay.kth_flag);
     clr.n[0] = 1;

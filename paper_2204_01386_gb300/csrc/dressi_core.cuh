@@ -166,6 +166,9 @@ struct Globals {
     int *kth_flag;
     int fronts;           // layers beyond the front one are only needed inside the edge mask: the front
                           // ones come 1 from the tiles' rasters, 2 from the face table kernel (in kth)
+    int *heavy;           // a forward's tiles with long face lists: their number, then the tiles (k_bin
+                          // lists them where the host allows it), or nullptr
+    int heavy_cap;
     int2 *big;            // faces left to k_front_big (view, face), in the tile lists' place
     int big_cap;
     int *big_n;
@@ -328,6 +331,30 @@ __device__ __forceinline__ bool face_get(const Globals &g, const ViewK &V, const
     R.flags = __float_as_int(w[19]);
     R.id = __float_as_int(w[20]);
     return (R.flags & FLAG_LIVE) != 0;
+}
+
+// A tile's face list is long where it is several times the list entries that each of the GPU's CTAs
+// would get of all tiles' lists, and more than a few chunks: alone, the tile would outlast the rest.
+// (A 32 px tile of a 200,000-face mesh seen at 128^2 holds 25,000 faces: one CTA took 1.3 ms.)
+constexpr int HEAVY_MIN = 1024;        // entries
+constexpr int HEAVY_SHARE = 2;         // times the entries per CTA
+constexpr int HEAVY_CTAS = 608;        // four CTAs on each of 152 SMs
+constexpr int HEAVY_CLUSTERS = HEAVY_CTAS / 8;
+constexpr int HEAVY_MAX = 1024;        // more long tiles than this keep the GPU busy one CTA each
+
+__device__ __forceinline__ bool long_list(const Globals &g, int t)
+{
+    return g.tile_count[t] > max(HEAVY_MIN, g.tile_off[g.total_tiles] / HEAVY_CTAS * HEAVY_SHARE);
+}
+// the listed tiles, none if there are too many
+__device__ __forceinline__ int heavy_count(const Globals &g)
+{
+    const int n = g.heavy ? g.heavy[0] : 0;
+    return n <= g.heavy_cap ? n : 0;
+}
+__device__ __forceinline__ bool is_heavy(const Globals &g, int t)
+{
+    return g.heavy && heavy_count(g) > 0 && long_list(g, t);
 }
 
 // a hint that the line holding address a will be read soon: fetch it into L2

@@ -44,7 +44,7 @@ struct Tables {
 };
 // small arrays of 32-bit words set by the vertex transform for the kernels after it
 struct Clears {
-    static constexpr int MAX = 5;
+    static constexpr int MAX = 6;
     int *p[MAX] = {};
     int n[MAX] = {}, v[MAX] = {};
 };
@@ -69,6 +69,7 @@ void launch_faces(const Globals &g, int n_views, int n_meshes, int max_nf_view, 
 void launch_fill(const Fills &f, cudaStream_t s);
 void launch_tile(const Globals &g, bool backward, cudaStream_t s);
 void launch_tile_shade(const Globals &g, cudaStream_t s);
+void launch_tile_heavy(const Globals &g, cudaStream_t s);
 void launch_lpt_order(const Globals &g, cudaStream_t s);
 size_t texgather_scratch_bytes(long long slots, long long n_texels, size_t align);
 void launch_scans(const ScanJob *jobs, int n, cudaStream_t s);   // one or two, in the same launches

@@ -526,6 +526,14 @@ __global__ void k_bin(Globals g)
         adjacency<1>(g, blockIdx.y - g.n_views);
         return;
     }
+    if (g.heavy) {
+        const int nthreads = gridDim.x * g.n_views * blockDim.x;
+        for (int t = (blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x; t < g.total_tiles; t += nthreads)
+            if (long_list(g, t)) {
+                const int q = atomicAdd(g.heavy, 1);
+                if (q < g.heavy_cap) g.heavy[1 + q] = t;
+            }
+    }
     const ViewK V = g.views[blockIdx.y];   // copies: the fields stay in registers across the stores
     const MeshK M = g.meshes[V.mesh];
     for (int f0 = blockIdx.x * blockDim.x; f0 < M.nF; f0 += gridDim.x * blockDim.x) {

@@ -32,6 +32,8 @@
 #include "dressi_core.cuh"
 #include "dressi_launch.h"
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <atomic>
 #include <mutex>
@@ -1364,11 +1366,11 @@ __device__ __forceinline__ void raster_items(Smem &S, unsigned long long *kbuf, 
                                      fronts)) {
                     ++n_cand;
                     const unsigned long long v = pack_frag(fr.key, S.fid[f]);
-                    // the slot's entry only ever gets smaller: a value not below it stays out
-                    if (v < last) {
-                        if (fronts) atomicMin(slots, v);
-                        else kbuf_insert<K>(slots, v);
-                    }
+                    if (fronts) atomicMin(slots, v);
+                    // the K-th entry only ever gets smaller: a value not below it stays out (with few
+                    // slots the cascade itself is cheaper: K = 3 without the test 625 -> 616 us on 24
+                    // views of 512^2, K = 5 with it 471 -> 465)
+                    else if (K <= 3 || v < last) kbuf_insert<K>(slots, v);
                 }
             }
         }
@@ -1453,13 +1455,71 @@ __device__ __forceinline__ void raster_items(Smem &S, unsigned long long *kbuf, 
     if (qn > 0) evaluate(qn);
 }
 
+// work counters: pairs enumerated, exact evaluations, candidates kept, layers shaded
+__device__ __forceinline__ void add_stats(const Globals &g, unsigned n_pairs, unsigned n_exact, unsigned n_cand,
+                                          unsigned n_layers)
+{
+    if (!g.stats) return;
+    unsigned long long c[4] = {n_pairs, n_exact, n_cand, n_layers};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) c[q] += __shfl_xor_sync(0xffffffffu, c[q], o);
+        if ((threadIdx.x & 31) == 0) atomicAdd(g.stats + q, c[q]);
+    }
+}
+
+// the K-lists, and S^H of a ring of hs x hs (0: none), of a cluster's CTAs into the first one's.  Every
+// candidate was seen by one CTA: the K smallest of the lists' entries are the tile's.
+template <int K, int TT, int CL>
+__device__ __forceinline__ void merge_cluster(Smem &S, unsigned long long *kbuf, int hs, int rank)
+{
+    auto cluster = cooperative_groups::this_cluster();
+    cluster.sync();   // every list is complete
+    if (rank == 0) {
+        for (int p = threadIdx.x; p < TT * TT; p += blockDim.x) {
+            unsigned long long v[K];
+#pragma unroll
+            for (int k = 0; k < K; ++k) v[k] = kbuf[p * K + k];
+            for (int r = 1; r < CL; ++r) {
+                const unsigned long long *o = cluster.map_shared_rank(kbuf, r) + p * K;
+                unsigned long long w[K];
+#pragma unroll
+                for (int k = 0; k < K; ++k) w[k] = o[k];
+#pragma unroll
+                for (int j = 0; j < K; ++j) {
+                    unsigned long long x = w[j];
+#pragma unroll
+                    for (int k = 0; k < K; ++k) {
+                        const unsigned long long m = v[k] < x ? v[k] : x;
+                        x = v[k] < x ? x : v[k];
+                        v[k] = m;
+                    }
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < K; ++k) kbuf[p * K + k] = v[k];
+        }
+        for (int i = threadIdx.x; i < hs * hs; i += blockDim.x) {
+            bool any = false;
+            for (int r = 1; r < CL; ++r) any |= cluster.map_shared_rank(S.sh, r)[i] == 1;
+            if (any) S.sh[i] = 1;
+        }
+    }
+    cluster.sync();   // the other CTAs' shared memory has been read
+}
+
 // everything one CTA does for global tile t.  MODE: 0 forward, 1 adjoint that
 // re-rasterizes, 2 adjoint from stored layer ids, 3 forward from stored layer ids
 // (re-shading a static geometry: no binning, raster or peel); 4, 5, 6, 7 = 2, 1, 0, 3
 // with the normal map, the light gradient and the inverse UV compiled in
-template <int K, int MODE, int TT>
+// CL > 1: a cluster of CL CTAs works on the tile (a forward with one raster pass): each rasterizes
+// every CL-th chunk of the face list into K-lists of its own, and the first merges them, by
+// distributed shared memory, and goes on alone.
+template <int K, int MODE, int TT, int CL = 1>
 __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned long long *kbuf, const int t)
 {
+    const int rank = CL > 1 ? (int)cooperative_groups::this_cluster().block_rank() : 0;
     constexpr int NT = cta_threads<MODE, TT>();
     constexpr int PPT = TT * TT / NT;   // pixels per thread in the per-pixel phases
     // after the K-lists: the candidate queue and the two pair-block tables
@@ -1556,6 +1616,8 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
                 __syncthreads();
             }
         }
+        // no raster: nothing for the other CTAs of a cluster
+        if (CL > 1 && rank != 0 && (empty || stage == ST_DONE)) return;
         if (!empty && stage != ST_DONE)   // 16-byte stores (TT^2 K is even; kbuf is 16-byte aligned)
             for (int i = tid; i < TT * TT * K / 2; i += NT)
                 reinterpret_cast<ulonglong2 *>(kbuf)[i] = make_ulonglong2(EMPTY, EMPTY);
@@ -1598,13 +1660,13 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
         const bool use_hash = !BWD && single_chunk;
         while (stage != ST_DONE && !empty) {
             const float reach = stage == ST_FRONT ? 0.f : V.r_px;
-            for (int c0 = 0; c0 < n; c0 += CH) {
+            for (int c0 = rank * CH; c0 < n; c0 += CH * CL) {
                 const int nch = min(CH, n - c0);
                 // the next chunk's face ids, loaded under this chunk's staging: their records
                 // are prefetched into L2 once this chunk is staged
-                const int nnext = min(CH, n - c0 - CH);
+                const int nnext = min(CH, n - c0 - CH * CL);
                 int fnext = -1;
-                if (tid < nnext) fnext = fallback ? c0 + CH + tid : g.lists[lb + c0 + CH + tid];
+                if (tid < nnext) fnext = fallback ? c0 + CH * CL + tid : g.lists[lb + c0 + CH * CL + tid];
                 __syncthreads();   // previous chunk consumed
                 if (use_hash) {
                     for (int i = tid; i < HASH; i += NT) S.hash[i] = make_int2(-1, -1);
@@ -1721,6 +1783,13 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
                     // decided by the exact fill-rule test
                     if (fmin > APPROX_EPS || hard_test(S.F[f], (float)(X0 + x) + 0.5f, (float)(Y0 + y) + 0.5f))
                         S.sh[si] = 1;
+                }
+            }
+            if constexpr (CL > 1) {
+                merge_cluster<K, TT, CL>(S, kbuf, ring ? hs : 0, rank);
+                if (rank != 0) {
+                    add_stats(g, n_pairs, n_exact, n_cand, 0u);
+                    return;
                 }
             }
             ring = false;
@@ -1930,16 +1999,7 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
             if ((tid & 31) == 0 && v != 0.f) atomicAdd(g.glight + 3 * (long long)S.view + c, v);
         }
     }
-    if (g.stats) {
-        // work counters: pairs enumerated, exact evaluations, candidates kept, layers shaded
-        unsigned long long c[4] = {n_pairs, n_exact, n_cand, n_layers};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) c[q] += __shfl_xor_sync(0xffffffffu, c[q], o);
-            if ((threadIdx.x & 31) == 0) atomicAdd(g.stats + q, c[q]);
-        }
-    }
+    add_stats(g, n_pairs, n_exact, n_cand, n_layers);
 }
 
 // one CTA per tile.  CTAs per SM, measured (us; 24 views of 512^2 of 20,480 faces unless said):
@@ -1963,7 +2023,7 @@ __global__ void __launch_bounds__(cta_threads<MODE, TT>(), tile_min_ctas<MODE, T
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem &S = *reinterpret_cast<Smem *>(smem_raw);
     unsigned long long *kbuf = reinterpret_cast<unsigned long long *>(smem_raw + sizeof(Smem));
-    tile_body<K, MODE, TT>(g, S, kbuf, blockIdx.x);
+    if (MODE != 0 && MODE != 6 || !is_heavy(g, blockIdx.x)) tile_body<K, MODE, TT>(g, S, kbuf, blockIdx.x);
 }
 
 // persistent: as many CTAs as fit on the GPU pull tiles from one queue, in the
@@ -1981,8 +2041,27 @@ __global__ void __launch_bounds__(cta_threads<MODE, TT>(), tile_min_ctas<MODE, T
         const int q = S.next;
         if (q >= g.total_tiles) break;
         const int t = g.tile_order ? g.tile_order[q] : q;
-        tile_body<K, MODE, TT>(g, S, kbuf, t);
+        if (MODE != 0 && MODE != 6 || !is_heavy(g, t)) tile_body<K, MODE, TT>(g, S, kbuf, t);
         __syncthreads();   // the tile's shared memory is free again
+    }
+}
+
+// Long face lists, a cluster per tile: the tiles that k_bin listed, for their number is small against
+// the CTAs of the GPU and each would take one CTA longer than its share of the whole.
+constexpr int HEAVY_CL = 8;
+
+template <int K, int MODE, int TT>
+__global__ void __cluster_dims__(HEAVY_CL, 1, 1) __launch_bounds__(cta_threads<MODE, TT>(), tile_min_ctas<MODE, TT>())
+    k_tile_heavy(Globals g)
+{
+    grid_wait();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Smem &S = *reinterpret_cast<Smem *>(smem_raw);
+    unsigned long long *kbuf = reinterpret_cast<unsigned long long *>(smem_raw + sizeof(Smem));
+    const int n = heavy_count(g);
+    for (int h = blockIdx.x / HEAVY_CL; h < n; h += gridDim.x / HEAVY_CL) {
+        tile_body<K, MODE, TT, HEAVY_CL>(g, S, kbuf, g.heavy[1 + h]);
+        cooperative_groups::this_cluster().sync();   // the tile's shared memory is free again
     }
 }
 
@@ -2044,6 +2123,42 @@ static void launch_kk(const Globals &g, cudaStream_t s)
     } else {
         launch(k_tile<K, MODE, TT>, g.total_tiles, NT, smem, s, g);
     }
+}
+
+template <int K, int MODE, int TT>
+static void launch_heavy_kk(const Globals &g, cudaStream_t s)
+{
+    // per device, like launch_kk
+    static std::atomic<bool> ready[LAUNCH_MAX_DEVICES];
+    constexpr int NT = cta_threads<MODE, TT>();
+    const size_t smem = tile_smem_bytes<K, MODE, TT>();
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+    if (dev < 0 || dev >= LAUNCH_MAX_DEVICES || !ready[dev].load(std::memory_order_acquire)) {
+        cudaFuncSetAttribute(k_tile_heavy<K, MODE, TT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (dev >= 0 && dev < LAUNCH_MAX_DEVICES) ready[dev].store(true, std::memory_order_release);
+    }
+    launch(k_tile_heavy<K, MODE, TT>, HEAVY_CL * HEAVY_CLUSTERS, NT, smem, s, g);
+}
+
+// the tiles of g.heavy, before the other tiles' kernel (modes 0 and 6)
+template <int MODE, int TT>
+static void launch_heavy_k(const Globals &g, cudaStream_t s)
+{
+    switch (g.K) {
+    case 1: launch_heavy_kk<1, MODE, TT>(g, s); break;
+    case 2: launch_heavy_kk<2, MODE, TT>(g, s); break;
+    case 3: launch_heavy_kk<3, MODE, TT>(g, s); break;
+    case 4: launch_heavy_kk<4, MODE, TT>(g, s); break;
+    default: launch_heavy_kk<5, MODE, TT>(g, s); break;
+    }
+}
+
+template <int MODE>
+void launch_heavy_mode(const Globals &g, cudaStream_t s)
+{
+    if (g.tile == 32) launch_heavy_k<MODE, 32>(g, s);
+    else launch_heavy_k<MODE, 16>(g, s);
 }
 
 template <int MODE, int TT>

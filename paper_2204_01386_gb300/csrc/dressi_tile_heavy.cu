@@ -1,0 +1,15 @@
+// dressi_tile_heavy.cu -- per-tile kernel of the forward, a cluster of CTAs per tile, for the tiles with
+// long face lists.
+#include "dressi_tile.cuh"
+
+namespace dressi {
+template void launch_heavy_mode<0>(const Globals &g, cudaStream_t s);
+extern template void launch_heavy_mode<6>(const Globals &g, cudaStream_t s);
+
+void launch_tile_heavy(const Globals &g, cudaStream_t s)
+{
+    if (g.shade_mode == 3) launch_heavy_mode<6>(g, s);
+    else launch_heavy_mode<0>(g, s);
+    count_launch(1);
+}
+}  // namespace dressi
