@@ -36,8 +36,8 @@ static void launch_tile_profiled(const Globals &g, int pass, cudaStream_t s)
     const bool bwd = pass == 1;
     cudaEvent_t b = g_prof[bwd ? 2 : 0], e = g_prof[bwd ? 3 : 1];
     if (b) cudaEventRecord(b, s);
-    if (g.heavy) launch_tile_heavy(g, s);
     if (pass == 2) launch_tile_shade(g, s);
+    else if (g.heavy) launch_tile_heavy(g, s);   // a forward's
     else launch_tile(g, bwd, s);
     if (e) cudaEventRecord(e, s);
 }
@@ -317,7 +317,7 @@ static void run_setup(Globals &g, const Plan &P, char *ws, bool need_bins, Clear
         clear(L.adj_cur, nv);
     }
     if (g.heavy) clear(L.sgrad, 1);
-    if (g.persistent || g.fronts == 2) clear(L.queue, 4);
+    if (g.persistent || g.fronts == 2 || g.heavy) clear(L.queue, 4);
     if (g.persistent) clear(L.lpt_hist, LPT_BINS);
     // the view and mesh tables, adjacent in the workspace
     const size_t words = (L.meshes + sizeof(MeshK) * P.meshes.size()) / 4;
@@ -369,8 +369,8 @@ static void choose_fronts(Globals &g, const Plan &P, bool only, char *ws, cudaSt
 }
 
 // Views of more faces than this per tile may have tiles that outlast the others (long_list): a
-// forward lists them, in the adjoint's vertex accumulators (free until then), for k_tile_heavy.  The
-// launch and the listing cost some 4 us where there turn out to be none.
+// forward lists them, in the adjoint's vertex accumulators (free until then), for k_tile_heavy, which
+// then takes all tiles.
 constexpr int HEAVY_FACES_PER_TILE = 256;
 
 static void allow_heavy(Globals &g, const Plan &P, char *ws)

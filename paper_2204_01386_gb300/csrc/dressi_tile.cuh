@@ -2023,11 +2023,26 @@ __global__ void __launch_bounds__(cta_threads<MODE, TT>(), tile_min_ctas<MODE, T
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem &S = *reinterpret_cast<Smem *>(smem_raw);
     unsigned long long *kbuf = reinterpret_cast<unsigned long long *>(smem_raw + sizeof(Smem));
-    if (MODE != 0 && MODE != 6 || !is_heavy(g, blockIdx.x)) tile_body<K, MODE, TT>(g, S, kbuf, blockIdx.x);
+    tile_body<K, MODE, TT>(g, S, kbuf, blockIdx.x);
 }
 
-// persistent: as many CTAs as fit on the GPU pull tiles from one queue, in the
-// order of g.tile_order (longest face list first) when it is given
+// CTAs pull tiles from one queue, in the order of g.tile_order (longest face list first) when it is
+// given; LONG: without the tiles that k_tile_heavy's clusters took
+template <int K, int MODE, int TT, bool LONG>
+__device__ __forceinline__ void pull_tiles(const Globals &g, Smem &S, unsigned long long *kbuf)
+{
+    for (;;) {
+        if (threadIdx.x == 0) S.next = atomicAdd(g.queue, 1);
+        __syncthreads();
+        const int q = S.next;
+        if (q >= g.total_tiles) break;
+        const int t = g.tile_order ? g.tile_order[q] : q;
+        if (!LONG || !is_heavy(g, t)) tile_body<K, MODE, TT>(g, S, kbuf, t);
+        __syncthreads();   // the tile's shared memory is free again
+    }
+}
+
+// persistent: as many CTAs as fit on the GPU
 template <int K, int MODE, int TT>
 __global__ void __launch_bounds__(cta_threads<MODE, TT>(), tile_min_ctas<MODE, TT>()) k_tile_persistent(Globals g)
 {
@@ -2035,19 +2050,12 @@ __global__ void __launch_bounds__(cta_threads<MODE, TT>(), tile_min_ctas<MODE, T
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem &S = *reinterpret_cast<Smem *>(smem_raw);
     unsigned long long *kbuf = reinterpret_cast<unsigned long long *>(smem_raw + sizeof(Smem));
-    for (;;) {
-        if (threadIdx.x == 0) S.next = atomicAdd(g.queue, 1);
-        __syncthreads();
-        const int q = S.next;
-        if (q >= g.total_tiles) break;
-        const int t = g.tile_order ? g.tile_order[q] : q;
-        if (MODE != 0 && MODE != 6 || !is_heavy(g, t)) tile_body<K, MODE, TT>(g, S, kbuf, t);
-        __syncthreads();   // the tile's shared memory is free again
-    }
+    pull_tiles<K, MODE, TT, false>(g, S, kbuf);
 }
 
-// Long face lists, a cluster per tile: the tiles that k_bin listed, for their number is small against
-// the CTAs of the GPU and each would take one CTA longer than its share of the whole.
+// Persistent, with the tiles of long face lists (k_bin listed them) first, a cluster of CTAs per tile:
+// few against the GPU's CTAs, each of them would take one CTA longer than its share of the whole.
+// The CTAs then pull the other tiles one by one.
 constexpr int HEAVY_CL = 8;
 
 template <int K, int MODE, int TT>
@@ -2058,11 +2066,23 @@ __global__ void __cluster_dims__(HEAVY_CL, 1, 1) __launch_bounds__(cta_threads<M
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem &S = *reinterpret_cast<Smem *>(smem_raw);
     unsigned long long *kbuf = reinterpret_cast<unsigned long long *>(smem_raw + sizeof(Smem));
+    auto cluster = cooperative_groups::this_cluster();
     const int n = heavy_count(g);
-    for (int h = blockIdx.x / HEAVY_CL; h < n; h += gridDim.x / HEAVY_CL) {
+    while (n > 0) {
+        if (cluster.block_rank() == 0 && threadIdx.x < HEAVY_CL) {
+            int h = 0;
+            if (threadIdx.x == 0) h = atomicAdd(g.queue + 2, 1);
+            h = __shfl_sync((1u << HEAVY_CL) - 1u, h, 0);
+            *cluster.map_shared_rank(&S.next, threadIdx.x) = h;
+        }
+        cluster.sync();
+        const int h = S.next;
+        if (h >= n) break;
         tile_body<K, MODE, TT, HEAVY_CL>(g, S, kbuf, g.heavy[1 + h]);
-        cooperative_groups::this_cluster().sync();   // the tile's shared memory is free again
+        cluster.sync();   // the tile's shared memory is free again
     }
+    __syncthreads();   // S.next has been read
+    pull_tiles<K, MODE, TT, true>(g, S, kbuf);
 }
 
 template <int K, int MODE, int TT>
@@ -2141,7 +2161,7 @@ static void launch_heavy_kk(const Globals &g, cudaStream_t s)
     launch(k_tile_heavy<K, MODE, TT>, HEAVY_CL * HEAVY_CLUSTERS, NT, smem, s, g);
 }
 
-// the tiles of g.heavy, before the other tiles' kernel (modes 0 and 6)
+// all tiles, those of g.heavy first and by clusters (modes 0 and 6)
 template <int MODE, int TT>
 static void launch_heavy_k(const Globals &g, cudaStream_t s)
 {

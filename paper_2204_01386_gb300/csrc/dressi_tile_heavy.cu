@@ -1,5 +1,5 @@
-// dressi_tile_heavy.cu -- per-tile kernel of the forward, a cluster of CTAs per tile, for the tiles with
-// long face lists.
+// dressi_tile_heavy.cu -- per-tile kernel of the forward with a cluster of CTAs for each tile that has a
+// long face list.
 #include "dressi_tile.cuh"
 
 namespace dressi {
