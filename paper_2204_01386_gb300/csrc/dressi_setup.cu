@@ -820,6 +820,19 @@ static int grid_x(long long n, int block, int cap)
 
 constexpr int MAX_GRID_Y = 65535;
 
+constexpr long long GRID_BLOCKS = 8192;
+
+// blocks along x for `rows` grid rows whose longest takes n: the rows of a ragged batch are mostly far
+// shorter, and past some thousands of blocks those without work cost more than a second round of
+// the others (32 meshes of 1,000 to 200,000 faces, us without / at 8,192 / at 4,096 blocks: face table
+// 85 / 53 / 60, list fill 52 / 32 / 38, end of the adjoint 60 / 35 / 50)
+static int grid_rows(long long n, int block, int cap, int rows)
+{
+    int x = grid_x(n, block, cap);
+    while (x > 64 && (long long)x * rows > GRID_BLOCKS) x = (x + 1) / 2;
+    return x;
+}
+
 template <int TABLES>
 static void launch_vertex_t(const Globals &g, dim3 grid, const unsigned *tables, int words, const Clears &clr,
                             cudaStream_t s)
@@ -836,7 +849,7 @@ static void launch_vertex_t(const Globals &g, dim3 grid, const unsigned *tables,
 void launch_vertex(const Globals &g, int n_views, int max_nv, const unsigned *tables, int words, const Clears &clr,
                    cudaStream_t s)
 {
-    dim3 grid(grid_x(max_nv, 256, 1024), n_views);
+    dim3 grid(grid_rows(max_nv, 256, 1024, n_views), n_views);
     if (words == 0) launch_vertex_t<0>(g, grid, tables, words, clr, s);
     else if (words <= 128) launch_vertex_t<128>(g, grid, tables, words, clr, s);
     else launch_vertex_t<TABLE_WORDS>(g, grid, tables, words, clr, s);
@@ -850,7 +863,8 @@ void launch_faces(const Globals &g, int n_views, int n_meshes, int max_nf_view, 
 {
     // (a launch holds 65,535 grid rows; views and meshes may be more together)
     const bool merge = normals && n_views + n_meshes <= MAX_GRID_Y;
-    const dim3 grid(grid_x(std::max(max_nf_view, merge ? max_nf : 0), 256, 2048), n_views + (merge ? n_meshes : 0));
+    const int rows = n_views + (merge ? n_meshes : 0);
+    const dim3 grid(grid_rows(std::max(max_nf_view, merge ? max_nf : 0), 256, 2048, rows), rows);
     const dim3 grid_m(grid_x(max_nf, 256, 2048), n_meshes);
     if (lists && g.fronts == 2) launch(k_face<true, true>, grid, 256, 0, s, g);
     else if (lists) launch(k_face<true, false>, grid, 256, 0, s, g);
@@ -882,7 +896,7 @@ void launch_faces(const Globals &g, int n_views, int n_meshes, int max_nf_view, 
         count_launch(1);
     }
     if (normals) {
-        launch(k_normal_csr, dim3(grid_x(max_nv, 256, 2048), n_meshes), 256, 0, s, g);
+        launch(k_normal_csr, dim3(grid_rows(max_nv, 256, 2048, n_meshes), n_meshes), 256, 0, s, g);
         count_launch(1);
     }
 }
@@ -919,7 +933,8 @@ void launch_vertex_bwd(const Globals &g, int n_views, int max_nv, int n_meshes, 
     const int rows = normals ? n_meshes : g.gcol ? 1 : 0;
     const bool merge = rows > 0 && n_views + rows <= MAX_GRID_Y;
     const long long wide = !merge ? 0 : normals ? max_nf : g.n_verts_total;
-    const dim3 grid(grid_x(std::max<long long>(max_nv, wide), 256, 2048), n_views + (merge ? rows : 0));
+    const int all = n_views + (merge ? rows : 0);
+    const dim3 grid(grid_rows(std::max<long long>(max_nv, wide), 256, 2048, all), all);
     launch(k_vertex_bwd, grid, 256, 0, s, g);
     count_launch(1);
     if (g.gcol && !merge) {
