@@ -162,7 +162,10 @@ class Renderer:
         self._setup = (key, bins or (old is not None and old[0] == key and old[1]))
 
     def _stream(self):
-        return C.c_void_p(torch.cuda.current_stream(self.scene.device).cuda_stream)
+        # the raw handle: building a torch.cuda.Stream around it takes 3.5 us, a tenth of the host
+        # side of a small forward
+        dev = self.scene.device
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if dev.index is None else dev.index)
 
     def signature(self) -> str:
         """Key of this workload for the autotune cache: GPU, views, meshes, parameters."""
