@@ -371,7 +371,7 @@ static void choose_fronts(Globals &g, const Plan &P, bool only, char *ws, cudaSt
 // Views of more faces than this per tile may have tiles that outlast the others (long_list): a
 // forward lists them, in the adjoint's vertex accumulators (free until then), for k_tile_heavy, which
 // then takes all tiles.
-constexpr int HEAVY_FACES_PER_TILE = 256;
+constexpr int HEAVY_FACES_PER_TILE = 512;
 
 static void allow_heavy(Globals &g, const Plan &P, char *ws)
 {
