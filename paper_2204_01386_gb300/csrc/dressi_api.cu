@@ -368,15 +368,36 @@ static void choose_fronts(Globals &g, const Plan &P, bool only, char *ws, cudaSt
     cudaMemsetAsync(ws + P.lay.kth, WORD_FILL, sizeof(unsigned long long) * (size_t)P.view_pixels, s);
 }
 
-// Views of more faces than this per tile may have tiles that outlast the others (long_list): a
-// forward lists them, in the adjoint's vertex accumulators (free until then), for k_tile_heavy, which
-// then takes all tiles.
-constexpr int HEAVY_FACES_PER_TILE = 512;
+// Whether a forward lists its tiles with long face lists (long_list), in the adjoint's vertex
+// accumulators (free until then), for k_tile_heavy, which then takes all tiles.  Forward tile kernel, us,
+// one CTA per tile / this (tiles of the scene; CTAs per long tile):
+//   5,120 faces at 128^2 (64; 8) 60 / 37, at 256^2 (256; 4) 46 / 37, at 352^2 (484; 2) 49 / 42
+//   8,000 faces at 521 x 337 (726; 8) 56 / 45
+//   20,480 faces at 512^2 in 32 px tiles, 1 view (256; 4) 134 / 128, 2 views (512; 2) 187 / 128
+//   5,120 faces, r = 7 px, K = 5, 224^2, 1 view (196; 4) 128 / 106, 4 views (784; 8) 169 / 175
+//   32 meshes of 1,000 to 200,000 faces (10,000; 8) 1481 / 874
+//   320 faces at 64^2 (16): nothing to share, 13 / 15 -- hence SMALL_FACES
+//   8 views of 2048^2 of 1.31 M faces (32,768): no long list, 1596 / 1657 -- hence 512 faces per tile
+constexpr int SMALL_TILES = 512, SMALL_MIN = 96, SMALL_FACES = 2048;
 
 static void allow_heavy(Globals &g, const Plan &P, char *ws)
 {
     // its tiles take one raster pass: the in-tile front pass is followed by a second one
-    if (g.fronts == 1 || P.dense < HEAVY_FACES_PER_TILE) return;
+    if (g.fronts == 1 || P.view_faces < SMALL_FACES) return;
+    const int tiles = P.lay.total_tiles;
+    if (tiles <= SMALL_TILES) {
+        // fewer tiles than the GPU has CTAs: those with faces to share take several each
+        g.heavy_min = SMALL_MIN;
+        g.heavy_ctas = tiles <= SMALL_TILES / 4 ? 8 : tiles <= SMALL_TILES / 2 ? 4 : 2;
+    } else if (tiles <= 2 * HEAVY_CTAS) {
+        g.heavy_min = 256;
+        g.heavy_ctas = 8;
+    } else if (P.dense >= 512) {   // faces per tile
+        g.heavy_min = 1024;
+        g.heavy_ctas = 8;
+    } else {
+        return;
+    }
     g.heavy_cap = (int)std::min<long long>(HEAVY_MAX, 4 * P.lay.n_vrec - 1);
     if (g.heavy_cap > 0) g.heavy = reinterpret_cast<int *>(ws + P.lay.sgrad);
 }

@@ -168,7 +168,7 @@ struct Globals {
                           // ones come 1 from the tiles' rasters, 2 from the face table kernel (in kth)
     int *heavy;           // a forward's tiles with long face lists: their number, then the tiles (k_bin
                           // lists them where the host allows it), or nullptr
-    int heavy_cap;
+    int heavy_cap, heavy_min, heavy_ctas;   // the list's room, the shortest long list, CTAs per tile
     int2 *big;            // faces left to k_front_big (view, face), in the tile lists' place
     int big_cap;
     int *big_n;
@@ -334,17 +334,15 @@ __device__ __forceinline__ bool face_get(const Globals &g, const ViewK &V, const
 }
 
 // A tile's face list is long where it is several times the list entries that each of the GPU's CTAs
-// would get of all tiles' lists, and more than a few chunks: alone, the tile would outlast the rest.
+// would get of all tiles' lists, and not too short to share: alone, the tile would outlast the rest.
 // (A 32 px tile of a 200,000-face mesh seen at 128^2 holds 25,000 faces: one CTA took 1.3 ms.)
-constexpr int HEAVY_MIN = 1024;        // entries
 constexpr int HEAVY_SHARE = 2;         // times the entries per CTA
 constexpr int HEAVY_CTAS = 608;        // four CTAs on each of 152 SMs
-constexpr int HEAVY_CLUSTERS = HEAVY_CTAS / 8;
 constexpr int HEAVY_MAX = 1024;        // more long tiles than this keep the GPU busy one CTA each
 
 __device__ __forceinline__ bool long_list(const Globals &g, int t)
 {
-    return g.tile_count[t] > max(HEAVY_MIN, g.tile_off[g.total_tiles] / HEAVY_CTAS * HEAVY_SHARE);
+    return g.tile_count[t] > max(g.heavy_min, g.tile_off[g.total_tiles] / HEAVY_CTAS * HEAVY_SHARE);
 }
 // the listed tiles, none if there are too many
 __device__ __forceinline__ int heavy_count(const Globals &g)

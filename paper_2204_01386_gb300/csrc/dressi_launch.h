@@ -12,20 +12,31 @@ struct Globals;
 // The ten short kernels of a textured 256^2 step idled some 2 us at each: 120 -> 106 us, inverse UV
 // on one 521 x 337 view 129 -> 112, a 1280 x 720 render 128 -> 102.  (Releasing the next kernel at
 // a kernel's start instead of its end: 101, 116 and 111 us.)
+// With clusters of `ctas` blocks (1: none).
 template <typename... P, typename... A>
-inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args)
+inline void launch_clusters(int ctas, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                            A &&...args)
 {
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr = {};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2] = {};
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = ctas;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = ctas > 1 ? 2 : 1;
     cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
+template <typename... P, typename... A>
+inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args)
+{
+    launch_clusters(1, kernel, grid, block, smem, s, std::forward<A>(args)...);
 }
 #ifdef __CUDACC__
 // the kernel's first statement: the grids before it in the stream are complete

@@ -1471,12 +1471,13 @@ __device__ __forceinline__ void add_stats(const Globals &g, unsigned n_pairs, un
 
 // the K-lists, and S^H of a ring of hs x hs (0: none), of a cluster's CTAs into the first one's.  Every
 // candidate was seen by one CTA: the K smallest of the lists' entries are the tile's.
-template <int K, int TT, int CL>
-__device__ __forceinline__ void merge_cluster(Smem &S, unsigned long long *kbuf, int hs, int rank)
+template <int K, int TT>
+__device__ __forceinline__ void merge_cluster(Smem &S, unsigned long long *kbuf, int hs)
 {
     auto cluster = cooperative_groups::this_cluster();
+    const int CL = cluster.num_blocks();
     cluster.sync();   // every list is complete
-    if (rank == 0) {
+    if (cluster.block_rank() == 0) {
         for (int p = threadIdx.x; p < TT * TT; p += blockDim.x) {
             unsigned long long v[K];
 #pragma unroll
@@ -1513,13 +1514,14 @@ __device__ __forceinline__ void merge_cluster(Smem &S, unsigned long long *kbuf,
 // re-rasterizes, 2 adjoint from stored layer ids, 3 forward from stored layer ids
 // (re-shading a static geometry: no binning, raster or peel); 4, 5, 6, 7 = 2, 1, 0, 3
 // with the normal map, the light gradient and the inverse UV compiled in
-// CL > 1: a cluster of CL CTAs works on the tile (a forward with one raster pass): each rasterizes
-// every CL-th chunk of the face list into K-lists of its own, and the first merges them, by
-// distributed shared memory, and goes on alone.
-template <int K, int MODE, int TT, int CL = 1>
+// CLUSTER: the CTAs of a cluster work on the tile (a forward with one raster pass): each rasterizes its
+// chunks of the face list into K-lists of its own, and the first merges them, by distributed shared
+// memory, and goes on alone.
+template <int K, int MODE, int TT, bool CLUSTER = false>
 __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned long long *kbuf, const int t)
 {
-    const int rank = CL > 1 ? (int)cooperative_groups::this_cluster().block_rank() : 0;
+    const int rank = CLUSTER ? (int)cooperative_groups::this_cluster().block_rank() : 0;
+    const int ctas = CLUSTER ? (int)cooperative_groups::this_cluster().num_blocks() : 1;
     constexpr int NT = cta_threads<MODE, TT>();
     constexpr int PPT = TT * TT / NT;   // pixels per thread in the per-pixel phases
     // after the K-lists: the candidate queue and the two pair-block tables
@@ -1617,7 +1619,7 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
             }
         }
         // no raster: nothing for the other CTAs of a cluster
-        if (CL > 1 && rank != 0 && (empty || stage == ST_DONE)) return;
+        if (CLUSTER && rank != 0 && (empty || stage == ST_DONE)) return;
         if (!empty && stage != ST_DONE)   // 16-byte stores (TT^2 K is even; kbuf is 16-byte aligned)
             for (int i = tid; i < TT * TT * K / 2; i += NT)
                 reinterpret_cast<ulonglong2 *>(kbuf)[i] = make_ulonglong2(EMPTY, EMPTY);
@@ -1655,18 +1657,20 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
         // forward 1667 -> 1130 us, the adjoint 1541 -> 764 us (four 768^2 views of 32,000 faces:
         // 310 -> 244 and 350 -> 217 us).
         bool ring = rho > 0 && !handed && !raw;
-        single_chunk = n <= CH && stage != ST_DONE;   // all of the list staged (and hashed) at once
+        single_chunk = !CLUSTER && n <= CH && stage != ST_DONE;   // all of the list staged (and hashed) at once
+        // a cluster shares a list of less than a chunk each evenly, by warps' worth of faces
+        const int ch = CLUSTER ? min(CH, ((n + ctas - 1) / ctas + 31) & ~31) : CH;
         // the id -> slot hash serves the forward's shading of a tile staged in one chunk
         const bool use_hash = !BWD && single_chunk;
         while (stage != ST_DONE && !empty) {
             const float reach = stage == ST_FRONT ? 0.f : V.r_px;
-            for (int c0 = rank * CH; c0 < n; c0 += CH * CL) {
-                const int nch = min(CH, n - c0);
+            for (int c0 = rank * ch; c0 < n; c0 += ch * ctas) {
+                const int nch = min(ch, n - c0);
                 // the next chunk's face ids, loaded under this chunk's staging: their records
                 // are prefetched into L2 once this chunk is staged
-                const int nnext = min(CH, n - c0 - CH * CL);
+                const int cn = c0 + ch * ctas, nnext = min(ch, n - cn);
                 int fnext = -1;
-                if (tid < nnext) fnext = fallback ? c0 + CH * CL + tid : g.lists[lb + c0 + CH * CL + tid];
+                if (tid < nnext) fnext = fallback ? cn + tid : g.lists[lb + cn + tid];
                 __syncthreads();   // previous chunk consumed
                 if (use_hash) {
                     for (int i = tid; i < HASH; i += NT) S.hash[i] = make_int2(-1, -1);
@@ -1785,8 +1789,8 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
                         S.sh[si] = 1;
                 }
             }
-            if constexpr (CL > 1) {
-                merge_cluster<K, TT, CL>(S, kbuf, ring ? hs : 0, rank);
+            if constexpr (CLUSTER) {
+                merge_cluster<K, TT>(S, kbuf, ring ? hs : 0);
                 if (rank != 0) {
                     add_stats(g, n_pairs, n_exact, n_cand, 0u);
                     return;
@@ -2053,14 +2057,11 @@ __global__ void __launch_bounds__(cta_threads<MODE, TT>(), tile_min_ctas<MODE, T
     pull_tiles<K, MODE, TT, false>(g, S, kbuf);
 }
 
-// Persistent, with the tiles of long face lists (k_bin listed them) first, a cluster of CTAs per tile:
-// few against the GPU's CTAs, each of them would take one CTA longer than its share of the whole.
-// The CTAs then pull the other tiles one by one.
-constexpr int HEAVY_CL = 8;
-
+// Persistent, with the tiles of long face lists (k_bin listed them) first, a cluster of CTAs (g.heavy_ctas,
+// of the launch) per tile: few against the GPU's CTAs, each of them would take one CTA longer than
+// its share of the whole.  The CTAs then pull the other tiles one by one.
 template <int K, int MODE, int TT>
-__global__ void __cluster_dims__(HEAVY_CL, 1, 1) __launch_bounds__(cta_threads<MODE, TT>(), tile_min_ctas<MODE, TT>())
-    k_tile_heavy(Globals g)
+__global__ void __launch_bounds__(cta_threads<MODE, TT>(), tile_min_ctas<MODE, TT>()) k_tile_heavy(Globals g)
 {
     grid_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -2069,16 +2070,16 @@ __global__ void __cluster_dims__(HEAVY_CL, 1, 1) __launch_bounds__(cta_threads<M
     auto cluster = cooperative_groups::this_cluster();
     const int n = heavy_count(g);
     while (n > 0) {
-        if (cluster.block_rank() == 0 && threadIdx.x < HEAVY_CL) {
+        if (cluster.block_rank() == 0 && threadIdx.x < 32) {
             int h = 0;
             if (threadIdx.x == 0) h = atomicAdd(g.queue + 2, 1);
-            h = __shfl_sync((1u << HEAVY_CL) - 1u, h, 0);
-            *cluster.map_shared_rank(&S.next, threadIdx.x) = h;
+            h = __shfl_sync(0xffffffffu, h, 0);
+            if (threadIdx.x < cluster.num_blocks()) *cluster.map_shared_rank(&S.next, threadIdx.x) = h;
         }
         cluster.sync();
         const int h = S.next;
         if (h >= n) break;
-        tile_body<K, MODE, TT, HEAVY_CL>(g, S, kbuf, g.heavy[1 + h]);
+        tile_body<K, MODE, TT, true>(g, S, kbuf, g.heavy[1 + h]);
         cluster.sync();   // the tile's shared memory is free again
     }
     __syncthreads();   // S.next has been read
@@ -2158,7 +2159,7 @@ static void launch_heavy_kk(const Globals &g, cudaStream_t s)
         cudaFuncSetAttribute(k_tile_heavy<K, MODE, TT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (dev >= 0 && dev < LAUNCH_MAX_DEVICES) ready[dev].store(true, std::memory_order_release);
     }
-    launch(k_tile_heavy<K, MODE, TT>, HEAVY_CL * HEAVY_CLUSTERS, NT, smem, s, g);
+    launch_clusters(g.heavy_ctas, k_tile_heavy<K, MODE, TT>, HEAVY_CTAS, NT, smem, s, g);
 }
 
 // all tiles, those of g.heavy first and by clusters (modes 0 and 6)

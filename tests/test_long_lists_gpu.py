@@ -28,12 +28,14 @@ def _launches(r, **kw):
     return res, B.load().dressi_launch_count() - c0
 
 
-def _check(s, tile, schedule, store):
+def _check(s, tile, schedule, store, copies=200):
     ps = PackedScene(s.meshes, "cuda")
     v = s.views[0]
     n = v.width * v.height
-    one = Renderer(ps, s.views, s.params, tile=tile, schedule=schedule)
-    many = Renderer(ps, s.views * 200, s.params, tile=tile, schedule=schedule)
+    # room for every entry: past the capacity tiles would take all faces of their view
+    cap = 16 * s.meshes[0].faces.shape[0]
+    one = Renderer(ps, s.views, s.params, tile=tile, schedule=schedule, list_cap=cap)
+    many = Renderer(ps, s.views * copies, s.params, tile=tile, schedule=schedule, list_cap=cap * copies)
     out, ids = one.forward(store_layers=store)
     ref, ref_ids = many.forward(store_layers=store)
     assert torch.equal(out, ref[:n]) and torch.equal(out, ref[-n:])
@@ -59,6 +61,15 @@ def test_long_lists(tile, schedule, K, store):
 def test_long_lists_edges(edge, r_px):
     for store in (True, False):
         _check(_scene(61, 64, edge_mode=edge, r_px=r_px), 32, 2, store)
+
+
+# scenes of few tiles share all but short lists among 8, 4 or 2 CTAs, by their number; batches of more
+# than 1,216 tiles do not
+@pytest.mark.parametrize("W,H,copies", [(90, 66, 45), (200, 150, 10), (300, 250, 5), (420, 400, 2)])
+@pytest.mark.parametrize("K", [2, 4])
+def test_small_scenes(W, H, copies, K):
+    _check(_scene(W, H, K=K), 16, 1, True, copies)
+    _check(_scene(W, H, K=K, subdiv=4, edge_mode=1, r_px=5.0), 16, 2, False, copies)
 
 
 def test_long_lists_normal_map():
