@@ -45,7 +45,7 @@ constexpr int NT_MAX = 256;            // threads per CTA, at most
 template <int MODE, int TT>
 __host__ __device__ constexpr int cta_threads()
 {
-    return 256;
+    return MODE == 8 ? 128 : 256;
 }
 constexpr int TT_MAX = 32;             // tile edges: 16 (one pixel per thread) or 32 (four)
 constexpr int RHO_MAX = 8;             // largest supported edge-mask radius
@@ -1513,7 +1513,8 @@ __device__ __forceinline__ void merge_cluster(Smem &S, unsigned long long *kbuf,
 // everything one CTA does for global tile t.  MODE: 0 forward, 1 adjoint that
 // re-rasterizes, 2 adjoint from stored layer ids, 3 forward from stored layer ids
 // (re-shading a static geometry: no binning, raster or peel); 4, 5, 6, 7 = 2, 1, 0, 3
-// with the normal map, the light gradient and the inverse UV compiled in
+// with the normal map, the light gradient and the inverse UV compiled in; 8 = 2 by CTAs of 128
+// threads
 // CLUSTER: the CTAs of a cluster work on the tile (a forward with one raster pass): each rasterizes its
 // chunks of the face list into K-lists of its own, and the first merges them, by distributed shared
 // memory, and goes on alone.
@@ -1543,9 +1544,9 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
     const int hs = TT + 2 * rho;
     const int wlim = min(TT, V.W - X0), hlim = min(TT, V.H - Y0);   // tile part inside the image
 
-    constexpr bool EXTRA = MODE >= 4;
-    constexpr bool BWD = MODE == 1 || MODE == 2 || MODE == 4 || MODE == 5;
-    constexpr bool from_ids = MODE == 2 || MODE == 3 || MODE == 4 || MODE == 7;
+    constexpr bool EXTRA = MODE >= 4 && MODE <= 7;
+    constexpr bool BWD = MODE == 1 || MODE == 2 || MODE == 4 || MODE == 5 || MODE == 8;
+    constexpr bool from_ids = MODE == 2 || MODE == 3 || MODE == 4 || MODE == 7 || MODE == 8;
     const bool light_grad = EXTRA && g.glight != nullptr && g.shade_mode >= 2;
     float *glacc = light_grad ? gl_slots[tid] : nullptr;
     if (light_grad) glacc[0] = glacc[1] = glacc[2] = 0.f;
@@ -1900,7 +1901,7 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
                 l2acc += dx * dx + dy * dy + dz * dz + dw * dw;
             }
         }
-    } else if constexpr (MODE == 2) {
+    } else if constexpr (MODE == 2 || MODE == 8) {
         // the adjoint from stored ids: a round's front ids and dL/dI are loaded under the round
         // before it
         int id0 = -1;
@@ -2017,7 +2018,7 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
 template <int MODE, int TT>
 constexpr int tile_min_ctas()
 {
-    return (MODE == 2 || MODE == 4) ? 2 : (MODE == 1 || MODE == 5) ? 3 : 4;
+    return (MODE == 2 || MODE == 4) ? 2 : (MODE == 1 || MODE == 5) ? 3 : 4;   // (mode 8: of 128 threads)
 }
 
 template <int K, int MODE, int TT>
@@ -2092,7 +2093,7 @@ constexpr size_t tile_smem_bytes()
     // from stored ids: the first part of Smem; otherwise Smem, the K-lists, the
     // candidate queue, the two pair-block tables; the adjoints with extras add the
     // per-thread dL/dlight slots
-    return (MODE == 2 || MODE == 3 || MODE == 4 || MODE == 7
+    return (MODE == 2 || MODE == 3 || MODE == 4 || MODE == 7 || MODE == 8
                 ? offsetof(Smem, F)
                 : sizeof(Smem) + sizeof(unsigned long long) * TT * TT * K +
                       sizeof(unsigned) * WQ * cta_threads<MODE, TT>() / 32 + 2 * NBLK) +
@@ -2201,7 +2202,8 @@ static void launch_k(const Globals &g, cudaStream_t s)
 template <int MODE>
 void launch_tile_mode(const Globals &g, cudaStream_t s)
 {
-    if (g.tile == 32) launch_k<MODE, 32>(g, s);
+    if constexpr (MODE == 8) launch_k<MODE, 16>(g, s);
+    else if (g.tile == 32) launch_k<MODE, 32>(g, s);
     else launch_k<MODE, 16>(g, s);
 }
 
