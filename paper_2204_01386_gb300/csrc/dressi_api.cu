@@ -624,6 +624,12 @@ int dressi_forward_from_layers(const dressi_scene *scene, const dressi_view *vie
 // adjoint 933 us, with their lines fetched ahead 697 us.  Where it fits (1024^2: 16 MB), the
 // prefetches cost 2 %: 368 -> 377 us.
 constexpr long long GRAD_PREFETCH_BYTES = 64LL << 20;
+// View pixels per face past which the adjoint from ids sums the gradients of a warp at one face before
+// it adds them to the corners' accumulators, which every pixel of the face shares.  us without / with:
+//   7,363 (320 faces, 1365 x 1726) 1191 / 243      383 (1,280 faces, 700^2) 128 / 81
+//   819 (320 faces, 512^2) 58 / 43                 205 (5,120 faces, 1024^2) 82 / 78
+//   13 (20,480 faces, 24 views of 512^2) 370 / 389: the kernel that can is slower where no warp is
+constexpr long long BIG_FACE_PX = 256;
 
 int dressi_backward(const dressi_scene *scene, const dressi_view *views, int32_t n_views,
                     const dressi_params *params, const float *grad_rgba, const int32_t *layer_ids, int64_t n_pix,
@@ -660,6 +666,7 @@ int dressi_backward_ex(const dressi_scene *scene, const dressi_view *views, int3
     const bool gather = tex_records && params->texgrad_mode == 1;
     const bool inv_uv = tex_records && params->texgrad_mode == 2;
     if (!tex_records) g.texgrad_mode = 0;
+    g.big_faces = P.view_pixels > BIG_FACE_PX * P.view_faces;
     g.grad_prefetch = g.gtex && g.texgrad_mode == 0 && P.n_texels * 16 > GRAD_PREFETCH_BYTES;
     // the outputs and accumulators, in one launch (a memset each costs a small call more than
     // its bytes); past 16 MB a range goes by cudaMemsetAsync, which alone reaches the full rate

@@ -185,6 +185,7 @@ struct Globals {
     float4 *sgrad;        // per (view, vertex): dX, dY, d(1/w)
     float4 *ngrad;        // [n_verts_total] gradient of the normalized vertex normals
     float *gpos, *gcol, *gtex;
+    int big_faces;        // whole warps at one face are common: their gradients are summed first
     int grad_prefetch;    // the texel gradient is larger than L2: lines are fetched ahead of the reductions
     float *gmvp;          // [n_views][16] dL/dMVP or nullptr
     float *gntex;         // shade_mode 3: [sum texels][4] normal-map texel gradient or nullptr

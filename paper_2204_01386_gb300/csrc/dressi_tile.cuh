@@ -386,13 +386,32 @@ __device__ __forceinline__ bool layer_build(const Globals &g, const ViewK &V, co
     return face_get(g, V, M, id, L.R) && layer_eval<X, ADJ>(g, V, M, px, py, front, L);
 }
 
+// adds v to *p (its x, y, z).  same: all lanes of the warp hold the same p; where they are all here, the
+// warp adds its sum once instead of 32 times (one face fills the warp's pixels: its corners'
+// accumulators would take every pixel's reduction one after another)
+template <bool SAME>
+__device__ __forceinline__ void reduce_add(float4 *p, float x, float y, float z, bool same)
+{
+    const unsigned FULL = 0xffffffffu;
+    if (SAME && same && __activemask() == FULL) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            x += __shfl_xor_sync(FULL, x, o);
+            y += __shfl_xor_sync(FULL, y, o);
+            z += __shfl_xor_sync(FULL, z, o);
+        }
+        if ((threadIdx.x & 31) != 0) return;
+    }
+    atomicAdd(p, make_float4(x, y, z, 0.f));
+}
+
 // ---------------------------------------------------------------------------
 // adjoint of one layer: gC = dL/dC_k, gD = dL/dD_k
 // ---------------------------------------------------------------------------
 // gl: this thread's dL/dlight accumulator, or nullptr.  Returns true when it stored
 // the sample's dL/d(albedo) in its record slot (texgrad_mode 2, the inverse UV).  EXTRA
 // compiles the light gradient and the inverse UV in (the adjoint without them is leaner).
-template <bool EXTRA>
+template <bool EXTRA, bool SAME>
 __device__ __forceinline__ bool layer_adjoint(const Globals &g, const ViewK &V, const MeshK &M, const Layer &L,
                                               float px, float py, const float gC[3], float gD, long long slot,
                                               float *gl)
@@ -408,6 +427,14 @@ __device__ __forceinline__ bool layer_adjoint(const Globals &g, const ViewK &V, 
         dy[i] = fsub(fsub(py, R.c[i].yh), R.c[i].yl);
     }
     float gX[3] = {0.f, 0.f, 0.f}, gY[3] = {0.f, 0.f, 0.f}, gW[3] = {0.f, 0.f, 0.f};
+    // whether the whole warp is at one face (the same corners in the same order)
+    bool same = false;
+    if (SAME && __activemask() == 0xffffffffu) {
+        bool eq = true;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) eq &= S.vi[i] == __shfl_sync(0xffffffffu, S.vi[i], 0);
+        same = __all_sync(0xffffffffu, eq);
+    }
     const float o = (R.flags & 1) ? 1.f : -1.f;
 
     // sigmoid -> signed distance -> corners (closest feature)
@@ -452,7 +479,7 @@ __device__ __forceinline__ bool layer_adjoint(const Globals &g, const ViewK &V, 
                 // dL/dcolour in the normals' accumulator, which this mode does not use: one 16-byte
                 // reduction per corner instead of three 4-byte ones (16 views of 224^2, K = 5:
                 // see k_vertex_bwd, which writes the planes)
-                if (g.gcol) atomicAdd(g.ngrad + gi, make_float4(S.b[i] * gC[0], S.b[i] * gC[1], S.b[i] * gC[2], 0.f));
+                if (g.gcol) reduce_add<SAME>(g.ngrad + gi, S.b[i] * gC[0], S.b[i] * gC[1], S.b[i] * gC[2], same);
 #pragma unroll
                 for (int c = 0; c < 3; ++c) gb[i] = fmaf(gC[c], __ldg(g.col + c * nvt + gi), gb[i]);
             }
@@ -551,7 +578,7 @@ __device__ __forceinline__ bool layer_adjoint(const Globals &g, const ViewK &V, 
                     for (int i = 0; i < 3; ++i) {
                         const long long gi = M.vert_off + S.vi[i];
                         const float4 nv = g.nrm[gi];
-                        atomicAdd(g.ngrad + gi, make_float4(S.b[i] * gm[0], S.b[i] * gm[1], S.b[i] * gm[2], 0.f));
+                        reduce_add<SAME>(g.ngrad + gi, S.b[i] * gm[0], S.b[i] * gm[1], S.b[i] * gm[2], same);
                         gb[i] += gm[0] * nv.x + gm[1] * nv.y + gm[2] * nv.z;
                     }
                 }
@@ -643,7 +670,7 @@ __device__ __forceinline__ bool layer_adjoint(const Globals &g, const ViewK &V, 
     float4 *sg = g.sgrad + V.vrec_off;
 #pragma unroll
     for (int i = 0; i < 3; ++i)
-        if (gX[i] != 0.f || gY[i] != 0.f || gW[i] != 0.f) atomicAdd(sg + S.vi[i], make_float4(gX[i], gY[i], gW[i], 0.f));
+        if ((SAME && same) || gX[i] != 0.f || gY[i] != 0.f || gW[i] != 0.f) reduce_add<SAME>(sg + S.vi[i], gX[i], gY[i], gW[i], same);
     return stored;
 }
 
@@ -1031,7 +1058,7 @@ __device__ __forceinline__ unsigned adjoint_pixel(const Globals &g, const Smem &
         const long long slot = (V.slot_base + (long long)Y * V.W + X) * K + k;
         if (any && layer_build<EXTRA, true>(g, V, M, ids[k], px, py, false, L)) {
             ++layers;
-            if (layer_adjoint<EXTRA>(g, V, M, L, px, py, gCl, gDl, slot, gl)) stored |= 1u << k;
+            if (layer_adjoint<EXTRA, false>(g, V, M, L, px, py, gCl, gDl, slot, gl)) stored |= 1u << k;
         }
     }
     if (inv) {
@@ -1191,7 +1218,7 @@ __device__ __forceinline__ unsigned finish_forward(const Globals &g, const Smem 
 // CTA-wide layer queue, which this replaced for the stored-ids adjoint, filled its lanes
 // better at the silhouettes but held all warps at its barriers.
 // ids: a pixel's layers (0x7fffffff none); outside the edge mask only the front one is read.
-template <int K, int TT>
+template <int K, int TT, bool SAME>
 __device__ __forceinline__ unsigned adjoint_warp(const Globals &g, const Smem &S, const ViewK &V, const MeshK &M,
                                                  int X0, int Y0, int p, bool in, const int (&ids)[K], float4 gi4)
 {
@@ -1319,7 +1346,7 @@ __device__ __forceinline__ unsigned adjoint_warp(const Globals &g, const Smem &S
                 Layer L;
                 if (layer_build<false, true>(g, V, M, id, px, py, !anyE, L)) {
                     ++layers;
-                    layer_adjoint<false>(g, V, M, L, px, py, gC, gD, slot, nullptr);
+                    layer_adjoint<false, SAME>(g, V, M, L, px, py, gC, gD, slot, nullptr);
                 }
             }
         }
@@ -1514,7 +1541,7 @@ __device__ __forceinline__ void merge_cluster(Smem &S, unsigned long long *kbuf,
 // re-rasterizes, 2 adjoint from stored layer ids, 3 forward from stored layer ids
 // (re-shading a static geometry: no binning, raster or peel); 4, 5, 6, 7 = 2, 1, 0, 3
 // with the normal map, the light gradient and the inverse UV compiled in; 8 = 2 by CTAs of 128
-// threads
+// threads; 9 = 2 for big faces
 // CLUSTER: the CTAs of a cluster work on the tile (a forward with one raster pass): each rasterizes its
 // chunks of the face list into K-lists of its own, and the first merges them, by distributed shared
 // memory, and goes on alone.
@@ -1545,8 +1572,8 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
     const int wlim = min(TT, V.W - X0), hlim = min(TT, V.H - Y0);   // tile part inside the image
 
     constexpr bool EXTRA = MODE >= 4 && MODE <= 7;
-    constexpr bool BWD = MODE == 1 || MODE == 2 || MODE == 4 || MODE == 5 || MODE == 8;
-    constexpr bool from_ids = MODE == 2 || MODE == 3 || MODE == 4 || MODE == 7 || MODE == 8;
+    constexpr bool BWD = MODE == 1 || MODE == 2 || MODE == 4 || MODE == 5 || MODE == 8 || MODE == 9;
+    constexpr bool from_ids = MODE == 2 || MODE == 3 || MODE == 4 || MODE == 7 || MODE == 8 || MODE == 9;
     const bool light_grad = EXTRA && g.glight != nullptr && g.shade_mode >= 2;
     float *glacc = light_grad ? gl_slots[tid] : nullptr;
     if (light_grad) glacc[0] = glacc[1] = glacc[2] = 0.f;
@@ -1901,7 +1928,7 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
                 l2acc += dx * dx + dy * dy + dz * dz + dw * dw;
             }
         }
-    } else if constexpr (MODE == 2 || MODE == 8) {
+    } else if constexpr (MODE == 2 || MODE == 8 || MODE == 9) {
         // the adjoint from stored ids: a round's front ids and dL/dI are loaded under the round
         // before it
         int id0 = -1;
@@ -1931,7 +1958,7 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
                     if (id != -1) ids[k] = id & 0x7fffffff;
                 }
             }
-            n_layers += adjoint_warp<K, TT>(g, S, V, M, X0, Y0, p, lx < wlim && ly < hlim, ids, gj);
+            n_layers += adjoint_warp<K, TT, MODE == 9>(g, S, V, M, X0, Y0, p, lx < wlim && ly < hlim, ids, gj);
         }
     } else for (int j = 0; j < PPT; ++j) {
         const int p = tid + j * NT;
@@ -1982,7 +2009,7 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
             float4 gi4 = make_float4(0.f, 0.f, 0.f, 0.f);
             if (in && (row_bit(S.eb, lx, ly) || row_bit(S.hb, lx, ly)))
                 gi4 = __ldg(reinterpret_cast<const float4 *>(g.gin) + V.pix_off + (long long)(Y0 + ly) * V.W + (X0 + lx));
-            n_layers += adjoint_warp<K, TT>(g, S, V, M, X0, Y0, p, in, ids, gi4);
+            n_layers += adjoint_warp<K, TT, false>(g, S, V, M, X0, Y0, p, in, ids, gi4);
         } else if constexpr (BWD)
             n_layers += adjoint_pixel<K, TT, EXTRA>(g, S, V, M, X0, Y0, lx, ly, ids, glacc);
         else
@@ -2018,7 +2045,7 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
 template <int MODE, int TT>
 constexpr int tile_min_ctas()
 {
-    return (MODE == 2 || MODE == 4) ? 2 : (MODE == 1 || MODE == 5) ? 3 : 4;   // (mode 8: of 128 threads)
+    return (MODE == 2 || MODE == 4 || MODE == 9) ? 2 : (MODE == 1 || MODE == 5) ? 3 : 4;   // (mode 8: of 128 threads)
 }
 
 template <int K, int MODE, int TT>
@@ -2093,7 +2120,7 @@ constexpr size_t tile_smem_bytes()
     // from stored ids: the first part of Smem; otherwise Smem, the K-lists, the
     // candidate queue, the two pair-block tables; the adjoints with extras add the
     // per-thread dL/dlight slots
-    return (MODE == 2 || MODE == 3 || MODE == 4 || MODE == 7 || MODE == 8
+    return (MODE == 2 || MODE == 3 || MODE == 4 || MODE == 7 || MODE == 8 || MODE == 9
                 ? offsetof(Smem, F)
                 : sizeof(Smem) + sizeof(unsigned long long) * TT * TT * K +
                       sizeof(unsigned) * WQ * cta_threads<MODE, TT>() / 32 + 2 * NBLK) +

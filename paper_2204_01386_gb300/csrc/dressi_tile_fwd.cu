@@ -9,6 +9,7 @@ extern template void launch_tile_mode<4>(const Globals &g, cudaStream_t s);
 extern template void launch_tile_mode<5>(const Globals &g, cudaStream_t s);
 extern template void launch_tile_mode<6>(const Globals &g, cudaStream_t s);
 extern template void launch_tile_mode<8>(const Globals &g, cudaStream_t s);
+extern template void launch_tile_mode<9>(const Globals &g, cudaStream_t s);
 
 // 16 px tiles past this number: the adjoint from ids takes CTAs of 128 threads, so that more tiles
 // are in flight and hide each other's starts (us by 256 / 128 threads: 8,192 tiles 176 / 147, five
@@ -23,6 +24,7 @@ void launch_tile(const Globals &g, bool backward, cudaStream_t s)
     const bool extra = (g.glight != nullptr && g.shade_mode >= 2) || g.texgrad_mode == 2 || g.shade_mode == 3;
     if (!backward) g.shade_mode == 3 ? launch_tile_mode<6>(g, s) : launch_tile_mode<0>(g, s);
     else if (g.ids_in && extra) launch_tile_mode<4>(g, s);
+    else if (g.ids_in && g.big_faces) launch_tile_mode<9>(g, s);
     else if (g.ids_in && g.tile == 16 && g.total_tiles > MANY_TILES) launch_tile_mode<8>(g, s);
     else if (g.ids_in) launch_tile_mode<2>(g, s);
     else extra ? launch_tile_mode<5>(g, s) : launch_tile_mode<1>(g, s);
