@@ -1,6 +1,7 @@
 // dressi_tile.cuh -- the per-tile hot kernel of HardSoftRas, forward and adjoint
 // (included by one translation unit per mode: dressi_tile_fwd.cu, _bwd.cu, _ids.cu,
-// _cached.cu, _extra_ids.cu, _extra_bwd.cu, _nmap_fwd.cu, _nmap_cached.cu).
+// _cached.cu, _extra_ids.cu, _extra_bwd.cu, _nmap_fwd.cu, _nmap_cached.cu, _heavy.cu,
+// _nmap_heavy.cu, _ids_many.cu, _ids_big.cu).
 //
 // One CTA owns one TT x TT pixel tile of one view (TT = 16 or 32; 256 threads).  Per CTA:
 //   1. the tile's face list is staged in shared memory, CH faces at a time, from the
@@ -23,10 +24,9 @@
 //      bilinear texture, Lambert or normal map) the layers its pixels blend as one list,
 //      and each pixel blends them (D_k = sigmoid(dist/sigma), colour and silhouette
 //      equations of Sec. 3.4.3), optionally with the L2 loss; adjoint: the same values are
-//      rebuilt by warp lists, and
-//      dL/dI is pushed back to the screen-space corners, vertex colours, vertex normals,
-//      texels, the camera and the light.
-// With layer ids stored by the forward (modes 2, 3, 4, 7), steps 1-3 are skipped: S^H of
+//      rebuilt by warp lists, and dL/dI is pushed back to the screen-space corners, vertex
+//      colours, vertex normals, texels, the camera and the light.
+// With layer ids stored by the forward (modes 2, 3, 4, 7, 8, 9), steps 1-3 are skipped: S^H of
 // the tile and its ring is the stored front layer's hard flag.
 #pragma once
 #include "dressi_core.cuh"
