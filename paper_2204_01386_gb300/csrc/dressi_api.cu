@@ -704,15 +704,13 @@ int dressi_backward_ex(const dressi_scene *scene, const dressi_view *views, int3
         g.fronts = only ? 1 : 0;
         if (!layer_ids) g.kth = reinterpret_cast<unsigned long long *>(w + P.lay.kth);
     } else {
-        Clears clr;
         choose_fronts(g, P, only, w, s);
-        if (g.fronts == 2) {
-            g.kth = reinterpret_cast<unsigned long long *>(w + P.lay.kth);
-            clr.p[0] = g.kth_flag;
-            clr.n[0] = 1;
-            clr.v[0] = KTH_RAW;
-        }
-        run_setup(g, P, w, layer_ids == nullptr, clr, g.fronts == 2 ? 1 : 0, s);
+        if (g.fronts == 2) g.kth = reinterpret_cast<unsigned long long *>(w + P.lay.kth);
+        Clears clr;   // an earlier forward's words are of another setup
+        clr.p[0] = g.kth_flag;
+        clr.n[0] = 1;
+        clr.v[0] = g.fronts == 2 ? KTH_RAW : KTH_NONE;
+        run_setup(g, P, w, layer_ids == nullptr, clr, 1, s);
     }
     run_tiles(g, P, w, layer_ids == nullptr, 1, s);
     if (gather)

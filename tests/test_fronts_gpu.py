@@ -91,3 +91,25 @@ def test_fronts_from_the_face_table(tile, schedule, K, edge, W, H):
     views = [synth.View(synth.camera_mvp(e, W, H), 0, W, H) for e in ((0, 0, 3), (0.5, 0.4, 2.9))]
     s = synth.Scene("front_words", [m], views, synth.Params(K=K, r=r, sigma=r / 7, delta=r, edge_mode=edge))
     _check(s, tile, schedule)
+
+
+@pytest.mark.parametrize("subdiv", [3, 6])
+def test_words_of_an_earlier_setup_are_not_used(subdiv):
+    """forward without ids, then moved positions: a rebuilding adjoint and the reusing one after it
+    (which finds the rebuilt setup, not the forward's words) agree."""
+    W, H = 90, 70
+    pos, f = synth.icosphere(subdiv)
+    m = synth.Mesh(synth.displace(pos, 0.1, 3).astype(np.float32), f,
+                   col=np.random.default_rng(0).random((pos.shape[0], 3)).astype(np.float32))
+    r = 2.0 / W
+    s = synth.Scene("moved", [m], [synth.View(synth.camera_mvp((0, 0, 3), W, H), 0, W, H)],
+                    synth.Params(K=3, r=r, sigma=r / 7, delta=r))
+    ps = PackedScene(s.meshes, "cuda")
+    rr = Renderer(ps, s.views, s.params)
+    out, _ = rr.forward(store_layers=False)
+    ps.pos.mul_(0.8)
+    g = torch.randn(out.shape, device="cuda", generator=torch.Generator(device="cuda").manual_seed(3))
+    want = [t.clone() for t in rr.backward(g, ids=None, reuse_setup=False) if t is not None]
+    got = [t for t in rr.backward(g, ids=None) if t is not None]
+    for a, b in zip(got, want):
+        assert _rel(a, b) < 1e-5
