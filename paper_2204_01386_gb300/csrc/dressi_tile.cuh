@@ -2096,7 +2096,10 @@ __global__ void __launch_bounds__(cta_threads<MODE, TT>(), tile_min_ctas<MODE, T
     Smem &S = *reinterpret_cast<Smem *>(smem_raw);
     unsigned long long *kbuf = reinterpret_cast<unsigned long long *>(smem_raw + sizeof(Smem));
     auto cluster = cooperative_groups::this_cluster();
-    const int n = heavy_count(g);
+    const int n = heavy_count(g);   // the same in every CTA
+    // the first CTA writes into the others' shared memory below: only once all of them run
+    // (grid_wait holds each CTA by itself)
+    if (n > 0) cluster.sync();
     while (n > 0) {
         if (cluster.block_rank() == 0 && threadIdx.x < 32) {
             int h = 0;
