@@ -336,7 +336,7 @@ static void run_setup(Globals &g, const Plan &P, char *ws, bool need_bins, Clear
 // Whether a pass without stored layer ids needs the layers behind the front one only inside the
 // edge mask (outside it a pixel shows its front hard layer alone).  Not where the mask is
 // everywhere; not for the inverse UV, which samples a soft front layer outside the mask too; and
-// keys have to stay below 2 for the words that the forward leaves (r < 2 screens).
+// soft keys have to stay below 2 for the words that the forward leaves (r < 2 screens).
 static bool fronts_only(const dressi_params *p)
 {
     const bool inv_uv = p->texgrad_mode == 2 && p->shade_mode != 0;

@@ -36,9 +36,11 @@ constexpr int FLAG_ODD = 1 << 9;    // the record's corner order is an odd permu
 constexpr unsigned long long EMPTY = ~0ULL;
 // A pixel's word in the workspace (*kth_flag says which): nothing; KTH_LAST the K-th (key, id) of every
 // pixel; KTH_RAW its front hard (key, id), WORD_NONE for none, as the face table kernel left it;
-// KTH_FRONTS the same, but E, S^H and the K-th (key, id) (all ones: none) where E = 1.  Keys of these
-// forms are below 2 (r < 2 screens): the two top bits are free.  WORD_NONE is one byte repeated
-// (it is filled in), above every hard key.
+// KTH_FRONTS the same, but E, S^H and the K-th (key, id) (all ones: none) where E = 1.  The two flags
+// take the top bits of keys of 2 and more.  Soft keys are below 2 (r < 2 screens) and so are a hard
+// fragment's, half its depth, as a rule; but where a face is so thin that its area is rounding noise its
+// interpolated depth is anything, and such an entry is left out of the word.  WORD_NONE is one byte
+// repeated (it is filled in), above every hard key of a depth up to 1.
 constexpr int KTH_NONE = 0, KTH_LAST = 1, KTH_RAW = 2, KTH_FRONTS = 3;
 constexpr int WORD_FILL = 0x3f;
 constexpr unsigned long long WORD_NONE = 0x3f3f3f3f3f3f3f3full;

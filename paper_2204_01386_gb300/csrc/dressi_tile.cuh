@@ -1890,7 +1890,9 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
                 if (g.fronts) {
                     const bool E = row_bit(S.eb, lx, ly), SH = row_bit(S.hb, lx, ly);
                     if (raw && !E) continue;   // the front word is there
-                    w = E ? (w & WORD_BITS) | WORD_E | (SH ? WORD_SH : 0ull) : SH ? slots[0] : WORD_NONE;
+                    // a K-th entry whose key needs the flags' bits (2 or more: a sliver's) is no use as a seed
+                    if (w & ~WORD_BITS) w = WORD_BITS;
+                    w = E ? w | WORD_E | (SH ? WORD_SH : 0ull) : SH ? slots[0] : WORD_NONE;
                 }
                 g.kth[V.slot_base + (long long)(Y0 + ly) * V.W + (X0 + lx)] = w;
             }
