@@ -40,7 +40,7 @@ constexpr unsigned long long EMPTY = ~0ULL;
 // take the top bits of keys of 2 and more.  Soft keys are below 2 (r < 2 screens) and so are a hard
 // fragment's, half its depth, as a rule; but where a face is so thin that its area is rounding noise its
 // interpolated depth is anything, and such an entry is left out of the word.  WORD_NONE is one byte
-// repeated (it is filled in), above every hard key of a depth up to 1.
+// repeated (it is filled in), above every front word: their keys are at most 1/2 (front_pixel).
 constexpr int KTH_NONE = 0, KTH_LAST = 1, KTH_RAW = 2, KTH_FRONTS = 3;
 constexpr int WORD_FILL = 0x3f;
 constexpr unsigned long long WORD_NONE = 0x3f3f3f3f3f3f3f3full;

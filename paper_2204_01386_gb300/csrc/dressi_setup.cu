@@ -314,8 +314,12 @@ __device__ __forceinline__ bool front_rect(const ViewK &V, const FaceGeo &R, int
 __device__ __forceinline__ void front_pixel(const ViewK &V, const FaceGeo &R, int f, int x, int y, unsigned long long *words)
 {
     Frag fr;
-    if (eval_face<false>(R, (float)x + 0.5f, (float)y + 0.5f, 0.f, V.half_inv_S, fr, true))
-        atomicMin(words + (long long)y * V.W + x, pack_frag(fr.key, f));
+    if (eval_face<false>(R, (float)x + 0.5f, (float)y + 0.5f, 0.f, V.half_inv_S, fr, true)) {
+        // a key of 1/2 or more (the far plane; the noise of a sliver's depth) is stored as 1/2: the pixel is
+        // covered (word_hard) and its tile decided from all layers (word_tie), whatever the value
+        const unsigned long long v = pack_frag(fr.key, f), tie = pack_frag(0.5f, f);
+        atomicMin(words + (long long)y * V.W + x, v < tie ? v : tie);
+    }
 }
 
 // a face's pixels by its own lane: each row of the box cut to where the three cross products, linear
