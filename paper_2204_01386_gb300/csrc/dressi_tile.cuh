@@ -124,7 +124,7 @@ struct Shade {
     int vi[3];
     float iw[3];
     int odd;              // the record's corner order is an odd permutation of the face's
-    float lam[3], b[3], iQ;   // iQ: 1 / sum lam_i / w_i
+    float lam[3], b[3], Q;    // Q: sum lam_i / w_i
     float C[3];
     float D;                  // not set for a layer built as a front one
     // texture
@@ -272,9 +272,10 @@ __device__ __forceinline__ void shade(const Globals &g, const ViewK &V, const Me
     float q[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) q[i] = fmul(S.lam[i], S.iw[i]);
-    S.iQ = __fdividef(1.f, fadd(fadd(q[0], q[1]), q[2]));   // 2 ulp
+    S.Q = fadd(fadd(q[0], q[1]), q[2]);
+    const float iQ = __fdividef(1.f, S.Q);   // 2 ulp
 #pragma unroll
-    for (int i = 0; i < 3; ++i) S.b[i] = fmul(q[i], S.iQ);
+    for (int i = 0; i < 3; ++i) S.b[i] = fmul(q[i], iQ);
     const long long nvt = g.n_verts_total;
     if (g.shade_mode == 0) {
 #pragma unroll
@@ -617,10 +618,11 @@ __device__ __forceinline__ bool layer_adjoint(const Globals &g, const ViewK &V, 
         }
         // perspective-correct barycentrics: b_i = q_i / Q, q_i = lam_i / w_i
         const float bdot = S.b[0] * gb[0] + S.b[1] * gb[1] + S.b[2] * gb[2];
+        const float iQ = 1.f / S.Q;
         float glam[3];
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            const float gq = (gb[i] - bdot) * S.iQ;
+            const float gq = (gb[i] - bdot) * iQ;
             glam[i] = gq * S.iw[i];
             gW[i] += gq * S.lam[i];
         }
