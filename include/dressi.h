@@ -126,8 +126,11 @@ typedef struct {
                              2 inverse UV (Sec. 3.3.2, Alg. 1; approximate: each texel takes the
                              dL/d(albedo) of the last shaded sample that lands on it) */
     int32_t tile;       /* tile edge in pixels: 16 or 32; 0 = 16 */
-    int32_t schedule;   /* per-tile kernel: 0 auto (= 1), 1 one CTA per tile, 2 persistent CTAs
-                           pulling (view, tile) items longest face list first */
+    int32_t schedule;   /* per-tile kernel: 0 auto, 1 one CTA per tile, 2 persistent CTAs pulling
+                           (view, tile) items longest face list first.  Auto is 1, but a forward
+                           of few tiles or with very long face lists, there and with 2, gives the
+                           tiles of long lists to clusters of 2 to 8 CTAs each and the others to
+                           persistent CTAs.  Results do not depend on it */
     int64_t list_cap;   /* tile-list capacity in entries; 0 = library default
                            max(4 x faces over all views, 64 x tiles).  Clamped to
                            2^31 - 2.  A tile whose list ends past it falls back to the

@@ -380,8 +380,9 @@ static void choose_fronts(Globals &g, const Plan &P, bool only, char *ws, cudaSt
 //   8 views of 2048^2 of 1.31 M faces (32,768): no long list, 1596 / 1657 -- hence 512 faces per tile
 constexpr int SMALL_TILES = 512, SMALL_MIN = 96, SMALL_FACES = 2048;
 
-static void allow_heavy(Globals &g, const Plan &P, char *ws)
+static void allow_heavy(Globals &g, const Plan &P, const dressi_params *p, char *ws)
 {
+    if (p->schedule == 1) return;   // one CTA per tile is asked for
     // its tiles take one raster pass: the in-tile front pass is followed by a second one
     if (g.fronts == 1 || P.view_faces < SMALL_FACES) return;
     const int tiles = P.lay.total_tiles;
@@ -409,7 +410,7 @@ static Clears keep_kth(Globals &g, const Plan &P, const dressi_params *p, char *
     const bool keep = g.ids == nullptr;
     g.kth = keep ? reinterpret_cast<unsigned long long *>(ws + P.lay.kth) : nullptr;
     choose_fronts(g, P, keep && fronts_only(p), ws, s);
-    allow_heavy(g, P, ws);
+    allow_heavy(g, P, p, ws);
     Clears clr;
     clr.p[0] = reinterpret_cast<int *>(ws + P.lay.kth_flag);
     clr.n[0] = 1;
