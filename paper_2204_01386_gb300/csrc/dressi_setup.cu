@@ -829,11 +829,18 @@ constexpr long long GRID_BLOCKS = 8192;
 // blocks along x for `rows` grid rows whose longest takes n: the rows of a ragged batch are mostly far
 // shorter, and past some thousands of blocks those without work cost more than a second round of
 // the others (32 meshes of 1,000 to 200,000 faces, us without / at 8,192 / at 4,096 blocks: face table
-// 85 / 53 / 60, list fill 52 / 32 / 38, end of the adjoint 60 / 35 / 50)
+// 85 / 53 / 60, list fill 52 / 32 / 38, end of the adjoint 60 / 35 / 50).  But a thread of the longest row
+// takes eight items at most: one long row among many short ones would keep a few blocks busy alone
+// (63 meshes of 320 faces and one of 1.31 M, at most 80 / 16 / 8 / 4 items: face table 427 / 157 / 141 / 141,
+// list fill 398 / 195 / 183 / 183, end of the adjoint 405 / 203 / 141 / 141; 255 and one of 327,680: face table
+// 151 / 105 / 108 / 171).
+constexpr int GRID_ITEMS = 8;
+
 static int grid_rows(long long n, int block, int cap, int rows)
 {
     int x = grid_x(n, block, cap);
-    while (x > 64 && (long long)x * rows > GRID_BLOCKS) x = (x + 1) / 2;
+    const long long least = std::max<long long>(64, n / ((long long)block * GRID_ITEMS));
+    while (x > least && (long long)x * rows > GRID_BLOCKS) x = (x + 1) / 2;
     return x;
 }
 
