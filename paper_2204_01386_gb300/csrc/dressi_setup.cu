@@ -273,10 +273,14 @@ __device__ __forceinline__ void bin_walk(const Globals &g, const ViewK &V, int f
             if (PASS == 0) {
                 if (lane == leader) atomicAdd(g.tile_count + t, __popc(grp));
             } else {
+                // the list's start loads under the reservation.  (Read after it, as the compiler has to where
+                // the kernel writes other integers too, k_bin took 14.4 instead of 13.3 us for 15,000 faces
+                // at 1024^2 and 1278 instead of 1211 us for two faces over 4,096 tiles.)
+                const int off = __ldg(g.tile_off + t);
                 int base = 0;
                 if (lane == leader) base = atomicAdd(g.tile_cursor + t, __popc(grp));
                 base = __shfl_sync(grp, base, leader) + __popc(grp & ((1u << lane) - 1u));
-                const long long idx = (long long)g.tile_off[t] + base;
+                const long long idx = (long long)off + base;
                 if (idx < g.list_cap) g.lists[idx] = f;
             }
             if (++tx > tx1) {
