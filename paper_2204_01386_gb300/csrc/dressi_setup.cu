@@ -301,8 +301,17 @@ __device__ __forceinline__ void bin_walk(const Globals &g, const ViewK &V, int f
 // the table, which alone takes 106; a warp-wide list of all box pixels took 198, and on 21-pixel
 // faces 84 instead of 44 us (its batches look up face, record and pixel for each pair).
 // ---------------------------------------------------------------------------
-constexpr int FRONT_LANE = 512;   // pixels of a bounding box that its face's lane visits alone
-constexpr int FRONT_BIG = 4096;   // pixels of a bounding box left to k_front_big
+// Pixels of a bounding box that its face's lane visits alone, and past which it is left to k_front_big,
+// whose warps share such faces out over the GPU.  A few hundred mid-sized faces among many small ones
+// follow one another in the mesh: with up to 4,096 pixels in their own warps' lists, ten warps had
+// 300 of them (forward, us, with 512 and 4,096 / 64 and 512 / 64 and 256 / 64 and 128, and without front
+// words; 1280 x 720):
+//   81,920 small faces and 300 of some 1,500 px   438 / 157 / 134 / 126, 199
+//   ... and 3,000 of some 700 px                  288 / 192 / 161 / 149, 212
+//   ... and 2,000 of some 3,000 px                645 / 247 / 237 / 239, 320
+//   the small ones alone                          102 / 101 / 100 / 100, 176
+//   those from close by, 1024^2                   163 / 111 / 110 / 127, 198
+constexpr int FRONT_LANE = 64, FRONT_BIG = 256;
 
 // the pixel centres inside the face's bounding box (grown by a margin over the corners' low parts)
 __device__ __forceinline__ bool front_rect(const ViewK &V, const FaceGeo &R, int &x0, int &y0, int &w, int &h)
