@@ -338,18 +338,24 @@ __device__ __forceinline__ void front_pixel(const ViewK &V, const FaceGeo &R, in
 // a face's pixels by its own lane: each row of the box cut to where the three cross products, linear
 // along the row, are above -FRONT_SLACK px (a division-free half-plane per edge), and the pixels
 // left tested exactly.  Where the crosses' rounding could reach the slack (corners far outside
-// the box, or an edge far shorter than the face), the whole rows are tested.
-constexpr float FRONT_SLACK = 2e-3f;
+// the box, or an edge far shorter than the face), the whole rows are tested.  With u = 2^-24 and no corner
+// farther than e from a pixel of the box along either axis, eval_face's cross is within 11 u e^2 of the exact
+// one (differences good to 2 u, two products, a sum), the row start's within 12 u e^2, the slope times a
+// column within 6 u e^2, and the bound's division moves it by up to 14 u e^2: together 43 u e^2 or
+// 2.6e-6 e^2 / (the edge's length) px.  (10 million accepted pixels of needles, slivers and cut faces,
+// emulated in FP32 with the limit ten times as far: none came closer than 0.91 slacks to being cut.)
+constexpr float FRONT_SLACK = 2e-3f, FRONT_CUT_ERR = 3e-6f;
 
 __device__ __forceinline__ void front_lane(const ViewK &V, const FaceGeo &R, int f, int x0, int y0, int w, int h,
                                            unsigned long long *words)
 {
     float dx[3], slope[3], inv[3], eps[3], sgn[3];
-    float ext = (float)h, sharp = 0.f;
+    float ext = 0.f, sharp = 0.f;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         dx[i] = ((float)x0 + 0.5f - R.c[i].xh) - R.c[i].xl;
-        ext = fmaxf(ext, fmaxf(fabsf(dx[i]), fabsf((float)y0 + 0.5f - R.c[i].yh) + (float)h));
+        const float ddy = (float)y0 + 0.5f - R.c[i].yh;
+        ext = fmaxf(ext, fmaxf(fmaxf(fabsf(dx[i]), fabsf(dx[i] + (float)(w - 1))), fmaxf(fabsf(ddy), fabsf(ddy + (float)(h - 1)))));
         sharp = fmaxf(sharp, fabsf(R.invL[i]));
     }
 #pragma unroll
@@ -362,7 +368,7 @@ __device__ __forceinline__ void front_lane(const ViewK &V, const FaceGeo &R, int
         inv[i] = __fdividef(1.f, slope[i]);
         eps[i] = __fdividef(FRONT_SLACK, fabsf(R.invL[i]));
     }
-    const bool cut = 1.2e-7f * ext * ext * sharp <= 0.5f * FRONT_SLACK;
+    const bool cut = FRONT_CUT_ERR * ext * ext * sharp <= FRONT_SLACK;
     for (int y = y0; y < y0 + h; ++y) {
         float lo = 0.f, hi = (float)(w - 1);
         if (cut) {
