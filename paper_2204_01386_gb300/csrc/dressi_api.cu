@@ -345,15 +345,18 @@ static bool fronts_only(const dressi_params *p)
 
 // Where the front fragments come from: the face table kernel, where a face's lane visits its pixels
 // with the record at hand, if the faces are small and enough of them to fill the GPU; else the
-// tiles' own rasters.  Face table + forward tile kernel, us, from the tiles / from the face table:
-//   1,280 x 720, 81,920 faces (11 pixels per face)      6 + 108 / 14 + 63
-//   4 views of 768^2, 32,000 faces each (18)            8 + 238 / 44 + 128
-//   8 views of 512^2, 20,480 faces each (13)           11 + 296 / 38 + 164
-//   2 views of 2048^2, 1.31 M faces (3)               106 + 1094 / 165 + 554
-//   256^2, 20,480 faces (3)                             6 + 56 / 9 + 30
-//   256^2, 5,120 faces (13)                             6 + 53 / 24 + 37   (and a launch and a fill)
-//   8 views of 512^2, 5,120 faces each (51)             8 + 223 / 169 + 128
-//   8 views of 512^2, 1,280 faces each (205)           10 + 195 / 398 + 108
+// tiles' own rasters.  Face table (with the large faces' kernel) + forward tile kernel, us, from the
+// tiles / from the face table (displaced icospheres):
+//   1,280 x 720, 81,920 faces (11 pixels per face)     12 + 108 / 21 + 53
+//   4 views of 700^2, 20,480 faces each (24)           11 + 236 / 49 + 113
+//   8 views of 512^2, 20,480 faces each (13)           24 + 284 / 50 + 133
+//   2 views of 2048^2, 1.31 M faces (3)               171 + 1049 / 262 + 477
+//   256^2, 20,480 faces (3)                            15 + 59 / 25 + 42
+//   256^2, 5,120 faces (13)                             7 + 38 / 20 + 32   (and a fill: 60 / 67 us in all)
+//   8 views of 512^2, 5,120 faces each (51)             9 + 214 / 55 + 103
+//   8 views of 512^2, 1,280 faces each (205)            9 + 168 / 70 + 80
+// The line at 24 pixels is from when a face of up to 4,096 pixels was its own warp's (the last two rows
+// then 169 + 128 and 398 + 108); since they are shared out it is on the safe side.
 constexpr long long FRONT_MIN_FACES = 16384;
 constexpr long long FRONT_MAX_PX = 24;   // view pixels per face
 

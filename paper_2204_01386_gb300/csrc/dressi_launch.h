@@ -9,9 +9,10 @@ struct Globals;
 // Kernel launches of this library overlap: a kernel may be set up while the one before it in the
 // stream ends (programmatic dependent launch), and waits, before it touches memory, until that one
 // is complete and its writes are visible.  Every kernel waits, so that completion is transitive.
-// The ten short kernels of a textured 256^2 step idled some 2 us at each: 120 -> 106 us, inverse UV
-// on one 521 x 337 view 129 -> 112, a 1280 x 720 render 128 -> 102.  (Releasing the next kernel at
-// a kernel's start instead of its end: 101, 116 and 111 us.)
+// The ten short kernels of a textured 256^2 step idled some 2 us at each: without / with, 113 / 91 us;
+// inverse UV on one 521 x 337 view 119 / 101, a 1280 x 720 render 128 / 109, a 64^2 step of 320 faces
+// 59 / 43.  (Releasing the next kernel at a kernel's start instead of its end made the textured step 5 us
+// faster and the other two 4 and 9 us slower.)
 // With clusters of `ctas` blocks (1: none).
 template <typename... P, typename... A>
 inline void launch_clusters(int ctas, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,

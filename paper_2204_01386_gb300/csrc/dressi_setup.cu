@@ -299,19 +299,20 @@ __device__ __forceinline__ void bin_walk(const Globals &g, const ViewK &V, int f
 // (measured on both sides of the line that chooses it: FRONT_MIN_FACES, dressi_api.cu).  A lane
 // visits a face's rows, cut to the covered interval: two 2048^2 views of 1.31 M faces 165 us with
 // the table, which alone takes 106; a warp-wide list of all box pixels took 198, and on 21-pixel
-// faces 84 instead of 44 us (its batches look up face, record and pixel for each pair).
+// faces 84 instead of 44 us (its batches look up face, record and pixel for each pair).  Larger faces
+// are k_front_big's.
 // ---------------------------------------------------------------------------
-// Pixels of a bounding box that its face's lane visits alone, and past which it is left to k_front_big,
-// whose warps share such faces out over the GPU.  A few hundred mid-sized faces among many small ones
-// follow one another in the mesh: with up to 4,096 pixels in their own warps' lists, ten warps had
-// 300 of them (forward, us, with 512 and 4,096 / 64 and 512 / 64 and 256 / 64 and 128, and without front
-// words; 1280 x 720):
-//   81,920 small faces and 300 of some 1,500 px   438 / 157 / 134 / 126, 199
-//   ... and 3,000 of some 700 px                  288 / 192 / 161 / 149, 212
-//   ... and 2,000 of some 3,000 px                645 / 247 / 237 / 239, 320
-//   the small ones alone                          102 / 101 / 100 / 100, 176
-//   those from close by, 1024^2                   163 / 111 / 110 / 127, 198
-constexpr int FRONT_LANE = 64, FRONT_BIG = 256;
+// Pixels of a bounding box that its face's lane visits alone; past them it is left to k_front_big, whose
+// warps share such faces out over the GPU.  A few hundred mid-sized faces among many small ones follow
+// one another in the mesh: while up to 4,096 pixels went through a list of their own warp's pixels, ten
+// warps had 300 of them.  Forward, us, with such lists / 96 / 128 / 192 / 256, without front words:
+//   81,920 small faces, 1280 x 720                102 / 101 / 101 / 100 / 100, 175
+//   ... and 300 of some 1,500 px                  436 / 125 / 127 / 136 / 144, 200
+//   ... and 3,000 of some 700 px                  286 / 157 / 150 / 157 / 168, 212
+//   ... and 2,000 of some 3,000 px                644 / 252 / 250 / 250 / 252, 321
+//   the small ones from close by, 1024^2          159 / 152 / 129 / 116 / 116, 197
+//   step of four 768^2 views of 32,000 faces      512 / 520 / 513 / 511 / 510, 874
+constexpr int FRONT_LANE = 192;
 
 // the pixel centres inside the face's bounding box (grown by a margin over the corners' low parts)
 __device__ __forceinline__ bool front_rect(const ViewK &V, const FaceGeo &R, int &x0, int &y0, int &w, int &h)
@@ -390,46 +391,6 @@ __device__ __forceinline__ void front_lane(const ViewK &V, const FaceGeo &R, int
     }
 }
 
-// the larger of the warp's 32 staged faces (stride 7 float4; c: box pixels of this lane's face f, 0 for none): their
-// pixels as one list, 32 at a time with full lanes.  A list entry's face is found by the bits of
-// the faces that start in its batch.
-__device__ __forceinline__ void front_warp(const ViewK &V, const float4 *recs, int f0, int c, int x0, int y0, int w,
-                                           unsigned long long *words, int2 *slot)
-{
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    int incl = c;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(FULL, incl, o);
-        if (lane >= o) incl += v;
-    }
-    const int total = __shfl_sync(FULL, incl, 31), first = incl - c;
-    const unsigned some = __ballot_sync(FULL, c > 0);
-    // the faces with pixels packed to the front: first | lane, and the box
-    const int rank = __popc(some & ((1u << lane) - 1u));
-    if (c > 0) slot[rank] = make_int2(first, lane);
-    __syncwarp();
-    int nb = -1;
-    for (int b0 = 0; b0 < total; b0 += 32) {
-        const unsigned starts = __reduce_or_sync(FULL, (c > 0 && (unsigned)(first - b0) < 32u) ? 1u << (first - b0) : 0u);
-        const int idx = nb + __popc(starts & (0xffffffffu >> (31 - lane)));
-        nb += __popc(starts);
-        const int2 e = slot[max(idx, 0)];
-        const int fx = __shfl_sync(FULL, x0, e.y), fy = __shfl_sync(FULL, y0, e.y), fw = __shfl_sync(FULL, w, e.y);
-        if (b0 + lane < total) {
-            const int k = b0 + lane - e.x;
-            // k / w: both are small integers, the quotient of the floats is off by at most one
-            int q = (int)__fdividef((float)k + 0.5f, (float)fw);
-            int r = k - q * fw;
-            if (r < 0) { --q; r += fw; }
-            else if (r >= fw) { ++q; r -= fw; }
-            front_pixel(V, *reinterpret_cast<const FaceGeo *>(recs + e.y * 7), f0 + e.y, fx + r, fy + q, words);
-        }
-    }
-    __syncwarp();
-}
-
 // a band of the rows of a face's box, by a warp
 __device__ __forceinline__ void front_band(const Globals &g, const ViewK &V, const FaceGeo &R, int f, int band, int bands)
 {
@@ -473,7 +434,7 @@ __global__ void __launch_bounds__(256) k_front_big(Globals g)
             if (f0 + lane < nF) {
                 const FaceGeo &R = g.frec[V.frec_off + f0 + lane];
                 int x0, y0, w, h;
-                big = (R.flags & FLAG_LIVE) && front_rect(V, R, x0, y0, w, h) && (long long)w * h > FRONT_BIG;
+                big = (R.flags & FLAG_LIVE) && front_rect(V, R, x0, y0, w, h) && (long long)w * h > FRONT_LANE;
             }
             for (unsigned todo = __ballot_sync(0xffffffffu, big); todo; todo &= todo - 1u) {
                 const int f = f0 + __ffs(todo) - 1;
@@ -497,7 +458,6 @@ __global__ void __launch_bounds__(256, FRONT ? 3 : 4) k_face(Globals g)
     // each warp's 32 records (7 float4 each) go through shared memory so that the warp
     // writes its 3,584 contiguous bytes with full-line stores
     __shared__ float4 stage[256 / 32][32 * 7];
-    __shared__ int2 slots[FRONT ? 256 : 1];
     if (blockIdx.y >= g.n_views) {
         adjacency<0>(g, blockIdx.y - g.n_views);
         return;
@@ -538,21 +498,14 @@ __global__ void __launch_bounds__(256, FRONT ? 3 : 4) k_face(Globals g)
             float4 *dst = reinterpret_cast<float4 *>(g.frec + V.frec_off + wf0);
             for (int i = lane; i < nrec * 7; i += 32) dst[i] = ws[i];
         }
-        if (FRONT) {
-            int x0 = 0, y0 = 0, w = 0, h = 0, c = 0;
-            if (live && front_rect(V, R, x0, y0, w, h)) {
-                c = w * h;
-                if (c <= FRONT_LANE) {
-                    c = 0;
-                    front_lane(V, R, f, x0, y0, w, h, g.kth + V.slot_base);
-                } else if ((long long)w * h > FRONT_BIG) {
-                    c = 0;
-                    const int q = atomicAdd(g.big_n, 1);
-                    if (q < g.big_cap) g.big[q] = make_int2(blockIdx.y, f);   // else: see k_front_big
-                }
+        int x0, y0, w, h;
+        if (FRONT && live && front_rect(V, R, x0, y0, w, h)) {
+            if ((long long)w * h <= FRONT_LANE) {
+                front_lane(V, R, f, x0, y0, w, h, g.kth + V.slot_base);
+            } else {
+                const int q = atomicAdd(g.big_n, 1);
+                if (q < g.big_cap) g.big[q] = make_int2(blockIdx.y, f);   // else: see k_front_big
             }
-            if (__any_sync(0xffffffffu, c > 0))
-                front_warp(V, ws, f0 + (threadIdx.x & ~31), c, x0, y0, w, g.kth + V.slot_base, slots + (threadIdx.x & ~31));
         }
         __syncwarp();   // the staged records are read before the next iteration writes them
         if (COUNT) {
