@@ -1,7 +1,7 @@
 // dressi_core.cuh -- device-side data layout and the geometric core of HardSoftRas.
 //
 // Precision plan (GB300, FP32 pixel math):
-//   * the vertex transform runs in FP64 with explicitly rounded operations, and
+//   * the vertex transform runs in double-float FP32 (error-free sums and products), and
 //     each pixel-space corner is kept as an unevaluated float pair hi + lo, so
 //     that p - V is accurate to one float ulp of |p - V| (not of |V|): the
 //     sigmoid of Sec. 3.4.3 is steep (sigma is a fraction of a pixel), so the

@@ -1036,8 +1036,7 @@ __device__ __forceinline__ bool pixel_weights(const Globals &g, const ViewK &V, 
 }
 
 // The adjoint of one pixel whose K layer ids are known, by pixel: the adjoints with
-// the extras (light gradient, inverse UV, normal map); S.sh holds the tile's S^H with its
-// ring.
+// the extras (light gradient, inverse UV, normal map); S.hb and S.eb hold the tile's S^H and E.
 template <int K, int TT, bool EXTRA>
 __device__ __forceinline__ unsigned adjoint_pixel(const Globals &g, const Smem &S, const ViewK &V, const MeshK &M,
                                                   int X0, int Y0, int lx, int ly, const int (&ids)[K],
