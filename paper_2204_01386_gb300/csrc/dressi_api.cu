@@ -360,9 +360,28 @@ static bool fronts_only(const dressi_params *p)
 constexpr long long FRONT_MIN_FACES = 16384;
 constexpr long long FRONT_MAX_PX = 24;   // view pixels per face
 
+// Lists up to this long get their layers in one pass, without one for the front fragments first, where the
+// tiles find those themselves: a tile's time is then that of its barriers and loads, once or twice.  Forward, us, without a limit / 8
+// / 16 / 32 (and without fronts first): 5,000 small triangles on 1024^2 132 / 113 / 110 / 110 (117);
+// eight 512^2 views of a 1,280-face mesh 203 / 204 / 219 / 218 (228); a 5,120-face mesh at 1024^2
+// 130 / 130 / 140 / 139 (151); one of 81,920 faces at 2048^2 443 / 445 / 444 / 499 (527).
+constexpr int FRONT_SHORT = 8;
+
+// The longest such list.  A mesh with more vertices than faces is of separate pieces (triangles, needles,
+// cards; a surface has about half as many): the edge mask is then nearly everywhere, and a pass for
+// the front fragments is one more.  Forward, us, with it / without, without fronts first (1024^2):
+// 15,000 triangles of some 90 px 222 / 195, 193; 12,000 needles of 80 x 2 px 363 / 315, 324; 4,000 of
+// them 234 / 206, 206.  (12,000 of some 800 px over each other at 768^2, where the front ones hide
+// most: 179 / 203, 222.)
+static int front_short(const Plan &P)
+{
+    return P.lay.n_vrec > P.view_faces ? 0x7fffffff : FRONT_SHORT;
+}
+
 static void choose_fronts(Globals &g, const Plan &P, bool only, char *ws, cudaStream_t s)
 {
     g.fronts = only ? 1 : 0;
+    g.front_short = front_short(P);
     if (!only || P.view_faces < FRONT_MIN_FACES || P.view_pixels > FRONT_MAX_PX * P.view_faces) return;
     g.fronts = 2;
     g.big = reinterpret_cast<int2 *>(ws + P.lay.lists);   // before the lists are written
@@ -706,6 +725,7 @@ int dressi_backward_ex(const dressi_scene *scene, const dressi_view *views, int3
     if (params->reuse_setup) {
         // re-rasterizing after a forward on this workspace: its pixels' words, if it kept them
         g.fronts = only ? 1 : 0;
+        g.front_short = front_short(P);
         if (!layer_ids) g.kth = reinterpret_cast<unsigned long long *>(w + P.lay.kth);
     } else {
         choose_fronts(g, P, only, w, s);

@@ -168,6 +168,7 @@ struct Globals {
     int *kth_flag;
     int fronts;           // layers beyond the front one are only needed inside the edge mask: the front
                           // ones come 1 from the tiles' rasters, 2 from the face table kernel (in kth)
+    int front_short;      // fronts 1: lists up to this long get all their layers in one pass
     int *heavy;           // a forward's tiles with long face lists: their number, then the tiles (k_bin
                           // lists them where the host allows it), or nullptr
     int heavy_cap, heavy_min, heavy_ctas;   // the list's room, the shortest long list, CTAs per tile

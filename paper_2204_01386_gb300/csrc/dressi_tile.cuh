@@ -57,12 +57,6 @@ constexpr int WQ = 160;                // a warp's queue of pretested pairs (31 
 constexpr int NBLK = 1024;             // pair blocks of 32 with a table entry (32,768 items)
 // the raster's passes (tile_body)
 constexpr int ST_FRONT = 0, ST_LAYERS = 1, ST_DONE = 2;
-// Lists up to this long get their layers in one pass, without one for the front fragments first: a
-// tile's time is then that of its barriers and loads, once or twice.  Forward, us, without a limit / 8
-// / 16 / 32 (and without fronts first): 5,000 small triangles on 1024^2 132 / 113 / 110 / 110 (117);
-// eight 512^2 views of a 1,280-face mesh 203 / 204 / 219 / 218 (228); a 5,120-face mesh at 1024^2
-// 130 / 130 / 140 / 139 (151); one of 81,920 faces at 2048^2 443 / 445 / 444 / 499 (527).
-constexpr int FRONT_SHORT = 8;
 
 // conservative tile-local data of a staged face: edge equations in pixels relative to
 // the tile origin (FP32, a few 1e-6 px of error) and the smallest corner depth.  12 words:
@@ -1653,7 +1647,7 @@ __device__ __forceinline__ void tile_body(const Globals &g, Smem &S, unsigned lo
                 __syncthreads();
             }
         }
-        if (stage == ST_FRONT && !raw && n <= FRONT_SHORT) {
+        if (stage == ST_FRONT && !raw && n <= g.front_short) {
             layered = true;
             stage = ST_LAYERS;
         }
